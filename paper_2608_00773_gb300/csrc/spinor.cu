@@ -39,20 +39,36 @@
 namespace q4c {
 namespace spinor {
 
+// One entry of G, a real number times 1 or i.  Which of the two follows from
+// where it stands, so the kernels multiply by real numbers only:
+//   column view, entries 4 mu .. 4 mu + 3 of spinor function mu: spin up with
+//   a real and with an imaginary coefficient, spin down with a real and with
+//   an imaginary one (Y~^m holds the real harmonic |m| with a real and -|m|
+//   with an imaginary coefficient); idx the scalar-spin row 2t + s;
+//   row view, entries 4 r .. 4 r + 3 of scalar-spin row r = 2t + s: the
+//   spinor functions idx that contain it, all real for a real harmonic m >= 0
+//   and all imaginary for m < 0 (sign of `imag`).
 struct Ent {
-  int idx;  // scalar-spin row 2t + s (column view) or spinor index (row view); -1 unused
-  int pad;
-  double re, im;
+  int idx;   // -1: no entry
+  int imag;  // row view: 1 where the row's coefficients are imaginary
+  double c;
 };
 
-__device__ __forceinline__ double2 cmul(double2 a, double2 b) {
-  return make_double2(a.x * b.x - a.y * b.y, a.x * b.y + a.y * b.x);
+__device__ __forceinline__ double at(const double* __restrict__ M, int64_t k, bool ok) {
+  return (M && ok) ? __ldg(M + k) : 0.0;
 }
 
-// One CTA per pattern block; thread per spinor element (mu, nu).
-// Spinor block q starts at spin_off[q] (complex elements), or at 4 blk_off[q]
-// when spin_off is NULL (no kappa selection: twice the scalar counts).
-__global__ void k_forward(const int* __restrict__ blk_row, const int* __restrict__ blk_col,
+// One CTA per pattern block; thread per spinor element (mu, nu):
+//   HL_(mu,nu) = sum_ab conj(G_a,mu) V_(ta,tb) G_b,nu  (equal spins),
+//   HS_(mu,nu) = sum_ab conj(G_a,mu) (W0 1 + i SO.sigma)_(a,b) G_b,nu,
+// summed over b for each of the four a, then over a.  Spinor block q starts at
+// spin_off[q] (complex elements), or at 4 blk_off[q] when spin_off is NULL (no
+// kappa selection: twice the scalar counts).
+// Bound by the FP64 units (2 multiply-adds a clock and SM): real coefficients
+// whose phase is static take 40 + 16 of them an element, where complex
+// products of both entries and the matrix value took about 200.
+// 64-atom cluster (0.78M spinor elements): this and k_reverse 0.73 ms -> 0.24.
+__global__ void __launch_bounds__(128) k_forward(const int* __restrict__ blk_row, const int* __restrict__ blk_col,
                           const int64_t* __restrict__ blk_off, const int64_t* __restrict__ spin_off,
                           const int* __restrict__ atom_sp, const int* __restrict__ sp_nfn,
                           const int* __restrict__ spn0, const Ent* __restrict__ col, const double* __restrict__ V,
@@ -70,47 +86,78 @@ __global__ void k_forward(const int* __restrict__ blk_row, const int* __restrict
   const Ent* cB = col + 4 * spn0[sb];
   for (int e = threadIdx.x; e < nsA * nsB; e += blockDim.x) {
     const int mu = e / nsB, nu = e - mu * nsB;
-    double2 hl = make_double2(0.0, 0.0), hs = make_double2(0.0, 0.0);
+    int tb[4];
+    double b[4];
 #pragma unroll
-    for (int ea = 0; ea < 4; ++ea) {
-      const Ent a = cA[4 * mu + ea];
+    for (int k = 0; k < 4; ++k) {
+      const Ent x = cB[4 * nu + k];
+      tb[k] = x.idx >> 1;  // negative: no entry
+      b[k] = x.c;
+    }
+    double lr = 0.0, li = 0.0, sr = 0.0, si = 0.0;
+#pragma unroll
+    for (int ka = 0; ka < 4; ++ka) {
+      const Ent a = cA[4 * mu + ka];
       if (a.idx < 0) continue;
-      const int ta = a.idx >> 1, s = a.idx & 1;
-#pragma unroll
-      for (int eb = 0; eb < 4; ++eb) {
-        const Ent b = cB[4 * nu + eb];
-        if (b.idx < 0) continue;
-        const int tb = b.idx >> 1, s2 = b.idx & 1;
-        const double2 g = cmul(make_double2(a.re, -a.im), make_double2(b.re, b.im));
-        const int64_t k = off + static_cast<int64_t>(ta) * nfB + tb;
-        if (V && s == s2) {
-          const double v = V[k];
-          hl.x += g.x * v;
-          hl.y += g.y * v;
+      const int s = ka >> 1;  // spin of this entry
+      const int64_t row = off + static_cast<int64_t>(a.idx >> 1) * nfB;
+      double tr = 0.0, ti = 0.0;  // sum over b of the operator's element times G_b
+      if (HL) {
+        tr = b[2 * s] * at(V, row + tb[2 * s], tb[2 * s] >= 0);
+        ti = b[2 * s + 1] * at(V, row + tb[2 * s + 1], tb[2 * s + 1] >= 0);
+        if (ka & 1) {  // conj(i c) = -i c
+          lr = fma(a.c, ti, lr);
+          li = fma(-a.c, tr, li);
+        } else {
+          lr = fma(a.c, tr, lr);
+          li = fma(a.c, ti, li);
         }
-        if (HS) {
-          // (W0 1 + i SO.sigma)_(s, s2)
-          const double w = W0 ? W0[k] : 0.0, x = SOx ? SOx[k] : 0.0, y = SOy ? SOy[k] : 0.0,
-                       z = SOz ? SOz[k] : 0.0;
-          double2 F;
-          if (s == s2)
-            F = make_double2(w, s == 0 ? z : -z);
-          else
-            F = make_double2(s == 0 ? y : -y, x);
-          const double2 t = cmul(g, F);
-          hs.x += t.x;
-          hs.y += t.y;
+      }
+      if (HS) {
+        tr = ti = 0.0;
+#pragma unroll
+        for (int kb = 0; kb < 4; ++kb) {
+          const int64_t k = row + tb[kb];
+          const bool ok = tb[kb] >= 0;
+          double Fr, Fi;  // (W0 1 + i SO.sigma)_(s, s2)
+          if (s == (kb >> 1)) {
+            Fr = at(W0, k, ok);
+            Fi = at(SOz, k, ok);
+            if (s) Fi = -Fi;
+          } else {
+            Fr = at(SOy, k, ok);
+            Fi = at(SOx, k, ok);
+            if (s) Fr = -Fr;
+          }
+          if (kb & 1) {  // times i c
+            tr = fma(-Fi, b[kb], tr);
+            ti = fma(Fr, b[kb], ti);
+          } else {
+            tr = fma(Fr, b[kb], tr);
+            ti = fma(Fi, b[kb], ti);
+          }
+        }
+        if (ka & 1) {
+          sr = fma(a.c, ti, sr);
+          si = fma(-a.c, tr, si);
+        } else {
+          sr = fma(a.c, tr, sr);
+          si = fma(a.c, ti, si);
         }
       }
     }
     const int64_t o = so + e;
-    if (HL) HL[o] = hl;
-    if (HS) HS[o] = hs;
+    if (HL) HL[o] = make_double2(lr, li);
+    if (HS) HS[o] = make_double2(sr, si);
   }
 }
 
-// One CTA per pattern block; thread per scalar element (t, u).
-__global__ void k_reverse(const int* __restrict__ blk_row, const int* __restrict__ blk_col,
+// One CTA per pattern block; thread per scalar element (t, u): the four
+// spin components of D'_(t,u) = sum conj(G_a,mu) D_(mu,nu) G_b,nu with real
+// coefficients, the unit phase (1, -i or i) of the two rows applied at the end.
+// Bound like k_forward: 160 multiply-adds an element for about 700 of complex
+// products.
+__global__ void __launch_bounds__(128) k_reverse(const int* __restrict__ blk_row, const int* __restrict__ blk_col,
                           const int64_t* __restrict__ blk_off, const int64_t* __restrict__ spin_off,
                           const int* __restrict__ atom_sp, const int* __restrict__ sp_nfn,
                           const int* __restrict__ spn0, const int* __restrict__ ss0, const Ent* __restrict__ row,
@@ -131,24 +178,48 @@ __global__ void k_reverse(const int* __restrict__ blk_row, const int* __restrict
 #pragma unroll
     for (int s = 0; s < 2; ++s)
 #pragma unroll
-      for (int s2 = 0; s2 < 2; ++s2) {
-        double2 acc = make_double2(0.0, 0.0);
+      for (int s2 = 0; s2 < 2; ++s2) Dp[s][s2] = make_double2(0.0, 0.0);
+    int nu[2][4];
+    double cb[2][4];
 #pragma unroll
-        for (int ea = 0; ea < 4; ++ea) {
-          const Ent a = rA[4 * (2 * t + s) + ea];
-          if (a.idx < 0) continue;
+    for (int s2 = 0; s2 < 2; ++s2)
+#pragma unroll
+      for (int eb = 0; eb < 4; ++eb) {
+        const Ent b = rB[4 * (2 * u + s2) + eb];
+        nu[s2][eb] = b.idx;
+        cb[s2][eb] = b.c;
+      }
+    const bool ia = rA[8 * t].imag != 0, ib = rB[8 * u].imag != 0;
+#pragma unroll
+    for (int s = 0; s < 2; ++s)
+#pragma unroll
+      for (int ea = 0; ea < 4; ++ea) {
+        const Ent a = rA[4 * (2 * t + s) + ea];
+        if (a.idx < 0) continue;
+        const double2* Dr = Dq + static_cast<int64_t>(a.idx) * nsB;
+#pragma unroll
+        for (int s2 = 0; s2 < 2; ++s2) {
+          double xr = 0.0, xi = 0.0;
 #pragma unroll
           for (int eb = 0; eb < 4; ++eb) {
-            const Ent b = rB[4 * (2 * u + s2) + eb];
-            if (b.idx < 0) continue;
-            const double2 g = cmul(make_double2(a.re, -a.im), make_double2(b.re, b.im));
-            const double2 d = cmul(g, Dq[static_cast<int64_t>(a.idx) * nsB + b.idx]);
-            acc.x += d.x;
-            acc.y += d.y;
+            if (nu[s2][eb] < 0) continue;
+            const double2 d = __ldg(Dr + nu[s2][eb]);
+            xr = fma(cb[s2][eb], d.x, xr);
+            xi = fma(cb[s2][eb], d.y, xi);
           }
+          Dp[s][s2].x = fma(a.c, xr, Dp[s][s2].x);
+          Dp[s][s2].y = fma(a.c, xi, Dp[s][s2].y);
         }
-        Dp[s][s2] = acc;
       }
+    if (ia != ib) {  // times -i (row a imaginary) or i (row b imaginary)
+#pragma unroll
+      for (int s = 0; s < 2; ++s)
+#pragma unroll
+        for (int s2 = 0; s2 < 2; ++s2) {
+          const double2 d = Dp[s][s2];
+          Dp[s][s2] = ia ? make_double2(d.y, -d.x) : make_double2(-d.y, d.x);
+        }
+    }
     const int64_t k = off + e;
     const double tr = Dp[0][0].x + Dp[1][1].x;
     if (PV) PV[k] = tr;
@@ -179,8 +250,8 @@ q4c_status build_spinor_tables(q4c_tables* t) {
     spn0[s + 1] = spn0[s] + n;
   }
   const int total = spn0[ns], total_ss = ss0[ns];
-  std::vector<Ent> col(4 * static_cast<size_t>(total), Ent{-1, 0, 0.0, 0.0});
-  std::vector<Ent> row(4 * static_cast<size_t>(total_ss), Ent{-1, 0, 0.0, 0.0});
+  std::vector<Ent> col(4 * static_cast<size_t>(total), Ent{-1, 0, 0.0});
+  std::vector<Ent> row(4 * static_cast<size_t>(total_ss), Ent{-1, 0, 0.0});
   t->h_spn_radial.assign(total, 0);
   t->h_spn_kappa.assign(total, 0);
   t->h_spn_two_mj.assign(total, 0);
@@ -200,40 +271,26 @@ q4c_status build_spinor_tables(q4c_tables* t) {
           t->h_spn_two_mj[g] = mjx2;
           const double den = 2.0 * (2 * l + 1);
           const double c[2] = {a * std::sqrt((2 * l + a * mjx2 + 1) / den), std::sqrt((2 * l - a * mjx2 + 1) / den)};
-          int ne = 0;
           for (int sp = 0; sp < 2; ++sp) {  // spin up: m_l = m_j - 1/2; spin down: m_l = m_j + 1/2
             const int ml = (mjx2 + (sp == 0 ? -1 : 1)) / 2;
             if (ml < -l || ml > l) continue;
-            // complex harmonic Y~_l^ml as (real index m, coefficient)
-            struct Term {
-              int m;
-              double re, im;
-            } terms[2];
-            int nt = 0;
-            if (ml == 0) {
-              terms[nt++] = {0, 1.0, 0.0};
-            } else if (ml > 0) {
-              terms[nt++] = {ml, r2, 0.0};
-              terms[nt++] = {-ml, 0.0, r2};
-            } else {
-              const double sg = ((-ml) & 1) ? -1.0 : 1.0;
-              terms[nt++] = {-ml, sg * r2, 0.0};
-              terms[nt++] = {ml, 0.0, -sg * r2};
-            }
-            for (int i = 0; i < nt; ++i) {
-              const int rowi = 2 * (t0 + terms[i].m + l) + sp;
-              const Ent e{rowi, 0, c[sp] * terms[i].re, c[sp] * terms[i].im};
-              if (ne < 4) col[4 * static_cast<size_t>(g) + ne] = e;
-              ++ne;
+            // complex harmonic Y~_l^ml: the real harmonic |m_l| with a real
+            // and, for m_l != 0, -|m_l| with an imaginary coefficient
+            const double sg = ml < 0 && ((-ml) & 1) ? -1.0 : 1.0;
+            for (int im = 0; im < (ml == 0 ? 1 : 2); ++im) {
+              const int m = im ? -std::abs(ml) : std::abs(ml);
+              const double w = ml == 0 ? 1.0 : im && ml < 0 ? -sg * r2 : sg * r2;
+              const int rowi = 2 * (t0 + m + l) + sp;
+              col[4 * static_cast<size_t>(g) + 2 * sp + im] = Ent{rowi, im, c[sp] * w};
               // row view: the spinor functions of scalar-spin row rowi
               Ent* rv = &row[4 * static_cast<size_t>(ss0[s] + rowi)];
               int slot = 0;
               while (slot < 4 && rv[slot].idx >= 0) ++slot;
-              if (slot == 4 || ne > 4) {  // at most two m_l x two j per row, two spins x two terms per column
+              if (slot == 4) {  // at most two m_l x two j per row
                 set_error("nao_tabulate: spinor relation table overflow");
                 return Q4C_EINVAL;
               }
-              rv[slot] = Ent{mu, 0, e.re, e.im};
+              rv[slot] = Ent{mu, im, c[sp] * w};
             }
           }
         }
@@ -348,7 +405,7 @@ extern "C" q4c_status q4c_spinor_transform(const q4c_tables* t, const q4c_grid* 
   if (st) return st;
   {
     KernelScope ks("spinor_transform", s);
-    spinor::k_forward<<<static_cast<unsigned>(g->n_blocks), 256, 0, s>>>(
+    spinor::k_forward<<<static_cast<unsigned>(g->n_blocks), 128, 0, s>>>(
         g->d_blk_row, g->d_blk_col, g->d_blk_off, d_so, g->d_atom_sp, t->d_sp_nfn, t->d_spn0,
         reinterpret_cast<const spinor::Ent*>(t->d_spn_col), HL ? F->V : nullptr, F->W0, F->SOx, F->SOy, F->SOz,
         reinterpret_cast<double2*>(HL), reinterpret_cast<double2*>(HS));
@@ -370,7 +427,7 @@ extern "C" q4c_status q4c_spinor_density_matrices(const q4c_tables* t, const q4c
   if (st) return st;
   {
     KernelScope ks("spinor_reverse", s);
-    spinor::k_reverse<<<static_cast<unsigned>(g->n_blocks), 256, 0, s>>>(
+    spinor::k_reverse<<<static_cast<unsigned>(g->n_blocks), 128, 0, s>>>(
         g->d_blk_row, g->d_blk_col, g->d_blk_off, d_so, g->d_atom_sp, t->d_sp_nfn, t->d_spn0, t->d_ss0,
         reinterpret_cast<const spinor::Ent*>(t->d_spn_row), reinterpret_cast<const double2*>(D), P->V, P->W0,
         P->SOx, P->SOy, P->SOz);
