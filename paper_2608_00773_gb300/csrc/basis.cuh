@@ -12,19 +12,35 @@
 
 namespace q4c {
 
+// place of a radius on the logarithmic knot grid, r < r_c: shared by every
+// radial function of a centre (its FP64 logarithm is the dearest step of the
+// evaluation and is taken once per centre and point)
+struct RadialPlace {
+  bool below;  // r < r_min
+  int k;       // knot interval
+  double s;    // coordinate in it
+};
+
+__device__ __forceinline__ RadialPlace radial_place(const DevBasis& B, double r) {
+  RadialPlace P{r < B.r_min, 0, 0.0};
+  if (P.below) return P;
+  const double t = log(r * B.inv_rmin) * B.inv_h;
+  P.k = static_cast<int>(t);
+  if (P.k > B.n_log - 2) P.k = B.n_log - 2;
+  P.s = t - P.k;
+  return P;
+}
+
 // cubic spline on the logarithmic grid: g = u/r^(l+1) and dg/dr, r < r_c
-__device__ __forceinline__ void radial_g(const DevBasis& B, int rad, int l, double r, double inv_r, double& g,
-                                         double& gp) {
-  if (r < B.r_min) {  // u = u(r_min) (r/r_min)^(l+1): g constant
+__device__ __forceinline__ void radial_g(const DevBasis& B, int rad, int l, const RadialPlace& P, double inv_r,
+                                         double& g, double& gp) {
+  if (P.below) {  // u = u(r_min) (r/r_min)^(l+1): g constant
     g = __ldg(B.g0 + rad);
     gp = 0.0;
     return;
   }
-  const double t = log(r * B.inv_rmin) * B.inv_h;
-  int k = static_cast<int>(t);
-  if (k > B.n_log - 2) k = B.n_log - 2;
-  const double s = t - k;
-  const double2* c2 = reinterpret_cast<const double2*>(B.coef + (static_cast<size_t>(rad) * (B.n_log - 1) + k) * 4);
+  const double s = P.s;
+  const double2* c2 = reinterpret_cast<const double2*>(B.coef + (static_cast<size_t>(rad) * (B.n_log - 1) + P.k) * 4);
   const double2 c01 = __ldg(c2), c23 = __ldg(c2 + 1);
   const double u = c01.x + s * (c01.y + s * (c23.x + s * c23.y));
   const double du_ds = c01.y + s * (2.0 * c23.x + 3.0 * s * c23.y);
@@ -131,11 +147,12 @@ __device__ __forceinline__ void atom_functions(const DevBasis& B, int species, d
   solid_harmonics(dx, dy, dz, lmax, S, dS);
   const double inv_r = r > 0.0 ? 1.0 / r : 0.0;
   const double ux = dx * inv_r, uy = dy * inv_r, uz = dz * inv_r;
+  const RadialPlace place = radial_place(B, r);
   int k = 0;
   for (int q = 0; q < nr; ++q) {
     const int l = __ldg(B.rad_l + r0 + q);
     double g, gp;
-    radial_g(B, r0 + q, l, r, inv_r, g, gp);
+    radial_g(B, r0 + q, l, place, inv_r, g, gp);
     for (int m = 0; m < 2 * l + 1; ++m) {
       const int idx = l * l + m;
       const double s = S[idx];

@@ -91,28 +91,69 @@ __device__ __forceinline__ int local_nf(const DevBasis& B, const DevGrid& G, int
 }
 
 // ------------------------------------------------------------ products
-// One CTA per 32x32 tile (ti <= tj) of one batch, 16x16 threads, 2x2
-// elements each; accumulates V, W0 and SO directly on the upper triangle
-// (i <= j) and scatters with FP64 atomics into the upper blocks.
+// One CTA per 32x32 tile (ti <= tj) of one batch: V, W0 and SO of its pairs
+// i <= j, scattered with FP64 atomics into the upper blocks.
+// The FP64 units (2 multiply-adds a clock and SM) bound it: 10 multiply-adds
+// per pair and point.  So only pairs that count are formed, in blocks of 4 x 4
+// (eight lanes each, two pairs a lane; a warp takes four blocks of the tile's
+// list): blocks wholly below the diagonal or past the batch's functions are left
+// out, and the points run to n_p, not to a multiple of the staged 16.  The
+// groups of four blocks are dealt to the warps starting at a warp that rotates
+// with the CTA, so that the four schedulers' FP64 units get equal shares over
+// the CTAs of an SM.  gridDim.y splits a batch's points where a wave has too
+// few tiles to fill the GPU (the partial sums meet in the scatter's atomics).
+// 64-atom cluster (5.5e9 n_p n_b^2): 91.6 ms with whole 32x32 tiles, 56.2 with
+// blocks of 8 x 8 -> 51.9; water (24 functions): 223 us -> 81.
 constexpr int kT = 32, kK = 16;
-__global__ void __launch_bounds__(256) k_products_fp64(DevBasis B, DevGrid G, const int4* __restrict__ tiles,
+constexpr int kPitch = kK + 1;  // doubles per staged function: rows fall into distinct banks
+constexpr int kSub = 4;         // side of a block of pairs
+__global__ void __launch_bounds__(256, 3) k_products_fp64(DevBasis B, DevGrid G, const int4* __restrict__ tiles,
                                                        int64_t t0, const int64_t* __restrict__ scr_off,
                                                        int64_t scr_base, const double* __restrict__ scratch,
                                                        const double* __restrict__ v, double* V, double* W0,
                                                        double* SOx, double* SOy, double* SOz) {
-  __shared__ double sa[4][kK][kT];  // D-scaled i side
-  __shared__ double sb[4][kK][kT];  // j side
-  __shared__ double sd[kK];
+  __shared__ double sa[4][kT][kPitch];  // D-scaled i side
+  __shared__ double sb[4][kT][kPitch];  // j side
   const int4 tile = tiles[t0 + blockIdx.x];
   const int64_t b = tile.x;
   const int ti = tile.y, tj = tile.z;
   const int64_t p0 = G.pt_ptr[b];
-  const int np = static_cast<int>(G.pt_ptr[b + 1] - p0);
-  const int ldp = (np + 7) & ~7;
+  const int n_pt = static_cast<int>(G.pt_ptr[b + 1] - p0);
+  const int ldp = (n_pt + 7) & ~7;
+  const int share = ((n_pt + gridDim.y - 1) / gridDim.y + kK - 1) & ~(kK - 1);  // points of this CTA: [kb, np)
+  const int kb = blockIdx.y * share, np = min(n_pt, kb + share);
+  if (kb >= np) return;
   const int nb = static_cast<int>(G.bat_fn_ptr[b + 1] - G.bat_fn_ptr[b]);
   const int64_t plane = static_cast<int64_t>(nb) * ldp;
   const double* base = scratch + (scr_off[b] - scr_base);
-  const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  // this warp's two groups of four blocks, one block for each eight lanes:
+  // first row and column of the lane's block, -1 for none
+  int ri[2], cj[2];
+  bool any[2];
+  {
+    const int nr = (min(kT, nb - ti * kT) + kSub - 1) / kSub, nc = (min(kT, nb - tj * kT) + kSub - 1) / kSub;
+    const int n_blk = ti == tj ? nr * (nr + 1) / 2 : nr * nc;
+#pragma unroll
+    for (int u = 0; u < 2; ++u) {
+      const int first = 4 * (((warp + blockIdx.x) & 7) + 8 * u);
+      int k = first + (lane >> 3);
+      any[u] = first < n_blk;
+      ri[u] = cj[u] = -1;
+      if (k < n_blk) {
+        int r = 0;
+        if (ti == tj) {
+          while (k >= nc - r) k -= nc - r++;
+          k += r;
+        } else {
+          r = k / nc;
+          k -= r * nc;
+        }
+        ri[u] = r * kSub + ((lane >> 1) & 3);
+        cj[u] = k * kSub + 2 * (lane & 1);
+      }
+    }
+  }
   double acc[2][2][5];
 #pragma unroll
   for (int u = 0; u < 2; ++u)
@@ -121,54 +162,59 @@ __global__ void __launch_bounds__(256) k_products_fp64(DevBasis B, DevGrid G, co
 #pragma unroll
       for (int q = 0; q < 5; ++q) acc[u][w][q] = 0.0;
 
-  for (int k0 = 0; k0 < np; k0 += kK) {
-    if (threadIdx.x < kK) {
-      const int p = k0 + threadIdx.x;
-      sd[threadIdx.x] = p < np ? G.w[p0 + p] * v[p0 + p] : 0.0;
-    }
+  for (int k0 = kb; k0 < np; k0 += kK) {
     __syncthreads();
-    for (int e = threadIdx.x; e < 4 * kK * kT; e += blockDim.x) {
-      const int q = e / (kK * kT), rem = e - q * kK * kT, f = rem / kK, kk = rem - f * kK;
-      const int p = k0 + kk;
-      const int fi = ti * kT + f, fj = tj * kT + f;
-      const double ai = (p < np && fi < nb) ? base[q * plane + static_cast<int64_t>(fi) * ldp + p] : 0.0;
-      const double bj = (p < np && fj < nb) ? base[q * plane + static_cast<int64_t>(fj) * ldp + p] : 0.0;
-      sa[q][kk][f] = ai * sd[kk];
-      sb[q][kk][f] = bj;
-    }
-    __syncthreads();
-#pragma unroll 4
-    for (int kk = 0; kk < kK; ++kk) {
-      double a[2][4], c[2][4];
+    {  // thread: point kk of the functions f, f + 16 of both sides
+      const int kk = threadIdx.x & (kK - 1), p = k0 + kk;
+      const double d = p < np ? G.w[p0 + p] * v[p0 + p] : 0.0;
 #pragma unroll
-      for (int u = 0; u < 2; ++u)
+      for (int q = 0; q < 4; ++q)
 #pragma unroll
-        for (int q = 0; q < 4; ++q) {
-          a[u][q] = sa[q][kk][2 * ty + u];
-          c[u][q] = sb[q][kk][2 * tx + u];
+        for (int h = 0; h < 2; ++h) {
+          const int f = (threadIdx.x >> 4) + 16 * h;
+          const int fi = ti * kT + f, fj = tj * kT + f;
+          const double bj = (p < np && fj < nb) ? base[q * plane + static_cast<int64_t>(fj) * ldp + p] : 0.0;
+          double ai = bj;
+          if (ti != tj) ai = (p < np && fi < nb) ? base[q * plane + static_cast<int64_t>(fi) * ldp + p] : 0.0;
+          sa[q][f][kk] = ai * d;
+          sb[q][f][kk] = bj;
         }
+    }
+    __syncthreads();
+    const int n_kk = min(kK, np - k0);
 #pragma unroll
-      for (int u = 0; u < 2; ++u)
+    for (int u = 0; u < 2; ++u) {
+      if (!any[u]) continue;
+      const int i = max(ri[u], 0), j = max(cj[u], 0);
+#pragma unroll 4
+      for (int kk = 0; kk < n_kk; ++kk) {
+        double a[4];
+#pragma unroll
+        for (int q = 0; q < 4; ++q) a[q] = sa[q][i][kk];
 #pragma unroll
         for (int w = 0; w < 2; ++w) {
-          acc[u][w][0] = fma(a[u][0], c[w][0], acc[u][w][0]);
-          acc[u][w][1] = fma(a[u][1], c[w][1], fma(a[u][2], c[w][2], fma(a[u][3], c[w][3], acc[u][w][1])));
-          acc[u][w][2] = fma(a[u][2], c[w][3], fma(-a[u][3], c[w][2], acc[u][w][2]));
-          acc[u][w][3] = fma(a[u][3], c[w][1], fma(-a[u][1], c[w][3], acc[u][w][3]));
-          acc[u][w][4] = fma(a[u][1], c[w][2], fma(-a[u][2], c[w][1], acc[u][w][4]));
+          double c[4];
+#pragma unroll
+          for (int q = 0; q < 4; ++q) c[q] = sb[q][j + w][kk];
+          acc[u][w][0] = fma(a[0], c[0], acc[u][w][0]);
+          acc[u][w][1] = fma(a[1], c[1], fma(a[2], c[2], fma(a[3], c[3], acc[u][w][1])));
+          acc[u][w][2] = fma(a[2], c[3], fma(-a[3], c[2], acc[u][w][2]));
+          acc[u][w][3] = fma(a[3], c[1], fma(-a[1], c[3], acc[u][w][3]));
+          acc[u][w][4] = fma(a[1], c[2], fma(-a[2], c[1], acc[u][w][4]));
         }
+      }
     }
-    __syncthreads();
   }
   // scatter the upper triangle
   const int64_t f0 = G.bat_fn_ptr[b];
   const int a0 = G.bat_atom_ptr[b], na = G.bat_atom_ptr[b + 1] - a0;
   const int64_t pp = G.bat_pair_ptr[b];
 #pragma unroll
-  for (int u = 0; u < 2; ++u)
+  for (int u = 0; u < 2; ++u) {
+    if (ri[u] < 0) continue;
 #pragma unroll
     for (int w = 0; w < 2; ++w) {
-      const int i = ti * kT + 2 * ty + u, j = tj * kT + 2 * tx + w;
+      const int i = ti * kT + ri[u], j = tj * kT + cj[u] + w;
       if (i >= nb || j >= nb || i > j) continue;
       const int ii = G.fn_info[f0 + i], jj = G.fn_info[f0 + j];
       const int ai = ii >> 16, ki = ii & 0xffff, aj = jj >> 16, kj = jj & 0xffff;
@@ -183,6 +229,7 @@ __global__ void __launch_bounds__(256) k_products_fp64(DevBasis B, DevGrid G, co
         atomicAdd(SOz + e, acc[u][w][4]);
       }
     }
+  }
 }
 
 // ------------------------------------------------- mirror + spinor blocks
@@ -264,8 +311,15 @@ q4c_status products_fp64_wave(const q4c_grid* g, int wv, const double* v, const 
                               cudaStream_t s) {
   const int64_t t0 = g->wave_t0[wv], t1 = g->wave_t0[wv + 1];
   if (t1 <= t0) return Q4C_OK;
+  // fewer than eight CTAs a SM: split each batch's points, into no less than
+  // 32 (a CTA's scatter then still costs less than its sums)
+  int dev = 0, n_sm = 0;
+  cudaGetDevice(&dev);
+  cudaDeviceGetAttribute(&n_sm, cudaDevAttrMultiProcessorCount, dev);
+  const int64_t want = (8ll * n_sm + t1 - t0 - 1) / (t1 - t0);
+  const unsigned split = static_cast<unsigned>(std::max<int64_t>(1, std::min<int64_t>(want, g->max_np / 32)));
   KernelScope ks("products_fp64", s);
-  k_products_fp64<<<static_cast<unsigned>(t1 - t0), 256, 0, s>>>(g->tables->view(), g->view(), g->d_tiles, t0,
+  k_products_fp64<<<dim3(static_cast<unsigned>(t1 - t0), split), 256, 0, s>>>(g->tables->view(), g->view(), g->d_tiles, t0,
                                                                    g->d_scr_off, 0, g->d_scratch, v, out->V,
                                                                    out->W0, out->SOx, out->SOy, out->SOz);
   Q4C_CUDA(cudaGetLastError());
@@ -411,76 +465,158 @@ q4c_status integrate_columns_fp64(const q4c_tables* t, const q4c_grid* g, const 
   return Q4C_OK;
 }
 
-// ------------------------------------------------------------- density
-// One CTA per batch, one thread per point; P rows gathered into shared
-// memory kRows at a time: n_p = sum_i Phi_pi sum_j P_ij Phi_pj.  kRows is 16,
-// or fewer where 16 rows of a large batch would not fit in shared memory.
-template <int kRows>
-__global__ void k_density_fp64(DevBasis B, DevGrid G, int64_t b0, const int64_t* __restrict__ scr_off,
-                               const double* __restrict__ scratch, const double* __restrict__ P,
-                               double* __restrict__ n_out) {
-  extern __shared__ double sP[];  // [kRows][nb]
+// ---------------------------------------------------- density and adjoint
+// n_p = sum_ij P_ij phi_i phi_j (NQ = 1), and with all four quantities (NQ = 4)
+//   y_p = sum_ij [G^V phi_i phi_j + G^W grad_i.grad_j + G^x (Y_i Z_j - Z_i Y_j)
+//                 + G^y (Z_i X_j - X_i Z_j) + G^z (X_i Y_j - Y_i X_j)],
+// dL/dv = w y.  Only the symmetric parts of P, G^V, G^W and the antisymmetric
+// parts of G^x, G^y, G^z contribute, so the sum runs over j >= i with
+// coefficients S_ij = G_ij + G_ji (G_ii on the diagonal) and A_ij = G_ij - G_ji:
+//   y = sum_i phi_i t0 + X_i tx + Y_i ty + Z_i tz,
+//   t0 = sum_j S^V phi_j,  tx = sum_j S^W X_j + A^z Y_j - A^y Z_j  (cyclic),
+// 10 (NQ = 1: one) FP64 multiply-adds per pair i <= j and point.  The FP64
+// units (2 a clock and SM) bound it; the sum over all i, j of the products
+// as written took 17 per ordered pair, 3.4 times as many.
+//
+// One CTA per batch and up to 32 of its points: a warp takes eight points
+// times four rows i (lane = point + 8 row), the eight warps two row groups of
+// up to four point octets; the row groups run over chunks of eight rows, the
+// coefficients of 8 rows x 64 columns staged in shared memory.  A group of four
+// rows starts at its own first column, so that almost nothing is spent below
+// the diagonal.  Water (128 batches of 70 points, 24
+// functions): 317 us -> 78 for the adjoint, 43 -> 16 for the density; 8-atom
+// cluster: 7.18 ms -> 0.58.
+constexpr int kRdRows = 8, kRdCols = 64, kRdPitch = kRdCols + 1;
+
+// octets of points per CTA of a batch: at most 4, evenly spread
+__device__ __forceinline__ int rd_octets(int np) {
+  const int oct = (np + 7) >> 3, tiles = (oct + 3) >> 2;
+  return (oct + tiles - 1) / tiles;
+}
+
+template <int NQ>
+__global__ void __launch_bounds__(256) k_rowdot_fp64(DevBasis B, DevGrid G, int64_t b0,
+                                                     const int64_t* __restrict__ scr_off,
+                                                     const double* __restrict__ scratch, const double* GV,
+                                                     const double* GW, const double* Gx, const double* Gy,
+                                                     const double* Gz, double* __restrict__ out, int weighted) {
+  constexpr int NM = NQ == 1 ? 1 : 5;  // matrices
+  __shared__ double sG[NM][kRdRows][kRdPitch];
+  __shared__ double s_acc[2][32];
   const int64_t b = b0 + blockIdx.x;
   const int64_t p0 = G.pt_ptr[b];
   const int np = static_cast<int>(G.pt_ptr[b + 1] - p0);
+  const int n_oct = rd_octets(max(np, 1));
+  const int pt0 = blockIdx.y * n_oct * 8;  // first point of this CTA
+  if (pt0 >= np) return;
   const int ldp = (np + 7) & ~7;
   const int nb = static_cast<int>(G.bat_fn_ptr[b + 1] - G.bat_fn_ptr[b]);
+  const int64_t plane = static_cast<int64_t>(nb) * ldp;
   const int64_t f0 = G.bat_fn_ptr[b];
   const int a0 = G.bat_atom_ptr[b], na = G.bat_atom_ptr[b + 1] - a0;
   const int64_t pp = G.bat_pair_ptr[b];
-  const double* Phi = scratch + scr_off[b];
-  for (int pbase = 0; pbase < np; pbase += blockDim.x) {
-    const int p = pbase + threadIdx.x;
-    double acc = 0.0;
-    for (int i0 = 0; i0 < nb; i0 += kRows) {
-      const int rows = min(kRows, nb - i0);
-      __syncthreads();
-      for (int e = threadIdx.x; e < rows * nb; e += blockDim.x) {
-        const int r = e / nb, j = e - r * nb;
-        const int ii = G.fn_info[f0 + i0 + r], jj = G.fn_info[f0 + j];
-        const int64_t off = G.pair_off[pp + static_cast<int64_t>(ii >> 16) * na + (jj >> 16)];
-        sP[e] = off < 0 ? 0.0 : P[off + static_cast<int64_t>(ii & 0xffff) * local_nf(B, G, a0, jj >> 16) +
-                                  (jj & 0xffff)];
-      }
-      __syncthreads();
-      if (p < np) {
-        double t[kRows];
+  const double* Gm[5] = {GV, GW, Gx, Gy, Gz};
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int oct = warp & 3, half = warp >> 2;
+  const int row = 4 * half + (lane >> 3);               // row within a chunk
+  const int pl = 8 * oct + (lane & 7), p = pt0 + pl;     // point within the CTA, within the batch
+  const bool work = oct < n_oct && pt0 + 8 * oct < np;   // whole warps; p < ldp then
+  const double* F = scratch + scr_off[b] + p;
+  double acc = 0.0;
+  for (int i0 = 0; i0 < nb; i0 += kRdRows) {
+    double t[NQ];
 #pragma unroll
-        for (int r = 0; r < kRows; ++r) t[r] = 0.0;
-        for (int j = 0; j < nb; ++j) {
-          const double pj = Phi[static_cast<int64_t>(j) * ldp + p];
+    for (int q = 0; q < NQ; ++q) t[q] = 0.0;
+    const bool live = work && i0 + 4 * half < nb;  // uniform in the warp
+    for (int j0 = i0; j0 < nb; j0 += kRdCols) {
+      __syncthreads();
+      for (int e = threadIdx.x; e < kRdRows * kRdCols; e += blockDim.x) {
+        const int r = e / kRdCols, c = e - r * kRdCols, i = i0 + r, j = j0 + c;
+        double x[NM];
 #pragma unroll
-          for (int r = 0; r < kRows; ++r)
-            if (r < rows) t[r] = fma(sP[r * nb + j], pj, t[r]);
+        for (int m = 0; m < NM; ++m) x[m] = 0.0;
+        if (i < nb && j < nb && j >= i) {
+          const int ii = G.fn_info[f0 + i], jj = G.fn_info[f0 + j];
+          const int ai = ii >> 16, ki = ii & 0xffff, aj = jj >> 16, kj = jj & 0xffff;
+          const int64_t o1 = G.pair_off[pp + static_cast<int64_t>(ai) * na + aj];
+          const int64_t o2 = G.pair_off[pp + static_cast<int64_t>(aj) * na + ai];
+          const int64_t e1 = o1 + static_cast<int64_t>(ki) * local_nf(B, G, a0, aj) + kj;
+          const int64_t e2 = o2 + static_cast<int64_t>(kj) * local_nf(B, G, a0, ai) + ki;
+#pragma unroll
+          for (int m = 0; m < NM; ++m) {
+            if (Gm[m] == nullptr) continue;
+            const double g1 = o1 < 0 ? 0.0 : Gm[m][e1];
+            if (i == j) {
+              x[m] = m < 2 ? g1 : 0.0;
+            } else {
+              const double g2 = o2 < 0 ? 0.0 : Gm[m][e2];
+              x[m] = m < 2 ? g1 + g2 : g1 - g2;
+            }
+          }
         }
 #pragma unroll
-        for (int r = 0; r < kRows; ++r)
-          if (r < rows) acc = fma(Phi[static_cast<int64_t>(i0 + r) * ldp + p], t[r], acc);
+        for (int m = 0; m < NM; ++m) sG[m][r][c] = x[m];
+      }
+      __syncthreads();
+      if (live) {
+        const int jb = max(j0, i0 + 4 * half), je = min(nb, j0 + kRdCols);
+        const double* Fj = F + static_cast<int64_t>(jb) * ldp;
+#pragma unroll 4
+        for (int j = jb; j < je; ++j, Fj += ldp) {
+          const double* g = &sG[0][row][j - j0];
+          if constexpr (NQ == 1) {
+            t[0] = fma(g[0], __ldg(Fj), t[0]);
+          } else {
+            constexpr int M = kRdRows * kRdPitch;
+            const double f = __ldg(Fj), x = __ldg(Fj + plane), y = __ldg(Fj + 2 * plane), z = __ldg(Fj + 3 * plane);
+            const double gw = g[M], gx = g[2 * M], gy = g[3 * M], gz = g[4 * M];
+            t[0] = fma(g[0], f, t[0]);
+            t[1] = fma(gw, x, fma(gz, y, fma(-gy, z, t[1])));
+            t[2] = fma(gw, y, fma(gx, z, fma(-gz, x, t[2])));
+            t[3] = fma(gw, z, fma(gy, x, fma(-gx, y, t[3])));
+          }
+        }
       }
     }
-    if (p < np) n_out[p0 + p] = acc;
+    if (live && i0 + row < nb) {
+      const double* Fi = F + static_cast<int64_t>(i0 + row) * ldp;
+#pragma unroll
+      for (int q = 0; q < NQ; ++q) acc = fma(__ldg(Fi + q * plane), t[q], acc);
+    }
   }
+  // the four rows of a warp, then the two row groups of a point
+  acc += __shfl_xor_sync(0xffffffffu, acc, 8);
+  acc += __shfl_xor_sync(0xffffffffu, acc, 16);
+  if (lane < 8) s_acc[half][pl] = acc;
+  __syncthreads();
+  if (work && half == 0 && lane < 8 && p < np) {
+    const double y = s_acc[0][pl] + s_acc[1][pl];
+    out[p0 + p] = weighted ? G.w[p0 + p] * y : y;
+  }
+}
+
+template <int NQ>
+static q4c_status rowdot_fp64_wave(const q4c_grid* g, int wv, const double* const M[5], double* out, bool weighted,
+                                   const char* name, cudaStream_t s) {
+  const int64_t b0 = g->wave_b0[wv], b1 = g->wave_b0[wv + 1];
+  if (b1 <= b0) return Q4C_OK;
+  const unsigned tiles = static_cast<unsigned>((std::max(g->max_np, 1) + 31) / 32);
+  KernelScope ks(name, s);
+  k_rowdot_fp64<NQ><<<dim3(static_cast<unsigned>(b1 - b0), tiles), 256, 0, s>>>(
+      g->tables->view(), g->view(), b0, g->d_scr_off, g->d_scratch, M[0], M[1], M[2], M[3], M[4], out,
+      weighted ? 1 : 0);
+  Q4C_CUDA(cudaGetLastError());
+  return Q4C_OK;
 }
 
 // the density of one wave (its basis tiles in place)
 q4c_status density_fp64_wave(const q4c_grid* g, int wv, const double* P, double* n, cudaStream_t s) {
-  const int64_t b0 = g->wave_b0[wv], b1 = g->wave_b0[wv + 1];
-  if (b1 <= b0) return Q4C_OK;
-  constexpr size_t kSmemMax = 232448;
-  const size_t row = sizeof(double) * std::max(g->max_nb, 1);  // one P row of a batch
-  const int rows = 16 * row <= kSmemMax ? 16 : 8 * row <= kSmemMax ? 8 : 4;
-  if (rows * row > kSmemMax) {
+  if (g->max_nb > 7264) {
     set_error("the FP64 density needs at most 7264 active functions per batch");
     return Q4C_EUNSUPPORTED;
   }
-  const size_t smem = rows * row;
-  auto k_density = rows == 16 ? k_density_fp64<16> : rows == 8 ? k_density_fp64<8> : k_density_fp64<4>;
-  Q4C_CUDA(cudaFuncSetAttribute(k_density, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem)));
-  KernelScope ks("density_fp64", s);
-  k_density<<<static_cast<unsigned>(b1 - b0), 128, smem, s>>>(g->tables->view(), g->view(), b0, g->d_scr_off,
-                                                                   g->d_scratch, P, n);
-  Q4C_CUDA(cudaGetLastError());
-  return Q4C_OK;
+  const double* M[5] = {P, nullptr, nullptr, nullptr, nullptr};
+  return rowdot_fp64_wave<1>(g, wv, M, n, false, "density_fp64", s);
 }
 
 q4c_status density_fp64(const q4c_tables* t, const q4c_grid* g, const double* P, double* n, cudaStream_t s) {
@@ -493,97 +629,16 @@ q4c_status density_fp64(const q4c_tables* t, const q4c_grid* g, const double* P,
   return Q4C_OK;
 }
 
-// ------------------------------------------------------------- adjoint
-// dL/dv_p = w_p sum_ij [G^V phi_i phi_j + G^W grad_i.grad_j
-//                        + G^x (Y_i Z_j - Z_i Y_j) + G^y (Z_i X_j - X_i Z_j)
-//                        + G^z (X_i Y_j - Y_i X_j)]
-// kRowsB rows of G per pass: 8, or 4, 2 or 1 where five 8-row blocks of a
-// large batch would not fit in shared memory
-template <int kRowsB>
-__global__ void k_backward_fp64(DevBasis B, DevGrid G, int64_t b0, const int64_t* __restrict__ scr_off,
-                                const double* __restrict__ scratch, const double* GV, const double* GW,
-                                const double* Gx, const double* Gy, const double* Gz, double* __restrict__ dLdv,
-                                int weighted) {
-  extern __shared__ double sG[];  // [5][kRowsB][nb]
-  const int64_t b = b0 + blockIdx.x;
-  const int64_t p0 = G.pt_ptr[b];
-  const int np = static_cast<int>(G.pt_ptr[b + 1] - p0);
-  const int ldp = (np + 7) & ~7;
-  const int nb = static_cast<int>(G.bat_fn_ptr[b + 1] - G.bat_fn_ptr[b]);
-  const int64_t plane = static_cast<int64_t>(nb) * ldp;
-  const int64_t f0 = G.bat_fn_ptr[b];
-  const int a0 = G.bat_atom_ptr[b], na = G.bat_atom_ptr[b + 1] - a0;
-  const int64_t pp = G.bat_pair_ptr[b];
-  const double* T = scratch + scr_off[b];
-  const double* Gm[5] = {GV, GW, Gx, Gy, Gz};
-  for (int pbase = 0; pbase < np; pbase += blockDim.x) {
-    const int p = pbase + threadIdx.x;
-    double acc = 0.0;
-    for (int i0 = 0; i0 < nb; i0 += kRowsB) {
-      const int rows = min(kRowsB, nb - i0);
-      __syncthreads();
-      for (int e = threadIdx.x; e < rows * nb; e += blockDim.x) {
-        const int r = e / nb, j = e - r * nb;
-        const int ii = G.fn_info[f0 + i0 + r], jj = G.fn_info[f0 + j];
-        const int64_t off = G.pair_off[pp + static_cast<int64_t>(ii >> 16) * na + (jj >> 16)];
-        const int64_t el = off < 0 ? -1 : off + static_cast<int64_t>(ii & 0xffff) * local_nf(B, G, a0, jj >> 16) +
-                                              (jj & 0xffff);
-#pragma unroll
-        for (int m = 0; m < 5; ++m)
-          sG[(m * kRowsB + r) * nb + j] = (el < 0 || Gm[m] == nullptr) ? 0.0 : Gm[m][el];
-      }
-      __syncthreads();
-      if (p < np) {
-        double fi[kRowsB][4];
-#pragma unroll
-        for (int r = 0; r < kRowsB; ++r)
-#pragma unroll
-          for (int q = 0; q < 4; ++q) fi[r][q] = r < rows ? T[q * plane + static_cast<int64_t>(i0 + r) * ldp + p] : 0.0;
-        for (int j = 0; j < nb; ++j) {
-          const double pj = T[static_cast<int64_t>(j) * ldp + p], xj = T[plane + static_cast<int64_t>(j) * ldp + p],
-                       yj = T[2 * plane + static_cast<int64_t>(j) * ldp + p],
-                       zj = T[3 * plane + static_cast<int64_t>(j) * ldp + p];
-#pragma unroll
-          for (int r = 0; r < kRowsB; ++r) {
-            if (r >= rows) continue;
-            const double* gr = sG + r * nb + j;
-            double s = gr[0] * fi[r][0] * pj;
-            s = fma(gr[kRowsB * nb], fi[r][1] * xj + fi[r][2] * yj + fi[r][3] * zj, s);
-            s = fma(gr[2 * kRowsB * nb], fi[r][2] * zj - fi[r][3] * yj, s);
-            s = fma(gr[3 * kRowsB * nb], fi[r][3] * xj - fi[r][1] * zj, s);
-            s = fma(gr[4 * kRowsB * nb], fi[r][1] * yj - fi[r][2] * xj, s);
-            acc += s;
-          }
-        }
-      }
-    }
-    if (p < np) dLdv[p0 + p] = weighted ? G.w[p0 + p] * acc : acc;
-  }
-}
-
 // the adjoint (weighted) or gradient density (unweighted) of one wave (its
 // basis tiles in place)
 q4c_status backward_fp64_wave(const q4c_grid* g, int wv, const q4c_matrices* Gm, double* dLdv, bool weighted,
                               cudaStream_t s) {
-  const int64_t b0 = g->wave_b0[wv], b1 = g->wave_b0[wv + 1];
-  if (b1 <= b0) return Q4C_OK;
-  constexpr size_t kSmemMax = 232448;
-  const size_t row = sizeof(double) * 5 * std::max(g->max_nb, 1);  // five G rows of a batch
-  if (row > kSmemMax) {
+  if (g->max_nb > 5811) {
     set_error("the FP64 adjoint needs at most 5811 active functions per batch");
     return Q4C_EUNSUPPORTED;
   }
-  const int rows = 8 * row <= kSmemMax ? 8 : 4 * row <= kSmemMax ? 4 : 2 * row <= kSmemMax ? 2 : 1;
-  const size_t smem = rows * row;
-  auto kern = rows == 8 ? k_backward_fp64<8> : rows == 4 ? k_backward_fp64<4> : rows == 2 ? k_backward_fp64<2>
-                                                                                        : k_backward_fp64<1>;
-  Q4C_CUDA(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem)));
-  KernelScope ks("backward_fp64", s);
-  kern<<<static_cast<unsigned>(b1 - b0), 128, smem, s>>>(g->tables->view(), g->view(), b0, g->d_scr_off,
-                                                         g->d_scratch, Gm->V, Gm->W0, Gm->SOx, Gm->SOy, Gm->SOz,
-                                                         dLdv, weighted ? 1 : 0);
-  Q4C_CUDA(cudaGetLastError());
-  return Q4C_OK;
+  const double* M[5] = {Gm->V, Gm->W0, Gm->SOx, Gm->SOy, Gm->SOz};
+  return rowdot_fp64_wave<4>(g, wv, M, dLdv, weighted, "backward_fp64", s);
 }
 
 q4c_status backward_fp64(const q4c_tables* t, const q4c_grid* g, const q4c_matrices* Gm, double* dLdv,
