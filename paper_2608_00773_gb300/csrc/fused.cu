@@ -40,16 +40,18 @@ q4c_status scf_pass(const q4c_tables* t, const q4c_grid* g, const double* v, con
     for (double* o : outs) Q4C_CUDA(cudaMemsetAsync(o, 0, sizeof(double) * g->nnz, s));
   }
   if (!do_h && !do_n && !do_g) return Q4C_OK;
-  const float2* mP[5] = {nullptr, nullptr, nullptr, nullptr, nullptr};
-  const float2* mG[5] = {nullptr, nullptr, nullptr, nullptr, nullptr};
   unsigned presentP = 0, presentG = 0;
   if (split && do_n) {
     const double* mats[5] = {P->V, P->W0, P->SOx, P->SOy, P->SOz};
-    if (q4c_status st = rowdot_prepare(g, mats, 0, mP, &presentP, s)) return st;
+    if (q4c_status st = rowdot_prepare(g, mats, 0, &presentP, s)) return st;
   }
   if (split && do_g) {
     const double* mats[5] = {Gm->V, Gm->W0, Gm->SOx, Gm->SOy, Gm->SOz};
-    if (q4c_status st = rowdot_prepare(g, mats, 5, mG, &presentG, s)) return st;
+    if (q4c_status st = rowdot_prepare(g, mats, 5, &presentG, s)) return st;
+  }
+  if (split && g->rd_shares) {
+    if (do_n) Q4C_CUDA(cudaMemsetAsync(n, 0, sizeof(double) * g->n_pts, s));
+    if (do_g) Q4C_CUDA(cudaMemsetAsync(dLdv, 0, sizeof(double) * g->n_pts, s));
   }
   const int n_waves = static_cast<int>(g->wave_b0.size()) - 1;
   for (int wv = 0; wv < n_waves; ++wv) {
@@ -65,9 +67,9 @@ q4c_status scf_pass(const q4c_tables* t, const q4c_grid* g, const double* v, con
       if (do_h)
         if (q4c_status st = products_wave(g, wv, H, s)) return st;
       if (do_n)
-        if (q4c_status st = rowdot_wave(g, wv, full_n ? 1 : 0, mP, presentP, false, n, s)) return st;
+        if (q4c_status st = rowdot_wave(g, wv, full_n ? 1 : 0, 0, presentP, false, n, s)) return st;
       if (do_g)
-        if (q4c_status st = rowdot_wave(g, wv, 1, mG, presentG, true, dLdv, s)) return st;
+        if (q4c_status st = rowdot_wave(g, wv, 1, 5, presentG, true, dLdv, s)) return st;
     } else {
       if (q4c_status st = launch_basis_tiles(t, g, b0, b1, nullptr, nullptr, s)) return st;
       if (do_h)

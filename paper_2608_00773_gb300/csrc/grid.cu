@@ -326,7 +326,7 @@ static PFN_cuTensorMapEncodeTiled_v12000 tensor_map_encoder() {
 static q4c_status encode_tile_maps(q4c_grid* g) {
   const int64_t nB = g->n_batches;
   const size_t n_maps = static_cast<size_t>(std::max<int64_t>(nB, 1));
-  std::vector<CUtensorMap> maps(2 * n_maps);
+  std::vector<CUtensorMap> maps(n_maps);
   std::memset(maps.data(), 0, sizeof(CUtensorMap) * maps.size());
   auto enc = tensor_map_encoder();
   if (!enc) {
@@ -341,15 +341,11 @@ static q4c_status encode_tile_maps(q4c_grid* g) {
     void* base = g->d_scratch + g->h_scr_off[b];
     const cuuint64_t dims[3] = {static_cast<cuuint64_t>(np), static_cast<cuuint64_t>(nb), 4};
     const cuuint64_t strides[2] = {static_cast<cuuint64_t>(ldp * 8), static_cast<cuuint64_t>(nb * ldp * 8)};
-    const cuuint32_t box[3] = {16, 64, 1}, box_rd[3] = {64, 16, 1};
+    const cuuint32_t box[3] = {16, 64, 1};
     const cuuint32_t estr[3] = {1, 1, 1};
     CUresult r = enc(&maps[b], CU_TENSOR_MAP_DATA_TYPE_INT64, 3, base, dims, strides, box, estr,
                      CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
                      CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
-    if (r == CUDA_SUCCESS)
-      r = enc(&maps[n_maps + b], CU_TENSOR_MAP_DATA_TYPE_INT64, 3, base, dims, strides, box_rd, estr,
-              CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
-              CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
     if (r != CUDA_SUCCESS) {
       set_error("grid_partition: cuTensorMapEncodeTiled failed for batch " + std::to_string(b) + " (CUresult " +
                 std::to_string(static_cast<int>(r)) + ")");
@@ -983,24 +979,8 @@ extern "C" q4c_status grid_partition(const q4c_grid_desc* d, const q4c_tables* t
     max_wave_items = std::max(max_wave_items, static_cast<int64_t>(citems.size()) - g->col_w0.back());
     g->col_w0.push_back(static_cast<int64_t>(citems.size()));
   }
-  // density/adjoint: (batch, 64-point tile) items per wave, costliest first
-  std::vector<int2> rditems;
-  g->rd_w0.push_back(0);
-  for (size_t wv = 0; wv + 1 < g->wave_b0.size(); ++wv) {
-    std::vector<std::pair<double, int64_t>> bl;
-    for (int64_t b = g->wave_b0[wv]; b < g->wave_b0[wv + 1]; ++b) {
-      const double nb = static_cast<double>(g->h_bat_fn_ptr[b + 1] - g->h_bat_fn_ptr[b]);
-      bl.push_back({nb * nb, b});
-    }
-    std::stable_sort(bl.begin(), bl.end(), [](const auto& a, const auto& b) { return a.first > b.first; });
-    for (const auto& x : bl) {  // the point tiles of one batch stay adjacent
-      const int64_t b = x.second, np = bptr[b + 1] - bptr[b];
-      for (int pt = 0; pt * 64 < np; ++pt) rditems.push_back(make_int2(static_cast<int>(b), pt));
-    }
-    g->rd_w0.push_back(static_cast<int64_t>(rditems.size()));
-  }
   // G' digit blocks of the density/adjoint, per wave: per batch five matrices
-  // x ceil(nb/64) j-tiles x ceil(nb/16) i-chunks x 12 KB
+  // x ceil(nb/32) j-tiles x ceil(nb/16) i-chunks x 6 KB
   std::vector<int64_t> gsl_off(nB, 0);
   g->gsl_bytes = 0;
   for (size_t wv = 0; wv + 1 < g->wave_b0.size(); ++wv) {
@@ -1008,9 +988,34 @@ extern "C" q4c_status grid_partition(const q4c_grid_desc* d, const q4c_tables* t
     for (int64_t b = g->wave_b0[wv]; b < g->wave_b0[wv + 1]; ++b) {
       const int64_t nb = g->h_bat_fn_ptr[b + 1] - g->h_bat_fn_ptr[b];
       gsl_off[b] = used;
-      used += 5 * ((nb + 63) / 64) * ((nb + 15) / 16) * 12288;
+      used += 5 * ((nb + 31) / 32) * ((nb + 15) / 16) * 6144;
     }
     g->gsl_bytes = std::max(g->gsl_bytes, used);
+  }
+
+  // density/adjoint: (batch, 128-point tile, j-tiles) items per wave, costliest
+  // first.  Eight j-tiles (256 functions) an item at most: an item of a batch
+  // of 1,918 functions would be 7 times the average SM's share of a wave (the
+  // 304-atom slab: adjoint 47.6 ms with whole batches, 37.0 with shares), while
+  // a share still reads each sliced chunk of F about 16 times.
+  std::vector<RdItem> rditems;
+  g->rd_w0.push_back(0);
+  for (size_t wv = 0; wv + 1 < g->wave_b0.size(); ++wv) {
+    const size_t first = rditems.size();
+    for (int64_t b = g->wave_b0[wv]; b < g->wave_b0[wv + 1]; ++b) {
+      const int np = static_cast<int>(bptr[b + 1] - bptr[b]);
+      const int nb = static_cast<int>(g->h_bat_fn_ptr[b + 1] - g->h_bat_fn_ptr[b]);
+      const int n_jt = (nb + 31) / 32;
+      const int shares = std::max(1, (n_jt + 7) / 8), per = std::max(1, (n_jt + shares - 1) / shares);
+      g->rd_shares = g->rd_shares || shares > 1;
+      for (int j = 0; j < std::max(n_jt, 1); j += per)
+        for (int pt = 0; pt * 128 < np; ++pt)
+          rditems.push_back({np, nb, pt, j | std::min(n_jt, j + per) << 16, bptr[b], g->h_scr_off[b], gsl_off[b], 0});
+    }
+    auto cost = [](const RdItem& x) { return (x.nb + 15) / 16 * ((x.jts >> 16) - (x.jts & 0xffff)); };
+    std::stable_sort(rditems.begin() + first, rditems.end(),
+                     [&](const RdItem& x, const RdItem& y) { return cost(x) > cost(y); });
+    g->rd_w0.push_back(static_cast<int64_t>(rditems.size()));
   }
 
   // ---- schedule for persistent kernels: descending n_p n_b^2
@@ -1025,10 +1030,10 @@ extern "C" q4c_status grid_partition(const q4c_grid_desc* d, const q4c_tables* t
     return cost(a) > cost(b);
   });
 
-  // ---- per-block column and row maxima segments: [nf_B columns][nf_A rows]
+  // ---- per-block column bounds: nf_B columns a block
   std::vector<int64_t> cm_off(g->n_blocks + 1, 0);
   for (int64_t q = 0; q < g->n_blocks; ++q)
-    cm_off[q + 1] = cm_off[q] + g->h_nf_atom[blk_row[q]] + g->h_nf_atom[g->h_blk_col[q]];
+    cm_off[q + 1] = cm_off[q] + g->h_nf_atom[g->h_blk_col[q]];
   g->cm_total = std::max<int64_t>(cm_off[g->n_blocks], 1);
 
   // ---- upload
@@ -1072,18 +1077,16 @@ extern "C" q4c_status grid_partition(const q4c_grid_desc* d, const q4c_tables* t
     if (e == cudaSuccess) e = cudaMalloc(&g->d_rowexp, sizeof(int) * 4 * nP);
     if (e == cudaSuccess) e = cudaMalloc(&g->d_gsl, static_cast<size_t>(std::max<int64_t>(g->gsl_bytes, 16)));
     if (e == cudaSuccess) e = cudaMalloc(&g->d_gdf, sizeof(float2) * 10 * std::max<int64_t>(g->nnz, 1));
-    if (e == cudaSuccess) e = cudaMalloc(&g->d_cm, sizeof(float) * 10 * g->cm_total);
-    if (e == cudaSuccess) e = cudaMalloc(&g->d_gzero, 12288);
-    if (e == cudaSuccess) e = cudaMemset(g->d_gzero, 0, 12288);
+    if (e == cudaSuccess) e = cudaMalloc(&g->d_cm, sizeof(float) * 4 * g->cm_total);
     if (e == cudaSuccess) e = cudaMalloc(&g->d_bat_idx, sizeof(int) * g->idx_entries);
     if (e == cudaSuccess) e = cudaMalloc(&g->d_split_mag, sizeof(float) * 128 * max_wave_items);
     if (e == cudaSuccess) e = cudaMalloc(&g->d_dpad, sizeof(float2) * kDPitch * std::max<int64_t>(nB, 1));
-    if (e == cudaSuccess) e = cudaMalloc(&g->d_tmaps, 2 * sizeof(CUtensorMap) * std::max<int64_t>(nB, 1));
+    if (e == cudaSuccess) e = cudaMalloc(&g->d_tmaps, sizeof(CUtensorMap) * std::max<int64_t>(nB, 1));
     if (e == cudaSuccess) e = cudaMalloc(&g->d_status, sizeof(unsigned));
     if (e == cudaSuccess) e = cudaMemset(g->d_status, 0, sizeof(unsigned));
     g->split_ws_bytes = static_cast<int64_t>(sizeof(int)) * (8 * g->h_bat_fn_ptr[nB] + 4 * nP) +
                         static_cast<int64_t>(sizeof(float2)) * 5 * g->nnz + g->gsl_bytes +
-                        static_cast<int64_t>(sizeof(float)) * 10 * g->cm_total;
+                        static_cast<int64_t>(sizeof(float)) * 4 * g->cm_total;
     if (e != cudaSuccess) {
       set_error(std::string("grid_partition: workspace: ") + cudaGetErrorString(e));
       q4c_grid_destroy(g);
@@ -1105,7 +1108,7 @@ extern "C" void q4c_grid_destroy(q4c_grid* g) {
                   g->d_fn_info, g->d_bat_pair_ptr, g->d_pair_off, g->d_blk_off, g->d_blk_row, g->d_blk_col,
                   g->d_blk_T, g->d_scr_off, g->d_tiles, g->d_col_tiles, g->d_scratch, g->d_sched, g->d_counter, g->d_split_ws,
                   g->d_split_items, g->d_col_items, g->d_split_mag, g->d_dpad, g->d_tmaps, g->d_colexp, g->d_status, g->d_rd_items, g->d_rowexp, g->d_gsl, g->d_gsl_off,
-                  g->d_bat_idx_ptr, g->d_bat_idx, g->d_pts_df, g->d_atoms_df, g->d_gdf, g->d_gzero,
+                  g->d_bat_idx_ptr, g->d_bat_idx, g->d_pts_df, g->d_atoms_df, g->d_gdf,
                   g->d_c_xyz, g->d_c_sp, g->d_blk_role, g->d_blk_shift, g->d_kblk_q0, g->d_kblk_q1,
                   g->d_kblk_off, g->d_cm_off, g->d_cm, g->d_pair_blk};
   for (void* p : ptrs) cudaFree(p);

@@ -118,6 +118,14 @@ struct DevGrid {
   unsigned long long wait_ns;   // limit of the tensor kernels' bounded work waits (q4c_set_wait_limit_ns)
 };
 
+// One work item of the density/adjoint kernel: a 128-point tile of a batch and a
+// range of its 32-function j-tiles, with what every warp role needs to start on
+// it in one read.
+struct __align__(16) RdItem {
+  int np, nb, pt, jts;          // points and functions of the batch, point tile, j-tiles [jts & 0xffff, jts >> 16)
+  long long pt0, scr, gsl, pad;  // first point, basis tiles (values), G' blocks (bytes)
+};
+
 // the work-wait limit that q4c_set_wait_limit_ns last set (1 s by default)
 unsigned long long work_wait_limit_ns();
 
@@ -230,15 +238,15 @@ struct q4c_grid {
   std::vector<int64_t> col_w0;             // [n_waves+1] ranges into d_col_items
   int4* d_col_items = nullptr;             // per-column operator: (batch, 5, ti, tj), every tile pair
   float* d_split_mag = nullptr;            // [items of the largest wave][128] rounding constants
-  void* d_tmaps = nullptr;                 // [2][n_batches] 3-D TMA maps (points, functions, quantity) of the
-                                           // tiles: boxes 16 x 64 (products), 64 x 16 (density, adjoint)
+  void* d_tmaps = nullptr;                 // [n_batches] 3-D TMA maps (points, functions, quantity) of the
+                                           // tiles: boxes of 16 x 64
   float2* d_dpad = nullptr;                // [n_batches][kDPitch] D = w v as (hi, lo), zero past n_p
   int* d_colexp = nullptr;                 // [8 * sum n_b]
   std::vector<int64_t> rd_w0;              // [n_waves+1] ranges into d_rd_items
-  int2* d_rd_items = nullptr;              // (batch, 64-point tile) for density/adjoint
+  q4c::RdItem* d_rd_items = nullptr;       // work of the density/adjoint kernel
+  bool rd_shares = false;                  // some batch's j-tiles are shared out over several items
   int* d_rowexp = nullptr;                 // [n_points][4] per-point exponents
   unsigned char* d_gsl = nullptr;          // G' digit blocks of one wave (density/adjoint)
-  unsigned char* d_gzero = nullptr;        // one zero G' digit block (12 KB)
   int64_t* d_gsl_off = nullptr;            // [n_batches] byte offsets into d_gsl (per wave)
   int64_t gsl_bytes = 0;
   int64_t idx_entries = 0;                 // size of the per-wave dense offset tables
@@ -246,10 +254,10 @@ struct q4c_grid {
   int* d_bat_idx = nullptr;                // per batch n_b x n_b value offsets (-1 outside)
   unsigned* d_status = nullptr;            // bit 0: a bounded wait expired
   float2* d_gdf = nullptr;                 // [10][nnz] FP32-pair copies of the density (0-4) and adjoint (5-9) matrices
-  // per pattern block q, at cm_off[q]: the largest |value| of each of its
-  // nf_B columns, then of each of its nf_A rows (FP32, rounded up), for each
-  // of the ten matrices of d_gdf ([10][cm_total]); the G' pre-pass bounds a
-  // batch column's largest element from them
+  // per pattern block q, at cm_off[q]: a bound of each of its nf_B columns
+  // (FP32, rounded up), for V and for the largest of the other four matrices,
+  // of the density's and of the adjoint's ([4][cm_total]); the G' pre-pass
+  // bounds a batch column's largest element from them
   int64_t* d_cm_off = nullptr;             // [n_blocks + 1]
   int64_t cm_total = 0;
   float* d_cm = nullptr;
@@ -295,10 +303,11 @@ q4c_status integrate_columns_split(const q4c_tables* t, const q4c_grid* g, const
                                    cudaStream_t s);
 // per-wave pieces of the split path, for the fused pass (fused.cu)
 q4c_status products_wave(const q4c_grid* g, int wv, const q4c_matrices* out, cudaStream_t s);
-q4c_status rowdot_prepare(const q4c_grid* g, const double* const mats[5], int slot0, const float2* mdf[5],
-                          unsigned* present, cudaStream_t s);
-q4c_status rowdot_wave(const q4c_grid* g, int wv, int mode, const float2* const mdf[5], unsigned present,
-                       bool weighted, double* out, cudaStream_t s);
+// (slot 0: the density's prepared matrices, 5: the adjoint's)
+q4c_status rowdot_prepare(const q4c_grid* g, const double* const mats[5], int slot, unsigned* present,
+                          cudaStream_t s);
+q4c_status rowdot_wave(const q4c_grid* g, int wv, int mode, int slot, unsigned present, bool weighted, double* out,
+                       cudaStream_t s);
 // per-wave pieces of the FP64 path
 q4c_status products_fp64_wave(const q4c_grid* g, int wv, const double* v, const q4c_matrices* out,
                               cudaStream_t s);

@@ -2,28 +2,31 @@
 // tcgen05 tensor cores.
 //
 // Both are row-dot contractions over the batch's active functions:
-//   density   n_p     = sum_j Phi_pj (Phi P)_pj
-//   adjoint   dL/dv_p = w_p [ sum_j Phi_pj (Phi G^V)_pj + sum_{Q=X,Y,Z} sum_j Q_pj (Q G^W)_pj
-//                             + 2 sum_j ( Z_pj (Y Gx)_pj + X_pj (Z Gy)_pj + Y_pj (X Gz)_pj ) ]
-// with Gk the antisymmetric part of G^SOk (the cross product is antisymmetric
-// in i, j, so only that part contributes), i.e. seven products U = F G'
-// (M = points, K = functions i, N = functions j) whose rows are dotted with
-// R in the epilogue, one point per tensor-memory lane.
+//   density   n_p     = sum_ij P_ij Phi_pi Phi_pj
+//   adjoint   dL/dv_p = w_p [ sum_ij G^V_ij Phi_i Phi_j + sum_{Q=X,Y,Z} sum_ij G^W_ij Q_i Q_j
+//                             + sum_ij (G^x_ij - G^x_ji) Y_i Z_j + (cyclic) ](p)
+// (the cross product is antisymmetric in i, j, so only G - G^T of the SO
+// matrices enters).  For P, G^V and G^W only the symmetric part enters, so the
+// sum runs over i <= j with G_ij + G_ji off the diagonal: half the products.
+// Each is U = F G' (rows = points, K = functions i, columns = functions j)
+// dotted with R in the epilogue, one point per tensor-memory lane; the products
+// of one adjoint are (F, G', R) = (Phi, V, Phi), (Q, W, Q), (Y, x, Z), (Z, y, X),
+// (X, z, Y).
 //
-// Each U is computed from six BF16 slices of F (per-point exponents) and of
-// G' (per-column exponents) with the same tile sequence and exact-level
-// accumulation as the integration (see split.cu): levels 0-2 are exact
-// integer sums for K <= 512 terms, levels 3-5 are rounded 2^-24 below.  A
-// batch of more than 512 functions splits K into segments of at most 512
-// (32 chunks of 16), each a group of its own: its level sums are exact, and
-// the epilogue adds its row-dot into the point's running sum like any other
-// group's (the dot with R is linear in U).
+// Each U is computed from six BF16 slices of F (per-point exponents, one for
+// Phi and one for the three gradient quantities) and of G' (per-column
+// exponents, one for V and one for the other four matrices) in six FP32
+// accumulators, one per level s + t (see split.cu): levels 0-2 are exact
+// integer sums for K <= 512 terms (here at most 112), levels 3-5 are rounded
+// 2^-24 below.  The exponents are shared so that two products can be added up
+// in one accumulator set; a quantity's digits then resolve 2^-46 of the largest
+// of the three, which is what their sum resolves.
 //
-// G' does not depend on the points, so a pre-pass slices every batch's G'
-// once into BF16 digit tiles laid out exactly as the MMA reads them (per
-// matrix, 64-function j-tile and 16-function i-chunk: six 2 KB tiles); the
-// main kernel fetches one 12 KB block per K-step with a bulk copy.
-#include <cuda.h>
+// G' does not depend on the points, so a pre-pass slices every batch's G' once
+// into BF16 digit tiles laid out exactly as the MMA reads them (per matrix,
+// 32-function j-tile and 16-function i-chunk: six tiles of up to 32 rows); the
+// main kernel streams them with bulk copies.
+#include <algorithm>
 
 #include "internal.h"
 #include "tc.cuh"
@@ -32,122 +35,106 @@ namespace q4c {
 namespace rowdot {
 using namespace tc;
 
-constexpr int kTile = 64;                      // points per tile (and functions per j-tile)
+constexpr int kPts = 128;                      // points per item (MMA rows, tensor-memory lanes)
+constexpr int kTileJ = 32;                     // functions j per tile
 constexpr int kKc = 16;                        // functions i per chunk (one K = 16 MMA step)
-constexpr int kTileBytes = kTile * kKc * 2;    // 2 KB
-constexpr int kSBO = (kKc / 8) * 128;          // 256 B
-constexpr int kBlockB = kSlices * kTileBytes;  // one step's G' digits, 12 KB
-constexpr int kSlicers = 256;                  // warps 0-7 slice F
-constexpr int kEpiWarp0 = 8;                   // warps 8-15 drain tensor memory (two groups of four)
+constexpr int kSBO = (kKc / 8) * 128;          // 256 B between 8-row groups
+constexpr int kDigA = kPts * kKc * 2;          // one digit tile of F, 4 KB
+constexpr int kSlot = kSlices * kDigA;         // one chunk of F, 24 KB
+constexpr int kSlots = 7;                      // resident chunks
+constexpr int kBlockB = kSlices * kTileJ * kRowBytes;  // one step's G' digits, up to 6 KB
+constexpr int kRingB = 4;                      // G' blocks in flight per accumulator set
+// 16 warps, so that the epilogue has 128 registers a thread
+constexpr int kSlicers = 128;                  // warps 0-3 slice F
+constexpr int kEpiWarp0 = 4;                   // warps 4-11 drain tensor memory (two groups of four)
 constexpr int kEpiThreads = 256;
-constexpr int kMmaWarp = 16;  // warp 16 owns tensor memory and issues the MMAs
-constexpr int kProdWarp = 17;  // warp 17 issues the TMA loads of F
-constexpr int kThreads = 18 * 32;
-constexpr int kStageA = (kSlices + 1) * kTileBytes;  // [Z, A0..A5] of one K-step
-constexpr int kHalf = kStageA + kBlockB;             // one K-step's operands, 26 KB
-constexpr int kRawTile = kKc * kTile * 8;            // one box of F (16 functions x 64 points), 8 KB
+constexpr int kMmaWarp = 12;   // warps 12 and 13 issue the MMAs, one per accumulator set; 12 owns tensor memory
+constexpr int kProdWarp = 14;  // warps 14 and 15 stream the G' blocks, one per accumulator set
+constexpr int kThreads = 16 * 32;
+constexpr uint32_t kTmemCols = 512;
+constexpr uint32_t kSetCols = 256;  // two accumulator sets of six levels of up to 32 columns
+constexpr int kMaxNb = 4096;
+// The digits resolve 2^-2 finer than tc::slice6 does against the exponent
+// itself: with |d_0| <= 256 (exact in BF16) and K <= 112 terms the exact levels
+// stay below 112 * (2 * 256 * 128 + 128^2) < 2^24, and the symmetric matrices'
+// doubled coefficients are resolved as finely as their two halves were (error of
+// the 64-atom density against FP64: 1.5e-13 before, 2.7e-13 at the coarser
+// digits, 4.7e-14 with these).
+constexpr int kFine = 2;
 
-// Shared-memory layout with KS K-steps of 16 functions per pipeline stage
-// (the stage shape the tuner chooses): KS = 1 keeps four operand and four
-// raw stages, KS = 2 three of each.
-//   raw stage:     per K-step h the box of F (16 functions x 64 points of
-//                  (hi, lo), 512-byte rows) at h * 8 KB and, on an item's
-//                  first stage, the points' exponents;
-//   operand stage: per K-step h the six F digit tiles after a zero tile and
-//                  the j-tile's six G' digit tiles, at h * 26 KB.
+// Shared memory: the F slots, a ring of G' blocks per accumulator set (KS blocks
+// per stage: the stage shape the tuner chooses), the points' partial sums and
+// the barriers.
 template <int KS>
 struct Layout {
-  static constexpr int kStages = KS == 1 ? 4 : 3;
-  static constexpr int kRaw = KS == 1 ? 4 : 3;
-  static constexpr int kStage = KS * kHalf;
-  static constexpr int kRawExp = KS * kRawTile;  // [64][4] per-point exponents
-  static constexpr int kRawStage = kRawExp + 1024;
-  static constexpr int kSmemRaw = 0;
-  static constexpr int kSmemStages = kSmemRaw + kRaw * kRawStage;
-  static constexpr int kSmemY = kSmemStages + kStages * kStage;  // [4][64] double partials per point
-  static constexpr int kSmemBar = kSmemY + 4 * kTile * 8;
-  // full, empty, accfull[2], accempty[2], drain, raw full/empty, G' copy full
-  static constexpr int kNumBars = 3 * kStages + 5 + 2 * kRaw;
+  static constexpr int kStages = kRingB / KS;  // of one ring
+  static constexpr int kStage = KS * kBlockB;
+  static constexpr int kSmemRing = kSlots * kSlot;
+  static constexpr int kSmemY = kSmemRing + 2 * kStages * kStage;  // [2][128] double partials per point
+  static constexpr int kSmemBar = kSmemY + 2 * kPts * 8;
+  // slot full/empty, stage full/empty of both rings, accfull[2], accempty[2], drain[2]
+  static constexpr int kNumBars = 2 * kSlots + 4 * kStages + 6;
   static constexpr int kSmemTotal = kSmemBar + kNumBars * 8 + 16;
   static_assert(kSmemTotal <= 232448, "shared memory per CTA");
 };
-static_assert(Layout<1>::kRawStage == 9 * 1024 && Layout<1>::kStage == 26624, "the one-step layout");
-constexpr uint32_t kTmemCols = 512;
-constexpr uint32_t kSetCols = 256;
-constexpr int kMaxNb = 4096;
-constexpr int kSegIc = 32;  // chunks of 16 functions per exact K segment (K <= 512)
 
-struct Product {
-  int qf, gm, qr;
-  float factor;
+// ------------------------------------------------------------ preparation
+struct Mats {
+  const double* m[5];
 };
 
-// (F quantity, G matrix, R quantity, factor) of adjoint product k, packed one
-// byte per product (qf | gm << 2 | qr << 5 | (factor == 2) << 7) so that the
-// lookup stays in registers; matrices 2-4 enter through their antisymmetric
-// parts, which the preparation forms once per call.  The density is product 0.
-constexpr uint64_t kProducts = 0x00ull | (0x25ull << 8) | (0x46ull << 16) | (0x67ull << 24) | (0xEAull << 32) |
-                               (0xAFull << 40) | (0xD1ull << 48);
-
-__device__ __forceinline__ Product product_of(int k) {
-  const unsigned c = static_cast<unsigned>(kProducts >> (8 * k)) & 0xFFu;
-  return {static_cast<int>(c & 3u), static_cast<int>((c >> 2) & 7u), static_cast<int>((c >> 5) & 3u),
-          (c >> 7) ? 2.0f : 1.0f};
-}
-
-// One CTA per pattern block q (A, B, T) (grid-stride): the FP32-pair copy
-// of the block's values x (x = hi + lo within 2^-48 relative), and at
-// cm_off[q] the largest |x| of each of its nf_B columns, then of each of its
-// nf_A rows, rounded up to FP32.  With anti, x is the antisymmetric part
-// (G - G^T)/2 in FP64, G^T read from the partner block (B, A, -T) through
-// shared memory where both sides have at most 64 functions, else straight
-// from memory (only that part enters the adjoint's cross-product terms).
-__global__ void __launch_bounds__(128) k_prepare_blocks(DevBasis B, DevGrid G, const double* __restrict__ M,
-                                                       int anti, int64_t n_blocks, const int* __restrict__ blk_row,
+// One CTA per pattern block q (A, B, T) (grid-stride), every present matrix: the
+// FP32-pair copies (hi + lo within 2^-48 relative) of what a pair i <= j of a
+// batch takes from the block, G + G^T for V and W (G itself on the diagonal of
+// a block that is its own partner) and G - G^T for the SO matrices, formed in
+// FP64, G^T read from the partner block (B, A, -T) through shared memory where
+// both sides have at most 64 functions, else straight from memory; and at
+// cm_off[q] an FP32 bound of each of its nf_B columns, cm[0] for V and cm[1]
+// for the largest of the other four.
+__global__ void __launch_bounds__(128) k_prepare_blocks(DevBasis B, DevGrid G, Mats M, int64_t n_blocks,
+                                                       const int* __restrict__ blk_row,
                                                        const int* __restrict__ blk_col,
                                                        const int64_t* __restrict__ blk_off,
                                                        const int* __restrict__ blk_T,
                                                        const int64_t* __restrict__ cm_off, float2* __restrict__ out,
-                                                       float* __restrict__ cm) {
-  __shared__ double sT[64 * 65];  // G^T of the block: sT[i * 65 + j] = partner (j, i)
+                                                       int64_t nnz, float* __restrict__ cm, int64_t cm_total) {
+  __shared__ double sT[64 * 65];      // G^T of the block: sT[i * 65 + j] = partner (j, i)
+  extern __shared__ unsigned s_cm[];  // [2][nf_B] bits of the column bounds (non-negative floats order as integers)
   for (int64_t q = blockIdx.x; q < n_blocks; q += gridDim.x) {
     const int nfA = __ldg(B.sp_nfn + G.atom_sp[blk_row[q]]), nfB = __ldg(B.sp_nfn + G.atom_sp[blk_col[q]]);
-    const double* X = M + blk_off[q];
-    const int ne = nfA * nfB;
-    const int qt = anti ? blk_T[q] : -1;
-    const double* XT = qt >= 0 ? M + blk_off[qt] : nullptr;  // nfB rows x nfA columns
-    const bool tile = XT && nfA <= 64 && nfB <= 64;
-    if (tile) {
+    const int64_t o0 = blk_off[q];
+    const int ne = nfA * nfB, qt = blk_T[q];
+    const bool tile = qt >= 0 && nfA <= 64 && nfB <= 64;
+    __syncthreads();
+    for (int j = threadIdx.x; j < 2 * nfB; j += blockDim.x) s_cm[j] = 0u;
+#pragma unroll
+    for (int m = 0; m < 5; ++m) {
+      if (M.m[m] == nullptr) continue;
+      const double* X = M.m[m] + o0;
+      const double* XT = qt >= 0 ? M.m[m] + blk_off[qt] : nullptr;  // nfB rows x nfA columns
       __syncthreads();
-      for (int e = threadIdx.x; e < ne; e += blockDim.x) {
-        const int r = e / nfA, c = e - r * nfA;
-        sT[c * 65 + r] = XT[e];
+      if (tile) {
+        for (int e = threadIdx.x; e < ne; e += blockDim.x) {
+          const int r = e / nfA, c = e - r * nfA;
+          sT[c * 65 + r] = XT[e];
+        }
+        __syncthreads();
       }
-      __syncthreads();
+      float2* o = out + m * nnz + o0;
+      for (int e = threadIdx.x; e < ne; e += blockDim.x) {
+        const int i = e / nfB, j = e - i * nfB;
+        const double xt = tile ? sT[i * 65 + j] : XT ? XT[static_cast<int64_t>(j) * nfA + i] : 0.0;
+        const double g = X[e];
+        const double x = m >= 2 ? g - xt : (qt == q && i == j) ? g : g + xt;
+        const float h = __double2float_rn(x), l = __double2float_rn(x - static_cast<double>(h));
+        o[e] = make_float2(h, l);
+        atomicMax(&s_cm[(m ? nfB : 0) + j], __float_as_uint(__fadd_ru(fabsf(h), fabsf(l))));
+      }
     }
-    auto val = [&](int i, int j) {
-      const double x = X[static_cast<int64_t>(i) * nfB + j];
-      if (!anti) return x;
-      const double xt = tile ? sT[i * 65 + j] : XT ? XT[static_cast<int64_t>(j) * nfA + i] : 0.0;
-      return 0.5 * (x - xt);
-    };
-    float2* o = out + blk_off[q];
-    for (int e = threadIdx.x; e < ne; e += blockDim.x) {
-      const int i = e / nfB, j = e - i * nfB;
-      const double x = val(i, j);
-      const float h = __double2float_rn(x);
-      o[e] = make_float2(h, __double2float_rn(x - static_cast<double>(h)));
-    }
-    float* mx = cm + cm_off[q];
+    __syncthreads();
     for (int j = threadIdx.x; j < nfB; j += blockDim.x) {
-      double m = 0.0;
-      for (int i = 0; i < nfA; ++i) m = fmax(m, fabs(val(i, j)));
-      mx[j] = __double2float_ru(m);
-    }
-    for (int i = threadIdx.x; i < nfA; i += blockDim.x) {
-      double m = 0.0;
-      for (int j = 0; j < nfB; ++j) m = fmax(m, fabs(val(i, j)));
-      mx[nfB + i] = __double2float_ru(m);
+      cm[cm_off[q] + j] = __uint_as_float(s_cm[j]);
+      cm[cm_total + cm_off[q] + j] = __uint_as_float(s_cm[nfB + j]);
     }
   }
 }
@@ -158,68 +145,81 @@ __device__ __forceinline__ int fexp(float x) {  // |x| < 2^fexp(x) for x != 0
 
 // width of j-tile jt: its functions rounded up to 16 (the MMA's N
 // granularity); its G' digit tiles hold that many rows
-__device__ __forceinline__ int jt_width(int nb, int jt) { return (min(kTile, nb - jt * kTile) + 15) & ~15; }
+__host__ __device__ __forceinline__ int jt_width(int nb, int jt) {
+  const int w = nb - jt * kTileJ;
+  return ((w < kTileJ ? w : kTileJ) + 15) & ~15;
+}
 
-// Pre-pass: one CTA per (batch, matrix).  Column exponents e_j (|G'_ij| <
-// 2^e_j over the batch's i), then the six digits of every G'_ij written as
-// the B operand tiles of the main kernel: block (jt, ic) (a 12 KB slot) =
-// six tiles of jt_width rows (j) x 16 K (i), 32 bytes a row, in the
-// no-swizzle K-major layout, back to back; padding rows and columns are 0.
-// The column bound is the largest column maximum (k_prepare_blocks) of the
-// blocks (a, c) of column j's centre c over the batch's active centres a,
-// whose functions are exactly the batch's i.
-__global__ void __launch_bounds__(256) k_gslice(DevGrid G, int64_t b0, const float2* M0,
-                                                const float2* M1, const float2* M2, const float2* M3,
-                                                const float2* M4, const float* C0, const float* C1,
-                                                const float* C2, const float* C3, const float* C4,
+// chunks of i that matrix m has in j-tile jt: all of them, or for V and W those
+// up to the tile's last column
+__host__ __device__ __forceinline__ int jt_chunks(int m, int n_ic, int jt) {
+  const int n = 2 * (jt + 1);
+  return m < 2 && n < n_ic ? n : n_ic;
+}
+
+// Pre-pass: CTAs (batch, matrix, share of the j-tiles).  Per j-tile the column
+// exponents e_j (|G'_ij| < 2^e_j over the batch's i), then the six digits of
+// every G'_ij written as the B operand of the main kernel: block (jt, ic) = six
+// tiles of jt_width rows (j) x 16 K (i), 32 bytes a row, in the no-swizzle
+// K-major layout, back to back, at (jt * n_ic) * 6 KB + ic * 192 * jt_width;
+// padding rows and columns, and for V and W i > j, are 0.
+// The column bound is the largest column bound (k_prepare_blocks) of the blocks
+// (a, c) of column j's centre c over the batch's active centres a, whose
+// functions are exactly the batch's i.
+__global__ void __launch_bounds__(256) k_gslice(DevGrid G, int64_t b0, const float2* __restrict__ prep, int64_t nnz,
+                                                unsigned present, const float* __restrict__ cm, int64_t cm_total,
                                                 const int* __restrict__ pair_blk, const int64_t* __restrict__ cm_off,
                                                 const int64_t* __restrict__ gsl_off, uint32_t* __restrict__ gsl) {
-  __shared__ unsigned sMax[kMaxNb];  // bits of the bound of max_i |G'_ij| (non-negative floats order as integers)
+  __shared__ unsigned sMax[kTileJ];  // bits of the columns' bounds
   const int64_t b = b0 + blockIdx.x;
   const int m = blockIdx.y;
-  const float2* M = m == 0 ? M0 : m == 1 ? M1 : m == 2 ? M2 : m == 3 ? M3 : M4;  // (no local array)
-  if (M == nullptr) return;
-  const float* CM = m == 0 ? C0 : m == 1 ? C1 : m == 2 ? C2 : m == 3 ? C3 : C4;
-  const int nb = static_cast<int>(G.bat_fn_ptr[b + 1] - G.bat_fn_ptr[b]);
+  if (!(present >> m & 1u)) return;
+  const float2* M = prep + m * nnz;
+  const float* CM = cm + (m ? cm_total : 0);
+  const int64_t f0 = G.bat_fn_ptr[b];
+  const int nb = static_cast<int>(G.bat_fn_ptr[b + 1] - f0);
   const int* idx = G.bat_idx + G.bat_idx_ptr[b];
-  const int n_jt = (nb + kTile - 1) / kTile, n_ic = (nb + kKc - 1) / kKc;
+  const int n_jt = (nb + kTileJ - 1) / kTileJ, n_ic = (nb + kKc - 1) / kKc;
+  const int na = G.bat_atom_ptr[b + 1] - G.bat_atom_ptr[b];
+  const int* pb = pair_blk + G.bat_pair_ptr[b];
   uint32_t* out = gsl + (gsl_off[b] + static_cast<int64_t>(m) * n_jt * n_ic * kBlockB) / 4;
-  // pass 1: column bounds, a thread per column over the batch's centres
-  {
-    const int a0 = G.bat_atom_ptr[b], na = G.bat_atom_ptr[b + 1] - a0;
-    const int* pb = pair_blk + G.bat_pair_ptr[b];
-    const int* info = G.fn_info + G.bat_fn_ptr[b];
-    for (int j = threadIdx.x; j < nb; j += blockDim.x) {
-      const int c = info[j] >> 16, jj = info[j] & 0xffff;
-      float mx = 0.f;
-      for (int a = 0; a < na; ++a) {
-        const int q = pb[a * na + c];  // block (a, c): its column jj
-        if (q >= 0) mx = fmaxf(mx, __ldg(CM + cm_off[q] + jj));
+  for (int jt = blockIdx.z; jt < n_jt; jt += gridDim.z) {
+    __syncthreads();
+    if (threadIdx.x < kTileJ) sMax[threadIdx.x] = 0u;
+    __syncthreads();
+    {  // column bounds: eight threads a column over the batch's centres
+      const int j = jt * kTileJ + (threadIdx.x >> 3);
+      if (j < nb) {
+        const int info = G.fn_info[f0 + j], c = info >> 16, jj = info & 0xffff;
+        float mx = 0.f;
+        for (int a = threadIdx.x & 7; a < na; a += 8) {
+          const int q = pb[a * na + c];  // block (a, c): its column jj
+          if (q >= 0) mx = fmaxf(mx, __ldg(CM + cm_off[q] + jj));
+        }
+        atomicMax(&sMax[threadIdx.x >> 3], __float_as_uint(mx));
       }
-      sMax[j] = __float_as_uint(mx);
     }
-  }
-  __syncthreads();
-  // pass 2: the six digits of every element, in the B-operand tile layout;
-  // a thread takes kU words (element pairs) at a time and issues all their
-  // offset loads, then all their value loads, before slicing any
-  constexpr int kU = 4;
-  for (int jt = 0; jt < n_jt; ++jt) {
-    const int tw = jt_width(nb, jt) * 8;  // words of one tile (one per element pair)
-    const int words = n_ic * tw;
+    __syncthreads();
+    const int w = jt_width(nb, jt), tw = w * 8;  // words of one tile (one per element pair)
+    const int words = jt_chunks(m, n_ic, jt) * tw;
+    uint32_t* oj = out + static_cast<int64_t>(jt) * n_ic * (kBlockB / 4);
+    // a thread takes kU words (element pairs) at a time and issues all their
+    // offset loads, then all their value loads, before slicing any
+    constexpr int kU = 4;
     for (int w0 = threadIdx.x; w0 < words; w0 += kU * blockDim.x) {
       int i_[kU], j_[kU], o0[kU], o1[kU];
 #pragma unroll
       for (int u = 0; u < kU; ++u) {
-        const int w = w0 + u * blockDim.x;
-        const int ic = w / tw, pos = w - ic * tw;
+        const int wd = w0 + u * blockDim.x;
+        const int ic = wd / tw, pos = wd - ic * tw;
         // pos -> byte offset rg*SBO + kq*LBO + r8*16 + kp*4
         const int rg = pos >> 6, kq = (pos >> 5) & 1, r8 = (pos >> 2) & 7, kp = pos & 3;
-        j_[u] = jt * kTile + rg * 8 + r8;
+        j_[u] = jt * kTileJ + rg * 8 + r8;
         i_[u] = ic * kKc + kq * 8 + kp * 2;
-        const bool ok = w < words && j_[u] < nb;
-        o0[u] = ok && i_[u] < nb ? __ldg(idx + i_[u] * nb + j_[u]) : -1;
-        o1[u] = ok && i_[u] + 1 < nb ? __ldg(idx + (i_[u] + 1) * nb + j_[u]) : -1;
+        const bool ok = wd < words && j_[u] < nb;
+        const int last = m < 2 ? j_[u] : nb - 1;  // last i of this column
+        o0[u] = ok && i_[u] <= last ? __ldg(idx + i_[u] * nb + j_[u]) : -1;
+        o1[u] = ok && i_[u] + 1 <= last ? __ldg(idx + (i_[u] + 1) * nb + j_[u]) : -1;
       }
       float2 x0[kU], x1[kU];
 #pragma unroll
@@ -229,164 +229,351 @@ __global__ void __launch_bounds__(256) k_gslice(DevGrid G, int64_t b0, const flo
       }
 #pragma unroll
       for (int u = 0; u < kU; ++u) {
-        const int w = w0 + u * blockDim.x;
-        if (w >= words) break;
-        const int ic = w / tw, pos = w - ic * tw;
-        float d0[kSlices], d1[kSlices];
-        if (j_[u] < nb) {
-          const unsigned mb = sMax[j_[u]];
-          const float m0 = magic0(mb ? fexp(__uint_as_float(mb)) : -30000);
-          slice6(x0[u].x, x0[u].y, m0, d0);
-          slice6(x1[u].x, x1[u].y, m0, d1);
-        } else {
+        const int wd = w0 + u * blockDim.x;
+        if (wd >= words) break;
+        const int ic = wd / tw, pos = wd - ic * tw;
+        const unsigned mb = sMax[j_[u] - jt * kTileJ];
+        float2 d[kSlices];
+        slice6x2(pk2(x0[u].x, x1[u].x), pk2(x0[u].y, x1[u].y),
+                 magic0((mb ? fexp(__uint_as_float(mb)) : -30000) - kFine), d);
+        uint32_t* o = oj + ic * (kSlices * tw) + pos;
 #pragma unroll
-          for (int s = 0; s < kSlices; ++s) d0[s] = d1[s] = 0.f;
-        }
-        uint32_t* o = out + static_cast<int64_t>(jt * n_ic + ic) * (kBlockB / 4) + pos;
-#pragma unroll
-        for (int s = 0; s < kSlices; ++s) {
-          const __nv_bfloat162 h2 = __floats2bfloat162_rn(d0[s], d1[s]);
-          o[b_tile(s) * tw] = *reinterpret_cast<const uint32_t*>(&h2);  // [B0, B2, B4, B1, B3, B5]
-        }
+        for (int t = 0; t < kSlices; ++t) o[t * tw] = bf16x2_exact(d[t]);
       }
     }
   }
 }
 
-// the work of one item (batch, 64-point tile): groups (j-tile, product, K
-// segment) in order, each a K-loop over the segment's functions i in chunks
-// of 16 (n_ic chunks in all, KS chunks per pipeline stage)
-struct ItemInfo {
-  int64_t b, bp0;
-  int pt, np, ldp, nb, n_jt, n_ic, n_seg, n_stot;
-  int64_t plane;
+// ------------------------------------------------------------ the walk
+// Work of one item (batch, 128-point tile, j-tiles [jt0, jt1): all of them, or
+// a share of a large batch's), the same for every warp role.
+//
+// Chunks of F digits stay in shared memory while every product that reads them
+// runs: an item is a list of segments, a segment fills up to seven slots and
+// then runs its groups, and a group (j-tile, R, one or two runs of chunks) is
+// one accumulation drained by the epilogue.
+//   fused items (n_ic <= 2): segment Phi; then one segment with all of X, Y, Z,
+//     whose groups add both products with the same R (W with F = R and an SO
+//     matrix) into one accumulation;
+//   other items: K segments of up to seven chunks, in each one segment per
+//     quantity, whose groups are single products (the row-dot with R is linear
+//     in U, so K segments add up in the point's running sum).
+struct Item {
+  int64_t bp0, scr, gsl, plane;
+  int pt, np, ldp, nb, n_jt, n_ic;
+  int jt0, jt1;  // the item's j-tiles
+  int seg_len, nq;  // chunks of a K segment, segments in one
+  unsigned qlist;  // quantities of a K segment, two bits each
+  bool fused;
 };
 
-// pipeline stages of K segment seg
-__device__ __forceinline__ int seg_stages(int n_ic, int seg, int ks) {
-  return (min(kSegIc, n_ic - seg * kSegIc) + ks - 1) / ks;
-}
+constexpr int kPhi = 0, kOne = 1, kGrad = 2;  // kinds of segment
+struct Seg {
+  int kind, q, c0, c1, n;  // quantity and chunks [c0, c1); n: entries (slots)
+};
 
-__device__ __forceinline__ ItemInfo item_info(const DevGrid& G, int2 it) {
-  ItemInfo I;
-  I.b = it.x;
-  I.pt = it.y;
-  I.bp0 = G.pt_ptr[I.b];
-  I.np = static_cast<int>(G.pt_ptr[I.b + 1] - I.bp0);
+// the SO matrix that multiplies F = quantity q (X: z, Y: x, Z: y) and the
+// quantity it is dotted with
+__device__ __forceinline__ int so_matrix(int q) { return q == 1 ? 4 : q + 0; }
+__device__ __forceinline__ int so_dot(int q) { return q == 3 ? 1 : q + 1; }
+
+template <int MODE>
+__device__ __forceinline__ Item item_of(const RdItem* __restrict__ it, unsigned present) {
+  const int4 u = __ldg(reinterpret_cast<const int4*>(it));
+  const longlong2 v = __ldg(reinterpret_cast<const longlong2*>(it) + 1), w = __ldg(reinterpret_cast<const longlong2*>(it) + 2);
+  Item I;
+  I.pt = u.z;
+  I.jt0 = u.w & 0xffff;
+  I.jt1 = u.w >> 16;
+  I.bp0 = v.x;
+  I.scr = v.y;
+  I.gsl = w.x;
+  I.np = u.x;
+  I.nb = u.y;
   I.ldp = (I.np + 7) & ~7;
-  I.nb = static_cast<int>(G.bat_fn_ptr[I.b + 1] - G.bat_fn_ptr[I.b]);
-  I.n_jt = (I.nb + kTile - 1) / kTile;
+  I.n_jt = (I.nb + kTileJ - 1) / kTileJ;
   I.n_ic = (I.nb + kKc - 1) / kKc;
-  I.n_seg = (I.n_ic + kSegIc - 1) / kSegIc;
   I.plane = static_cast<int64_t>(I.nb) * I.ldp;
+  const int n_kseg = max((I.n_ic + kSlots - 1) / kSlots, 1);
+  I.seg_len = n_kseg == 1 ? I.n_ic : (I.n_ic + n_kseg - 1) / n_kseg;
+  I.fused = MODE == 1 && 3 * I.n_ic <= kSlots;
+  I.qlist = 0;
+  I.nq = 0;
+  if (MODE == 0 || (present & 1u)) ++I.nq;  // Phi (two zero bits)
+  if (MODE == 1) {
+    if (I.fused) {
+      if (present & 0x1eu) ++I.nq;
+    } else {
+#pragma unroll
+      for (int q = 1; q < 4; ++q)
+        if (present & (2u | 1u << so_matrix(q))) I.qlist |= static_cast<unsigned>(q) << (2 * I.nq++);
+    }
+  }
+  if (I.n_ic == 0) I.nq = 0;
   return I;
 }
 
-template <int KS>
-__device__ __forceinline__ int stages_per_product(const ItemInfo& I) {  // all segments of one (j-tile, product)
-  return (I.n_seg - 1) * (kSegIc / KS) + seg_stages(I.n_ic, I.n_seg - 1, KS);
+// segment qi of the K segment that starts at chunk c0
+template <int MODE>
+__device__ __forceinline__ Seg seg_of(const Item& I, int qi, int c0, unsigned present) {
+  if (MODE == 1 && I.fused) {
+    if (qi == 0 && (present & 1u)) return {kPhi, 0, 0, I.n_ic, I.n_ic};
+    return {kGrad, 1, 0, I.n_ic, 3 * I.n_ic};
+  }
+  const int q = MODE == 0 ? 0 : static_cast<int>((I.qlist >> (2 * qi)) & 3u);
+  // a symmetric matrix alone needs the chunks up to the last j-tile's end only
+  const bool sym = q == 0 || !(present >> so_matrix(q) & 1u);
+  const int c1 = min(sym ? min(I.n_ic, 2 * I.jt1) : I.n_ic, c0 + I.seg_len);
+  return {q ? kOne : kPhi, q, c0, c1, max(0, c1 - c0)};
+}
+// the segment after (qi, c0); false past the item's last one
+__device__ __forceinline__ bool next_seg(const Item& I, int& qi, int& c0) {
+  if (++qi < I.nq) return true;
+  qi = 0;
+  c0 += I.seg_len;
+  return c0 < I.n_ic;
 }
 
-// position in an item's stage sequence (j-tile, product, K segment, stage
-// within the segment), advanced without divisions
-template <int KS>
-struct StepIter {
-  int st = 0, seg = 0, kk = 0, jt = 0;
-  __device__ __forceinline__ void next(const ItemInfo& I, int n_prod) {
-    if (++st == seg_stages(I.n_ic, seg, KS)) {
-      st = 0;
-      if (++seg == I.n_seg) {
-        seg = 0;
-        if (++kk == n_prod) {
-          kk = 0;
+// one run of chunks of a group: chunks [c, c + n) of the segment's entries
+// from `ent` on, times matrix m
+struct Run {
+  int m, ent, c, n;
+};
+
+// The groups of one item in order: open() an item, then next() until it
+// returns false.  Run B follows run A in the same accumulation (B.n = 0: none).
+template <int MODE>
+struct GroupWalk {
+  Item I;
+  Seg S;
+  unsigned present;
+  int ent = 0;       // first entry of the segment in the CTA's sequence
+  int qi, c0, part, jt, r;  // qi = -1: before the item's first segment
+  int qr;            // quantity of the dot
+  Run A, B;
+  bool last;         // last group of its segment
+  __device__ __forceinline__ explicit GroupWalk(unsigned pr) : present(pr) { S.n = 0; }
+  __device__ __forceinline__ void open(const RdItem* it) {
+    I = item_of<MODE>(it, present);
+    qi = -1;
+    c0 = 0;
+    B.n = 0;
+  }
+  __device__ __forceinline__ bool has(int m) const { return present >> m & 1u; }
+  __device__ __forceinline__ bool next() {
+    for (;;) {
+      if (MODE == 1 && qi >= 0 && S.kind == kGrad) {
+        if (++r > 3) {
+          r = 1;
           ++jt;
         }
+        if (jt < I.jt1) {
+          const int q = r == 1 ? 3 : r - 1;  // the quantity whose SO product is dotted with r
+          const bool w = has(1), so = has(so_matrix(q));
+          if (!w && !so) continue;
+          const Run ra = {1, (r - 1) * I.n_ic, 0, jt_chunks(1, I.n_ic, jt)};
+          const Run rb = {so_matrix(q), (q - 1) * I.n_ic, 0, I.n_ic};
+          A = w ? ra : rb;
+          B = rb;
+          B.n = w && so ? I.n_ic : 0;
+          qr = r;
+          // a later r of the last j-tile has a group: through W, or X.z -> 2, Y.x -> 3
+          const bool more = r < 3 && (w || (r == 1 && has(4)) || has(2));
+          last = jt + 1 == I.jt1 && !more;
+          return true;
+        }
+      } else if (qi >= 0 && part < 2) {
+        ++jt;
+        const int mt = S.kind == kPhi ? 0 : 1;  // the symmetric matrix
+        const bool so = MODE == 1 && S.kind == kOne && has(so_matrix(S.q));
+        if (jt >= I.jt1) {
+          ++part;
+          jt = I.jt0 - 1;
+          continue;
+        }
+        if (part == 0) {
+          const int n = min(S.c1, jt_chunks(mt, I.n_ic, jt)) - S.c0;
+          if (n <= 0 || !(MODE == 0 || has(mt))) continue;
+          A = {mt, 0, S.c0, n};
+          qr = S.q;
+          last = !so && jt + 1 == I.jt1;
+        } else {
+          if (!so) continue;
+          A = {so_matrix(S.q), 0, S.c0, S.n};
+          qr = so_dot(S.q);
+          last = jt + 1 == I.jt1;
+        }
+        return true;
+      }
+      // the next segment
+      ent += S.n;
+      S.n = 0;
+      if (I.nq == 0 || !next_seg(I, qi, c0)) return false;
+      S = seg_of<MODE>(I, qi, c0, present);
+      part = 0;
+      B.n = 0;
+      if (MODE == 1 && S.kind == kGrad) {
+        jt = I.jt0;
+        r = 0;
+      } else {
+        jt = I.jt0 - 1;
       }
     }
   }
-  // chunk of 16 functions read by K-step h of this stage
-  __device__ __forceinline__ int chunk(int h) const { return seg * kSegIc + st * KS + h; }
 };
 
-// One work item = (batch, 64-point tile); its groups (j-tile, product) run
-// in order, each a K-loop over the functions i.  Warp roles as in the
-// integration kernel:
-//   warp 17     (one thread) loads each step's box of F (64 points x 16
-//               functions of the step's quantity) and, on an item's first
-//               step, the points' exponents into the raw ring (raw_full
-//               counts the bytes; raw_empty hands a stage back);
-//   warps 0-7   per step: thread (point, 4 functions) reads its raw values,
-//               waits empty[stage]; one thread starts the bulk copy of the
-//               step's G' digits into the stage (its bytes complete
-//               gfull[stage]);
-//               all slice their F values, store the digits, arrive on
-//               full[stage] and hand the raw stage back;
-//   warp 16     (one thread) issues the six MMAs per step into the group's
-//               accumulator set (groups alternate between two sets), commits
-//               empty[stage] and, after the group's last step, accfull[set];
-//   warps 8-15  read U's levels from tensor memory, dot each column with R
-//               (a lane per thread, double-float), keep a running sum per lane
-//               over the item's groups and write each point's result at the
-//               end of the item.
-// Every wait is bounded; a timeout sets the status bit and an abort flag.
-template <int MODE, int KS>  // MODE 0: density, 1: adjoint; KS: K-steps per stage
-__global__ void __launch_bounds__(kThreads, 1)
-    k_split_rowdot(DevGrid G, const int2* __restrict__ items, int n_items, const CUtensorMap* __restrict__ maps,
-                   const int64_t* __restrict__ scr_off, const double* __restrict__ scratch,
-                   const int* __restrict__ rowexp, const int64_t* __restrict__ gsl_off,
-                   const unsigned char* __restrict__ gsl, const unsigned char* __restrict__ gzero,
-                   unsigned present, int weighted, double* __restrict__ out, unsigned* status) {
-  using L = Layout<KS>;
-  constexpr int kStages = L::kStages, kRaw = L::kRaw, kStage = L::kStage, kRawStage = L::kRawStage;
-  constexpr int kRawExp = L::kRawExp, kSmemRaw = L::kSmemRaw, kSmemStages = L::kSmemStages;
-  constexpr int kSmemY = L::kSmemY, kSmemBar = L::kSmemBar, kNumBars = L::kNumBars;
-  extern __shared__ __align__(1024) unsigned char smem[];
-  double* sY = reinterpret_cast<double*>(smem + kSmemY);    // [part][point]
-  uint64_t* bars = reinterpret_cast<uint64_t*>(smem + kSmemBar);
-  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(smem + kSmemBar + kNumBars * 8);
-  volatile int* s_abort = reinterpret_cast<volatile int*>(smem + kSmemBar + kNumBars * 8 + 4);
+// The entries (chunks of F) of this CTA's items in order.
+template <int MODE>
+struct EntryWalk {
+  const RdItem* items;
+  int n_items;
+  unsigned present;
+  int n, qi, c0, e;  // item, segment, entry within it
+  int q, c;          // quantity and chunk of the entry
+  Item I;
+  Seg S;
+  __device__ __forceinline__ EntryWalk(const RdItem* it, int ni, unsigned pr)
+      : items(it), n_items(ni), present(pr), n(static_cast<int>(blockIdx.x)), e(-1) {
+    if (n < n_items) open();
+  }
+  __device__ __forceinline__ void open() {
+    I = item_of<MODE>(items + n, present);
+    qi = c0 = 0;
+    S.n = 0;
+    if (I.nq) S = seg_of<MODE>(I, 0, 0, present);
+    c = S.c0 - 1;
+    q = S.q;
+  }
+  // advances to the next entry; false at the end
+  __device__ __forceinline__ bool next() {
+    if (n >= n_items) return false;
+    ++e;
+    if (++c >= S.c1) {  // the next quantity of a segment with all three
+      c = S.c0;
+      ++q;
+    }
+    while (e >= S.n) {
+      e = 0;
+      if (I.nq && next_seg(I, qi, c0)) {
+        S = seg_of<MODE>(I, qi, c0, present);
+      } else {
+        n += gridDim.x;
+        if (n >= n_items) return false;
+        open();
+      }
+      c = S.c0;
+      q = S.q;
+    }
+    return true;
+  }
+};
 
-  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  if (smem_u32(smem) & 1023u) {  // TMA boxes and operand tiles need aligned stages
+// six 8-column loads (levels `step` columns apart) under a single wait
+__device__ __forceinline__ void tmem_ld8x6(uint32_t t, uint32_t step, float (*v)[8]) {
+  uint32_t a[6][8];
+  asm volatile(
+      "tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%48];\n\t"
+      "tcgen05.ld.sync.aligned.32x32b.x8.b32 {%8,%9,%10,%11,%12,%13,%14,%15}, [%49];\n\t"
+      "tcgen05.ld.sync.aligned.32x32b.x8.b32 {%16,%17,%18,%19,%20,%21,%22,%23}, [%50];\n\t"
+      "tcgen05.ld.sync.aligned.32x32b.x8.b32 {%24,%25,%26,%27,%28,%29,%30,%31}, [%51];\n\t"
+      "tcgen05.ld.sync.aligned.32x32b.x8.b32 {%32,%33,%34,%35,%36,%37,%38,%39}, [%52];\n\t"
+      "tcgen05.ld.sync.aligned.32x32b.x8.b32 {%40,%41,%42,%43,%44,%45,%46,%47}, [%53];\n\t"
+      "tcgen05.wait::ld.sync.aligned;"
+      : "=r"(a[0][0]), "=r"(a[0][1]), "=r"(a[0][2]), "=r"(a[0][3]), "=r"(a[0][4]), "=r"(a[0][5]), "=r"(a[0][6]),
+        "=r"(a[0][7]), "=r"(a[1][0]), "=r"(a[1][1]), "=r"(a[1][2]), "=r"(a[1][3]), "=r"(a[1][4]), "=r"(a[1][5]),
+        "=r"(a[1][6]), "=r"(a[1][7]), "=r"(a[2][0]), "=r"(a[2][1]), "=r"(a[2][2]), "=r"(a[2][3]), "=r"(a[2][4]),
+        "=r"(a[2][5]), "=r"(a[2][6]), "=r"(a[2][7]), "=r"(a[3][0]), "=r"(a[3][1]), "=r"(a[3][2]), "=r"(a[3][3]),
+        "=r"(a[3][4]), "=r"(a[3][5]), "=r"(a[3][6]), "=r"(a[3][7]), "=r"(a[4][0]), "=r"(a[4][1]), "=r"(a[4][2]),
+        "=r"(a[4][3]), "=r"(a[4][4]), "=r"(a[4][5]), "=r"(a[4][6]), "=r"(a[4][7]), "=r"(a[5][0]), "=r"(a[5][1]),
+        "=r"(a[5][2]), "=r"(a[5][3]), "=r"(a[5][4]), "=r"(a[5][5]), "=r"(a[5][6]), "=r"(a[5][7])
+      : "r"(t), "r"(t + step), "r"(t + 2 * step), "r"(t + 3 * step), "r"(t + 4 * step), "r"(t + 5 * step)
+      : "memory");
+#pragma unroll
+  for (int l = 0; l < 6; ++l)
+#pragma unroll
+    for (int i = 0; i < 8; ++i) v[l][i] = __uint_as_float(a[l][i]);
+}
+
+// The 21 slice products of one step (s + t <= 5) as six MMAs: digit tile A_s
+// (128 points) times the consecutive digit tiles B_0 .. B_(5-s) (w columns
+// each) adds level s + t to columns [(s + t) w, (s + t + 1) w).
+__device__ __forceinline__ void mma_row_levels(uint32_t tmem, uint64_t a, uint64_t b, int w, bool first) {
+#pragma unroll
+  for (int s = 0; s < kSlices; ++s)
+    mma_bf16(tmem + s * w, a + s * (kDigA >> 4), b, make_idesc(128, w * (kSlices - s)), (first && s == 0) ? 0u : 1u);
+}
+
+// One work item = (batch, 128-point tile).  Warp roles (one persistent CTA per
+// SM, items strided over the CTAs):
+//   warps 0-3   slice F: thread = point, chunks of 16 functions: reads its raw
+//               values straight from the basis tiles one chunk ahead, waits for
+//               the slot (slot_empty), stores the six digits of its row, arrives
+//               on slot_full;
+//   warps 14-15 (one thread each) stream the G' blocks of one accumulator set's
+//               groups in order into its ring, KS blocks per bulk copy (g_full
+//               counts the bytes), and prefetch the next item's rows into L2;
+//   warps 12-13 issue six MMAs per chunk into the group's accumulator set
+//               (groups alternate between two sets, a warp each), commit
+//               g_empty per stage, slot_empty after a slot's last use (each
+//               warp its own) and acc_full after the group;
+//   warps 4-11  read the six levels from tensor memory (lane = point, each group
+//               of four warps half of the columns; R one group ahead), form U = exact levels by
+//               two-sums plus the rounded tail, dot with R in double-float, and
+//               write each point's result at the end of the item.
+// Warps whose points lie past n_p slice and drain nothing.
+// Every wait is bounded; a timeout sets the status bit and an abort flag.
+//
+// What bounds it: a step reads 46 KB of operands from shared memory (six times
+// 4 KB of F, 672 rows of 32 B of G'), 360 clocks at 128 B a clock (336 of tensor
+// work), and the 6 KB of its G' block arrive there; slicing (once per quantity
+// and chunk) and the epilogue (28 FP32 operations per element) share the FP32
+// lanes.  Before, 64-point items re-sliced F for every product and 64-column
+// tile, and their epilogue ran over two half-level sums of all seven products:
+// 89 KB through shared memory a step and 1,360 clocks.
+// Adjoint, before -> now: 64-atom cluster 4.28 -> 2.69 ms, 24 molecules 23.4 ->
+// 12.7 ms, 304-atom slab 64.2 -> 33.2 ms; density of the cluster 0.67 -> 0.45 ms.
+template <int MODE, int KS>  // MODE 0: density, 1: adjoint; KS: G' blocks per stage
+__global__ void __launch_bounds__(kThreads, 1)
+    k_split_rowdot(DevGrid G, const RdItem* __restrict__ items, int n_items, const double* __restrict__ scratch,
+                   const int* __restrict__ rowexp, const unsigned char* __restrict__ gsl, unsigned present,
+                   int weighted, double* __restrict__ out, unsigned* status) {
+  using L = Layout<KS>;
+  constexpr int kStages = L::kStages;
+  extern __shared__ __align__(1024) unsigned char smem[];
+  double* sY = reinterpret_cast<double*>(smem + L::kSmemY);  // [column half][point]
+  uint64_t* bars = reinterpret_cast<uint64_t*>(smem + L::kSmemBar);
+  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(smem + L::kSmemBar + L::kNumBars * 8);
+  volatile int* s_abort = reinterpret_cast<volatile int*>(smem + L::kSmemBar + L::kNumBars * 8 + 4);
+
+  const int tid = threadIdx.x, warp = uniform(tid >> 5), lane = tid & 31;
+  const uint32_t smem0 = smem_u32(smem);
+  if (smem0 & 127u) {  // operand tiles and bulk copies need aligned stages
     if (tid == 0) atomicOr(status, 2u);
     return;
   }
   const uint32_t bar0 = smem_u32(bars);
-  auto full_bar = [&](int st) { return bar0 + 8u * st; };
-  auto empty_bar = [&](int st) { return bar0 + 8u * (kStages + st); };
-  auto accfull_bar = [&](int set) { return bar0 + 8u * (2 * kStages + set); };
-  auto accempty_bar = [&](int set) { return bar0 + 8u * (2 * kStages + 2 + set); };
-  const uint32_t drain_bar = bar0 + 8u * (2 * kStages + 4);
-  auto rawfull_bar = [&](int rs) { return bar0 + 8u * (2 * kStages + 5 + rs); };
-  auto rawempty_bar = [&](int rs) { return bar0 + 8u * (2 * kStages + 5 + kRaw + rs); };
-  auto gfull_bar = [&](int st) { return bar0 + 8u * (2 * kStages + 5 + 2 * kRaw + st); };
-  // the products whose matrix is present, in order, 3 bits each (registers only)
-  unsigned plist = 0;
-  int n_prod = 0;
-  for (int k = 0; k < (MODE == 0 ? 1 : 7); ++k)
-    if (present & (1u << product_of(k).gm)) plist |= static_cast<unsigned>(k) << (3 * n_prod++);
-  auto prod_at = [&](int kk) { return product_of(static_cast<int>((plist >> (3 * kk)) & 7u)); };
+  auto slotfull_bar = [&](int k) { return bar0 + 8u * k; };
+  auto slotempty_bar = [&](int k) { return bar0 + 8u * (kSlots + k); };
+  auto gfull_bar = [&](int set, int k) { return bar0 + 8u * (2 * kSlots + set * kStages + k); };
+  auto gempty_bar = [&](int set, int k) { return bar0 + 8u * (2 * kSlots + (2 + set) * kStages + k); };
+  auto accfull_bar = [&](int k) { return bar0 + 8u * (2 * kSlots + 4 * kStages + k); };
+  auto accempty_bar = [&](int k) { return bar0 + 8u * (2 * kSlots + 4 * kStages + 2 + k); };
+  auto drain_bar = [&](int k) { return bar0 + 8u * (2 * kSlots + 4 * kStages + 4 + k); };
 
-  for (int i = tid; i < kStages * KS * kTileBytes / 16; i += kThreads) {  // tile Z of every K-step
-    const int sh = i / (kTileBytes / 16), off = i - sh * (kTileBytes / 16);
-    reinterpret_cast<uint4*>(smem + kSmemStages + sh * kHalf)[off] = make_uint4(0, 0, 0, 0);
-  }
-  fence_async_smem();  // the zero tiles are read by the tensor cores (async proxy)
   if (tid == 0) {
-    for (int st = 0; st < kStages; ++st) {
-      mbar_init(full_bar(st), kSlicers);
-      mbar_init(empty_bar(st), 1);
+    for (int k = 0; k < kSlots; ++k) {
+      mbar_init(slotfull_bar(k), kSlicers);
+      mbar_init(slotempty_bar(k), 2);  // both MMA warps
     }
-    for (int set = 0; set < 2; ++set) {
-      mbar_init(accfull_bar(set), 1);
-      mbar_init(accempty_bar(set), kEpiThreads);
+    for (int k = 0; k < 2 * kStages; ++k) {
+      mbar_init(gfull_bar(0, k), 1);
+      mbar_init(gempty_bar(0, k), 1);
     }
-    mbar_init(drain_bar, 1);
-    for (int rs = 0; rs < kRaw; ++rs) {
-      mbar_init(rawfull_bar(rs), 1);
-      mbar_init(rawempty_bar(rs), kSlicers / 32);
+    for (int k = 0; k < 2; ++k) {
+      mbar_init(accfull_bar(k), 1);
+      mbar_init(accempty_bar(k), kEpiThreads);
+      mbar_init(drain_bar(k), 1);
     }
-    for (int st = 0; st < kStages; ++st) mbar_init(gfull_bar(st), 1);
     *s_abort = 0;
   }
   if (warp == kMmaWarp) {
@@ -398,269 +585,333 @@ __global__ void __launch_bounds__(kThreads, 1)
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
-  const uint32_t tmem = *tmem_slot;
+  const uint32_t tmem = uniform(*tmem_slot);
 
   if (warp < kSlicers / 32) {
     // ---------------------------------------------------------- slicers
-    // thread = (point p, functions 4q..4q+3 of the step); a warp takes 16
-    // points and one pair of q.  Each half warp holds points 0-7 of one q and
-    // points 8-15 of the other, so its 8-byte raw loads cover 128 distinct
-    // bytes and its 8-byte digit stores land in distinct banks of the two
-    // 8-row core matrices.
-    const int sub = (lane >> 3) & 1;
-    const int p = 16 * (warp >> 1) + 8 * (sub ^ (lane >> 4)) + (lane & 7), q = 2 * (warp & 1) + sub;
-    const int dst_off = (p >> 3) * kSBO + (q >> 1) * kLBO + (p & 7) * 16 + (q & 1) * 8;
-    bool ok = true;
-    int g = 0;  // steps of this CTA
-    for (int n = blockIdx.x; n < n_items; n += gridDim.x) {
-      const ItemInfo I = item_info(G, items[n]);
-      const bool live = I.pt * kTile + p < I.np;
-      const unsigned char* gblk = gsl + gsl_off[I.b];
-      const int n_steps = I.n_jt * n_prod * stages_per_product<KS>(I);
-      float m0 = 0.f, m1 = 0.f, m2 = 0.f, m3 = 0.f;  // rounding constants of the point's four quantities
-      StepIter<KS> it;
-      for (int s = 0; s < n_steps; ++s, ++g) {
-        const int rs = g % kRaw, st = g % kStages;
-        if (!mbar_wait_abort(rawfull_bar(rs), (g / kRaw) & 1, s_abort, status, G.wait_ns)) {
-          ok = false;
-          break;
+    const int r = warp * 32 + lane;  // point row
+    const uint32_t dst0 = smem0 + (r >> 3) * kSBO + (r & 7) * 16;
+    EntryWalk<MODE> W(items, n_items, present);
+    float2 x[kKc];
+    float mag = 0.f;
+    bool live = false;
+    int left = 0;  // functions from the chunk's first on
+    int item = -1;
+    float mPhi = 0.f, mGrad = 0.f;  // rounding constants of the walk's current item
+    // raw values of the walk's entry (zeros past the batch's functions and points)
+    auto load = [&]() {
+      const Item& I = W.I;
+      const int p = I.pt * kPts + r;
+      live = p < I.np;
+      if (item != W.n) {
+        item = W.n;
+        mPhi = mGrad = 0.f;
+        if (live) {
+          const int4 e = *reinterpret_cast<const int4*>(rowexp + 4 * (I.bp0 + p));
+          mPhi = magic0(e.x - kFine);
+          mGrad = magic0(max(e.y, max(e.z, e.w)) - kFine);
         }
-        const unsigned char* raw = smem + kSmemRaw + rs * kRawStage;
-        if (s == 0 && live) {
-          const int4 e = *reinterpret_cast<const int4*>(raw + kRawExp + p * 16);
-          m0 = magic0(e.x);
-          m1 = magic0(e.y);
-          m2 = magic0(e.z);
-          m3 = magic0(e.w);
+      }
+      const int q = W.q, f0 = W.c * kKc;
+      mag = q ? mGrad : mPhi;
+      // no load is conditional: functions past the batch's read the last one and
+      // are cleared below, points past n_p the row's end (their rows are dropped)
+      const float2* src = reinterpret_cast<const float2*>(scratch) + I.scr + q * I.plane + min(p, I.ldp - 1);
+      left = I.nb - f0;
+#pragma unroll
+      for (int k = 0; k < kKc; ++k) x[k] = ldg_stream(src + static_cast<int64_t>(min(f0 + k, I.nb - 1)) * I.ldp);
+    };
+    int slot = 0, ph = 1;
+    bool more = W.next();
+    if (more) load();
+    while (more) {
+      if (!mbar_wait_abort(slotempty_bar(slot), ph, s_abort, status, G.wait_ns)) break;
+      const uint32_t dst = dst0 + slot * kSlot;
+      const bool store = __any_sync(0xffffffffu, live);  // a warp with no point leaves its rows as they are
+      const float m = mag;
+      if (left < kKc) {
+#pragma unroll
+        for (int k = 0; k < kKc; ++k)
+          if (k >= left) x[k] = make_float2(0.f, 0.f);
+      }
+#pragma unroll
+      for (int h = 0; h < 2; ++h) {  // functions 8h .. 8h + 7: one 16-byte row piece per digit
+        uint32_t w[kSlices][4];
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+          float2 d[kSlices];
+          slice6x2(pk2(x[8 * h + 2 * u].x, x[8 * h + 2 * u + 1].x), pk2(x[8 * h + 2 * u].y, x[8 * h + 2 * u + 1].y),
+                   m, d);
+#pragma unroll
+          for (int t = 0; t < kSlices; ++t) w[t][u] = bf16x2_exact(d[t]);
         }
-        float2 x[KS][4];
+        if (store) {
 #pragma unroll
-        for (int h = 0; h < KS; ++h)
-#pragma unroll
-          for (int k = 0; k < 4; ++k)
-            x[h][k] = *reinterpret_cast<const float2*>(raw + h * kRawTile + (4 * q + k) * (kTile * 8) + p * 8);
-        if (!mbar_wait_abort(empty_bar(st), ((g / kStages) & 1) ^ 1, s_abort, status, G.wait_ns)) {
-          ok = false;
-          break;
-        }
-        const Product P = prod_at(it.kk);
-        unsigned char* sA = smem + kSmemStages + st * kStage;
-        if (tid == 0) {  // this stage's G' digits: one block (up to 12 KB) per K-step
-          const uint32_t bytes = kSlices * jt_width(I.nb, it.jt) * kRowBytes;  // the j-tile's six digit tiles
-          arrive_expect_tx(gfull_bar(st), KS * bytes);
-#pragma unroll
-          for (int h = 0; h < KS; ++h) {
-            // a K-step past the last chunk of functions (odd chunk counts,
-            // KS = 2) multiplies zeros: its F box is zero-filled and its G'
-            // block is the zero block
-            const int ic = it.chunk(h);
-            const unsigned char* src =
-                ic < I.n_ic ? gblk + (static_cast<int64_t>(P.gm) * I.n_jt * I.n_ic +
-                                      static_cast<int64_t>(it.jt) * I.n_ic + ic) * kBlockB
-                            : gzero;
-            bulk_copy(smem_u32(sA + h * kHalf + kStageA), src, bytes, gfull_bar(st));
-          }
-        }
-        const float m = P.qf == 0 ? m0 : P.qf == 1 ? m1 : P.qf == 2 ? m2 : m3;
-#pragma unroll
-        for (int h = 0; h < KS; ++h) {
-          // functions (4q, 4q+1) and (4q+2, 4q+3) of K-step h as packed pairs
-          float2 d01[kSlices], d23[kSlices];
-          slice6x2(pk2(x[h][0].x, x[h][1].x), pk2(x[h][0].y, x[h][1].y), m, d01);
-          slice6x2(pk2(x[h][2].x, x[h][3].x), pk2(x[h][2].y, x[h][3].y), m, d23);
-#pragma unroll
-          for (int t = 0; t < kSlices; ++t) {
-            asm volatile("st.shared.v2.b32 [%0], {%1, %2};" ::"r"(
-                             smem_u32(sA + h * kHalf + (1 + t) * kTileBytes + dst_off)),
-                         "r"(bf16x2_exact(d01[t])), "r"(bf16x2_exact(d23[t]))
+          for (int t = 0; t < kSlices; ++t)
+            asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(dst + t * kDigA + h * kLBO), "r"(w[t][0]),
+                         "r"(w[t][1]), "r"(w[t][2]), "r"(w[t][3])
                          : "memory");
-          }
-        }
-        fence_async_smem();
-        mbar_arrive(full_bar(st));
-        // Only now is the raw stage free: the digit stores above take their
-        // data from the loaded values, so once they have issued the loads
-        // have landed (freeing it right after issuing the loads let the next
-        // TMA box overwrite values that were still on their way).
-        __syncwarp();
-        if (lane == 0) mbar_arrive(rawempty_bar(rs));
-        it.next(I, n_prod);
-      }
-      // agree on stopping (a wait that gave up in one warp ends every role)
-      if (bar_red_or(1, kSlicers, !ok || *s_abort)) break;
-    }
-    // no G' copy outlives the CTA: thread 0 issued one per completed step;
-    // the last kStages of them may not have been consumed after an abort
-    if (tid == 0)
-      for (int h = max(0, g - kStages); h < g; ++h)
-        (void)mbar_wait(gfull_bar(h % kStages), (h / kStages) & 1, status);
-  } else if (warp == kProdWarp) {
-    // ---------------------------------------------------------- TMA producer
-    if (lane == 0) {
-      int g = 0;
-      bool ok = true;
-      for (int n = blockIdx.x; n < n_items && ok; n += gridDim.x) {
-        const ItemInfo I = item_info(G, items[n]);
-        const CUtensorMap* map = maps + I.b;
-        const int r0 = I.pt * kTile, rows = min(kTile, I.np - r0);
-        const int n_steps = I.n_jt * n_prod * stages_per_product<KS>(I);
-        StepIter<KS> it;
-        for (int s = 0; s < n_steps; ++s, ++g) {
-          const int rs = g % kRaw;
-          if (!mbar_wait_abort(rawempty_bar(rs), ((g / kRaw) & 1) ^ 1, s_abort, status, G.wait_ns, 32)) {
-            ok = false;
-            break;
-          }
-          const uint32_t dst = smem_u32(smem + kSmemRaw + rs * kRawStage), fb = rawfull_bar(rs);
-          arrive_expect_tx(fb, KS * kRawTile + (s == 0 ? rows * 16 : 0));
-#pragma unroll
-          for (int h = 0; h < KS; ++h)  // boxes past the last function read zeros
-            tma_load_3d(dst + h * kRawTile, map, r0, it.chunk(h) * kKc, prod_at(it.kk).qf, fb);
-          if (s == 0) bulk_copy(dst + kRawExp, rowexp + 4 * (I.bp0 + r0), rows * 16, fb);
-          it.next(I, n_prod);
         }
       }
-      // no copy outlives the CTA: the last kRaw issued steps have landed
-      for (int h = max(0, g - kRaw); h < g; ++h) (void)mbar_wait(rawfull_bar(h % kRaw), (h / kRaw) & 1, status);
+      fence_async_smem();
+      mbar_arrive(slotfull_bar(slot));
+      if (++slot == kSlots) {
+        slot = 0;
+        ph ^= 1;
+      }
+      // the next entry's loads fly while its slot is awaited
+      more = W.next();
+      if (more) load();
     }
-    __syncwarp();
-  } else if (warp == kMmaWarp) {
-    // ---------------------------------------------------------- MMA issue
-    if (lane == 0) {
-      int g = 0, k = 0;
-      bool ok = true;
-      for (int n = blockIdx.x; n < n_items && ok; n += gridDim.x) {
-        const ItemInfo I = item_info(G, items[n]);
-        int seg = 0, kk = 0, jt = 0;  // groups run (j-tile, product, segment) in order
-        for (int grp = 0; grp < I.n_jt * n_prod * I.n_seg && ok; ++grp, ++k) {
-          const int set = k & 1;
-          if (!mbar_wait_abort(accempty_bar(set), ((k >> 1) & 1) ^ 1, s_abort, status, G.wait_ns, 64)) {
-            ok = false;
-            break;
-          }
-          tc_fence_after();
-          const uint32_t t0 = tmem + set * kSetCols;
-          const int nbj = jt_width(I.nb, jt);
-          const int n_st = seg_stages(I.n_ic, seg, KS);
-          if (++seg == I.n_seg) {
-            seg = 0;
-            if (++kk == n_prod) {
-              kk = 0;
-              ++jt;
+  } else if (warp >= kProdWarp) {
+    // ---------------------------------------------------------- G' stream
+    // A block takes its thread a few hundred clocks of barrier round trips, so
+    // each ring has a producer of its own.
+    const int set = warp - kProdWarp;
+    int st = 0, ph = 1, k = 0, filled = 0;  // ring position and parity, groups, stages filled
+    bool ok = true;
+    GroupWalk<MODE> W(present);
+    const uint32_t ring = smem0 + L::kSmemRing + set * kStages * L::kStage;
+    for (int n = blockIdx.x; n < n_items && ok; n += gridDim.x) {
+      W.open(items + n);
+      // the next item's rows of F and R, fetched into L2 while this one runs:
+      // its first readers would each wait for DRAM (only where all CTAs'
+      // next items fit there beside the current ones)
+      if (n + gridDim.x < n_items) {
+        const Item N = item_of<MODE>(items + n + gridDim.x, present);
+        const int rows = (MODE == 0 ? 1 : 4) * N.nb;
+        if (N.nb <= 128) {
+          const int p0 = N.pt * kPts;
+          const uint32_t bytes = (min(kPts, N.ldp - p0) * 8);  // ldp is a multiple of 8: 64-byte pieces
+          const float2* src = reinterpret_cast<const float2*>(scratch) + N.scr + p0;
+          for (int f = 32 * set + lane; f < rows; f += 64)
+            prefetch_l2(src + static_cast<int64_t>(f) * N.ldp, bytes);
+        }
+      }
+      if (lane == 0) {
+        const unsigned char* gb = gsl + W.I.gsl;
+        for (; ok && W.next(); ++k) {
+          if ((k & 1) != set) continue;
+          const uint32_t blk = kSlices * kRowBytes * jt_width(W.I.nb, W.jt);
+          Run R = W.A;
+          for (int run = 0; run < 2 && ok; ++run, R = W.B) {
+            const unsigned char* src = gb + (static_cast<int64_t>(R.m) * W.I.n_jt + W.jt) * W.I.n_ic * kBlockB +
+                                       static_cast<int64_t>(R.c) * blk;
+            for (int c = 0; c < R.n; c += KS) {
+              if (!mbar_wait_abort(gempty_bar(set, st), ph, s_abort, status, G.wait_ns)) {
+                ok = false;
+                break;
+              }
+              const uint32_t bytes = min(KS, R.n - c) * blk;
+              arrive_expect_tx(gfull_bar(set, st), bytes);
+              bulk_copy(ring + st * L::kStage, src, bytes, gfull_bar(set, st));
+              src += bytes;
+              ++filled;
+              if (++st == kStages) {
+                st = 0;
+                ph ^= 1;
+              }
             }
           }
-          for (int c = 0; c < n_st; ++c, ++g) {
-            const int st = g % kStages;
-            if (!mbar_wait_abort(full_bar(st), (g / kStages) & 1, s_abort, status, G.wait_ns, 32) ||
-                !mbar_wait_abort(gfull_bar(st), (g / kStages) & 1, s_abort, status, G.wait_ns, 32)) {
+        }
+      }
+      ok = __shfl_sync(0xffffffffu, ok, 0);
+    }
+    // no copy outlives the CTA: the last kStages issued ones have landed
+    if (lane == 0)
+      for (int h = max(0, filled - kStages); h < filled; ++h)
+        (void)mbar_wait(gfull_bar(set, h % kStages), (h / kStages) & 1, status);
+    __syncwarp();
+  } else if (warp == kMmaWarp || warp == kMmaWarp + 1) {
+    // ---------------------------------------------------------- MMA issue
+    // The whole warp walks and waits; one lane issues.  Operands of
+    // tcgen05.mma are uniform registers: from values the compiler knows to be
+    // the same in every lane an instruction issues in a few clocks, from a
+    // single-lane loop each took about 200.  The tensor unit queues only a few
+    // instructions, so what a warp does between its steps leaves it idle: two
+    // warps issue, each the groups of one accumulator set, and one's
+    // bookkeeping runs under the other's products.
+    //
+    // A wait by parity is only sound for a warp that has seen the barrier's
+    // previous phase: each set has a ring of G' blocks of its own, and each
+    // warp waits for every entry in order, also for those whose groups it
+    // leaves to the other, before it gives the slot back.
+    const int set = uniform(warp - kMmaWarp);
+    int st = 0, ph = 0, k = 0, known = 0;  // ring position and parity, groups, entries seen in place
+    bool ok = true;
+    GroupWalk<MODE> W(present);
+    const uint64_t descA = make_desc(smem0, kSBO);
+    const uint64_t descB = make_desc(smem0 + L::kSmemRing + set * kStages * L::kStage, kSBO);
+    const uint32_t t0 = uniform(tmem + set * kSetCols);
+    auto see = [&](int e) {  // every entry up to e is in place
+      for (; known <= e; ++known)
+        if (!mbar_wait_abort(slotfull_bar(known % kSlots), (known / kSlots) & 1, s_abort, status, G.wait_ns))
+          return false;
+      return true;
+    };
+    for (int n = blockIdx.x; n < n_items && ok; n += gridDim.x) {
+      W.open(items + n);
+      for (; ok && W.next(); ++k) {
+        if ((k & 1) != set) {  // the other warp's group
+          if (W.last) {  // this warp is through with the segment's slots
+            ok = see(W.ent + W.S.n - 1);
+            if (ok && elect_one())
+              for (int e = W.ent; e < W.ent + W.S.n; ++e) mma_commit(slotempty_bar(e % kSlots));
+          }
+          continue;
+        }
+        if (!mbar_wait_abort(accempty_bar(set), ((k >> 1) & 1) ^ 1, s_abort, status, G.wait_ns)) {
+          ok = false;
+          break;
+        }
+        tc_fence_after();
+        // every entry the group reads (the last one is in its last run)
+        if (!see(W.ent + (W.B.n ? max(W.A.ent + W.A.n, W.B.ent + W.B.n) : W.A.ent + W.A.n) - 1)) {
+          ok = false;
+          break;
+        }
+        tc_fence_after();
+        const int w = uniform(jt_width(W.I.nb, W.jt));
+        const bool release = W.last && W.S.kind != kGrad;  // the last group reads every chunk of its segment in order
+        bool first = true;
+        Run R = W.A;
+        for (int run = 0; run < 2 && ok; ++run, R = W.B)
+          for (int c = 0; c < R.n && ok; c += KS) {
+            if (!mbar_wait_abort(gfull_bar(set, st), ph, s_abort, status, G.wait_ns)) {
               ok = false;
               break;
             }
             tc_fence_after();
 #pragma unroll
             for (int h = 0; h < KS; ++h) {
-              const uint32_t a = smem_u32(smem + kSmemStages + st * kStage + h * kHalf), bb = a + kStageA;
-              mma_levels(t0, a, bb, (c == 0 && h == 0) ? 0u : 1u, nbj);
+              if (c + h >= R.n) break;
+              const int slot = uniform((W.ent + R.ent + c + h) % kSlots);
+              const uint64_t a = descA + static_cast<uint32_t>(slot * (kSlot >> 4));
+              const uint64_t bd = descB + static_cast<uint32_t>((st * L::kStage + h * kSlices * kRowBytes * w) >> 4);
+              if (elect_one()) {
+                mma_row_levels(t0, a, bd, w, first);
+                if (release) mma_commit(slotempty_bar(slot));
+              }
+              first = false;
             }
-            mma_commit(empty_bar(st));
+            if (ok && elect_one()) mma_commit(gempty_bar(set, st));
+            if (++st == kStages) {
+              st = 0;
+              ph ^= 1;
+            }
           }
-          if (ok) mma_commit(accfull_bar(set));
+        if (ok && W.last && !release) ok = see(W.ent + W.S.n - 1);
+        if (!ok) break;
+        if (elect_one()) {
+          mma_commit(accfull_bar(set));
+          if (W.last && !release)
+            for (int e = W.ent; e < W.ent + W.S.n; ++e) mma_commit(slotempty_bar(e % kSlots));
         }
       }
-      // every MMA issued by this thread has completed before tensor memory is freed
-      mma_commit(drain_bar);
-      (void)mbar_wait(drain_bar, 0, status);
+    }
+    // every MMA issued by this warp has completed before tensor memory is freed
+    if (elect_one()) {
+      mma_commit(drain_bar(set));
+      (void)mbar_wait(drain_bar(set), 0, status);
     }
     __syncwarp();
   } else {
     // ---------------------------------------------------------- epilogue
-    // Thread = one TMEM lane: lanes 0-63 hold levels 0, 2, 4 and lanes 64-127
-    // levels 1, 3, 5 of the same 64 points.  The dot with R is linear in the
-    // levels, so each lane keeps its own double-float partial sum; the two
-    // halves and the two column groups meet once per item.
-    const int eg = (warp - kEpiWarp0) >> 2;  // column group: 8-column chunks eg, eg + 2, ...
-    const int quarter = warp & 3;            // TMEM lanes 32 quarter .. +31
-    const int r = (quarter & 1) * 32 + lane, lvl = quarter >> 1;
+    // Thread = one point; column group eg takes half of the group's columns
+    const int eg = (warp - kEpiWarp0) >> 2;
+    const int quarter = warp & 3;  // TMEM lanes 32 quarter .. +31
+    const int r = quarter * 32 + lane;
     const uint32_t lane_base = static_cast<uint32_t>(quarter * 32) << 16;
     int k = 0;
     bool ok = true;
-    for (int n = blockIdx.x; n < n_items && ok; n += gridDim.x) {
-      const ItemInfo I = item_info(G, items[n]);
-      const float2* base = reinterpret_cast<const float2*>(scratch) + scr_off[I.b];
-      const int p = I.pt * kTile + r;
+    GroupWalk<MODE> W(present);
+    for (int n = blockIdx.x; n < n_items; n += gridDim.x) {
+      W.open(items + n);
+      const Item& I = W.I;
+      const float2* base = reinterpret_cast<const float2*>(scratch) + I.scr;
+      const int p = I.pt * kPts + r;
       const bool live = p < I.np;
+      const bool busy = I.pt * kPts + quarter * 32 < I.np;  // some point of this warp exists
       df y = {0.f, 0.f};  // running sum over the item's groups
-      int seg = 0, kk = 0, jt = 0;
-      for (int grp = 0; grp < I.n_jt * n_prod * I.n_seg; ++grp, ++k) {
-        const int set = k & 1;
-        const int j0 = jt * kTile;
-        const Product P = prod_at(kk);
-        const int N = jt_width(I.nb, jt);  // accumulator blocks are N columns wide
-        const float2* Rrow = base + P.qr * I.plane + p;
-        // R of this thread's point, 8 columns per chunk; the first chunk's
-        // values load while the MMAs finish, later ones one chunk ahead
-        auto load_R = [&](int c0, float2* R) {
+      // R of this thread's point and its 16 columns (8 in a 16-wide tile) of the
+      // walk's group.  Columns past the batch's functions read the last one (their
+      // U is zero), points past n_p the row's end (their result is dropped): no
+      // load is conditional, so that all are in flight at once.
+      const float2* mine = base + min(p, I.ldp - 1);
+      auto load_R = [&](float2* R) {
+        const int w = jt_width(I.nb, W.jt), j0 = W.jt * kTileJ + eg * (w >> 1);
+        const float2* plane = mine + W.qr * I.plane;
 #pragma unroll
-          for (int i = 0; i < 8; ++i) {
-            const int j = j0 + c0 + i;
-            R[i] = (live && j < I.nb) ? __ldg(Rrow + static_cast<int64_t>(j) * I.ldp) : make_float2(0.f, 0.f);
-          }
-        };
-        float2 Rc[8], Rn[8];
-        if (eg * 8 < N) load_R(eg * 8, Rc);
-        ok = mbar_wait_abort(accfull_bar(set), (k >> 1) & 1, s_abort, status, G.wait_ns, 256);
-        if (bar_red_or(2, kEpiThreads, !ok)) {
+        for (int i = 0; i < 8; ++i) R[i] = ldg_stream(plane + static_cast<int64_t>(min(j0 + i, I.nb - 1)) * I.ldp);
+        if (w > 16) {
+#pragma unroll
+          for (int i = 8; i < 16; ++i) R[i] = ldg_stream(plane + static_cast<int64_t>(min(j0 + i, I.nb - 1)) * I.ldp);
+        }
+      };
+      // values load one group ahead, across the item's groups
+      float2 Rc[16], Rn[16];
+      bool have = W.next();
+      if (have && busy) load_R(Rc);
+      while (have) {
+        const int set = k & 1, w = jt_width(I.nb, W.jt);
+        have = W.next();
+        if (have && busy) load_R(Rn);
+        ok = mbar_wait_abort(accfull_bar(set), (k >> 1) & 1, s_abort, status, G.wait_ns);
+        if (!__all_sync(0xffffffffu, ok)) {
           ok = false;
           break;
         }
         tc_fence_after();
-        // this group's sum yh + yl: per column u = v0 + v1 + v2 (top lanes
-        // L0 + L2 + L4 with L0, L2 exact; bottom lanes L1 + L3 + L5) as the
-        // exact two-sum of v0, v1 with v2 (2^-16 and further below) folded
-        // into its error; the product with R = (rh, rl) keeps its FMA error
+        // this group's sum yh + yl, even and odd columns apart (packed
+        // instructions: the issue slots are shared with the slicers): per column
+        // u = two-sums of the exact levels 0-2, the rounded levels and the errors
+        // as its low part; the product with R = (rh, rl) keeps its FMA error
         // term unnormalised, and the sum adds each product by a two-sum whose
-        // error joins yl (all terms about 2^-24 below yh and beyond)
-        float yh = 0.f, yl = 0.f;
-        for (int c0 = eg * 8; c0 < N; c0 += 16) {
-          if (c0 + 16 < N) load_R(c0 + 16, Rn);
-          float v0[8], v1[8], v2[8];
-          const uint32_t ta = tmem + lane_base + set * kSetCols + c0;
-          tmem_ld8x3(ta, ta + N, ta + 2 * N, v0, v1, v2);
+        // error joins yl
+        float2 yh = {0.f, 0.f}, yl = {0.f, 0.f};
+        if (busy) {
+          const uint32_t t = tmem + lane_base + set * kSetCols + eg * (w >> 1);
 #pragma unroll
-          for (int i = 0; i < 8; ++i) {
-            const df u = two_sum(v0[i], v1[i]);
-            const float ul = __fadd_rn(u.lo, v2[i]);
-            const float rh = Rc[i].x, rl = Rc[i].y;
-            const float ph = __fmul_rn(rh, u.hi);
-            float pl = __fmaf_rn(rh, u.hi, -ph);
-            pl = __fmaf_rn(rh, ul, pl);
-            pl = __fmaf_rn(rl, u.hi, pl);
-            const df a = two_sum(yh, ph);
-            yh = a.hi;
-            yl = __fadd_rn(yl, __fadd_rn(a.lo, pl));
+          for (int c = 0; c < 16; c += 8) {
+            if (c && w <= 16) break;
+            float v[6][8];
+            tmem_ld8x6(t + c, w, v);
+#pragma unroll
+            for (int i = 0; i < 8; i += 2) {
+              float2 s, es, u, eu, a, ea;
+              two_sum2(pk2(v[0][i], v[0][i + 1]), pk2(v[1][i], v[1][i + 1]), s, es);
+              two_sum2(s, pk2(v[2][i], v[2][i + 1]), u, eu);
+              const float2 ul = add2(add2(es, eu), add2(pk2(v[3][i], v[3][i + 1]),
+                                                        add2(pk2(v[4][i], v[4][i + 1]), pk2(v[5][i], v[5][i + 1]))));
+              const float2 rh = pk2(Rc[c + i].x, Rc[c + i + 1].x), rl = pk2(Rc[c + i].y, Rc[c + i + 1].y);
+              const float2 ph = mul2(rh, u);
+              float2 pl = fma2(rh, u, pk2(-ph.x, -ph.y));
+              pl = fma2(rh, ul, pl);
+              pl = fma2(rl, u, pl);
+              two_sum2(yh, ph, a, ea);
+              yh = a;
+              yl = add2(yl, add2(ea, pl));
+            }
           }
-#pragma unroll
-          for (int i = 0; i < 8; ++i) Rc[i] = Rn[i];
         }
         tc_fence_before();
         mbar_arrive(accempty_bar(set));
-        y = df_add(y, df{P.factor * yh, P.factor * yl});  // factor 1 or 2: exact
-        if (++seg == I.n_seg) {
-          seg = 0;
-          if (++kk == n_prod) {
-            kk = 0;
-            ++jt;
-          }
-        }
+        ++k;
+        y = df_add(y, df_add(df{yh.x, yl.x}, df{yh.y, yl.y}));
+#pragma unroll
+        for (int i = 0; i < 16; ++i) Rc[i] = Rn[i];
       }
-      if (!ok) break;
-      // the four partial sums of each point (two level halves x two column groups)
-      sY[(eg * 2 + lvl) * kTile + r] = static_cast<double>(y.hi) + static_cast<double>(y.lo);
-      bar_sync(2, kEpiThreads);
-      if (eg == 0 && lvl == 0 && live) {
-        const double val = (sY[r] + sY[kTile + r]) + (sY[2 * kTile + r] + sY[3 * kTile + r]);
+      // the two column halves of each point (a warp that gave up ends them all)
+      sY[eg * kPts + r] = static_cast<double>(y.hi) + static_cast<double>(y.lo);
+      if (bar_red_or(2, kEpiThreads, !ok)) break;
+      if (eg == 0 && live) {
+        const double val = sY[r] + sY[kPts + r];
         const int64_t gp = I.bp0 + p;
-        out[gp] = weighted ? G.w[gp] * val : val;
+        const double res = weighted ? G.w[gp] * val : val;
+        if (I.jt1 - I.jt0 == I.n_jt)
+          out[gp] = res;
+        else
+          atomicAdd(out + gp, res);  // shares of one batch (zeroed before the first wave)
       }
       bar_sync(2, kEpiThreads);
     }
@@ -671,47 +922,43 @@ __global__ void __launch_bounds__(kThreads, 1)
     asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(kTmemCols));
 }
 
-// FP32-pair copies of the present matrices into slots [slot0, slot0 + 5) of
-// the grid's buffer (of the antisymmetric parts of matrices 2-4, the SO
-// slots), with their per-block column and row maxima; returns the mask of
-// present matrices
-q4c_status prepare(const q4c_grid* g, const double* const mats[5], int slot0, const float2* mdf[5],
-                   unsigned* present, cudaStream_t s) {
+// the prepared matrices of one call: FP32-pair copies in slots [slot, slot + 5)
+// of the grid's buffer and two column bounds per block; slot 0 for the density,
+// 5 for the adjoint.  Returns the mask of present matrices.
+q4c_status prepare(const q4c_grid* g, const double* const mats[5], int slot, unsigned* present, cudaStream_t s) {
   int dev = 0, n_sm = 0;
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&n_sm, cudaDevAttrMultiProcessorCount, dev);
   *present = 0;
-  KernelScope ks("split_gslice", s);
+  if (g->nnz == 0) return Q4C_OK;
+  Mats M;
   for (int m = 0; m < 5; ++m) {
-    mdf[m] = nullptr;
-    if (!mats[m] || g->nnz == 0) continue;
-    float2* dst = g->d_gdf + (slot0 + m) * g->nnz;
-    const unsigned nblk = static_cast<unsigned>(std::min<int64_t>(g->n_blocks, 64 * n_sm));
-    k_prepare_blocks<<<nblk, 128, 0, s>>>(g->tables->view(), g->view(), mats[m], m >= 2 ? 1 : 0, g->n_blocks,
-                                          g->d_blk_row, g->d_blk_col, g->d_blk_off, g->d_blk_T, g->d_cm_off, dst,
-                                          g->d_cm + (slot0 + m) * g->cm_total);
-    mdf[m] = dst;
-    *present |= 1u << m;
+    M.m[m] = mats[m];
+    if (mats[m]) *present |= 1u << m;
   }
+  const size_t smem = sizeof(unsigned) * 2 * *std::max_element(g->tables->nfn.begin(), g->tables->nfn.end());
+  if (smem > 12 * 1024)
+    Q4C_CUDA(cudaFuncSetAttribute(k_prepare_blocks, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem)));
+  KernelScope ks("split_gslice", s);
+  const unsigned nblk = static_cast<unsigned>(std::min<int64_t>(g->n_blocks, 64 * n_sm));
+  k_prepare_blocks<<<nblk, 128, smem, s>>>(g->tables->view(), g->view(), M, g->n_blocks, g->d_blk_row, g->d_blk_col,
+                                           g->d_blk_off, g->d_blk_T, g->d_cm_off, g->d_gdf + slot * g->nnz, g->nnz,
+                                           g->d_cm + (slot ? 2 : 0) * g->cm_total, g->cm_total);
   Q4C_CUDA(cudaGetLastError());
   return Q4C_OK;
 }
 
-// one wave [b0, b1) of the density (MODE 0) or adjoint (MODE 1): G' digit
-// blocks and the row-dot kernel with KS K-steps per stage; the wave's offset
-// tables and basis tiles (with per-point exponents) must already be in place
+// G' digit blocks of one wave [b0, b1); the wave's offset tables must be in place
 template <int MODE>
-q4c_status gslice_wave(const q4c_grid* g, int wv, const float2* const mdf[5], cudaStream_t s) {
+q4c_status gslice_wave(const q4c_grid* g, int wv, int slot, unsigned present, cudaStream_t s) {
   const int64_t b0 = g->wave_b0[wv], b1 = g->wave_b0[wv + 1];
   if (b1 <= b0) return Q4C_OK;
-  // each matrix's block maxima sit in the slot of its FP32-pair copy
-  const float* cmp[5];
-  for (int m = 0; m < 5; ++m)
-    cmp[m] = mdf[m] ? g->d_cm + ((mdf[m] - g->d_gdf) / std::max<int64_t>(g->nnz, 1)) * g->cm_total : nullptr;
+  // four j-tiles a CTA: the batches of a wave differ widely in n_b
+  const unsigned z = static_cast<unsigned>(std::max(1, (g->max_nb + 4 * kTileJ - 1) / (4 * kTileJ)));
   KernelScope ks("split_gslice", s);
-  k_gslice<<<dim3(static_cast<unsigned>(b1 - b0), MODE == 0 ? 1 : 5), 256, 0, s>>>(
-      g->view(), b0, mdf[0], mdf[1], mdf[2], mdf[3], mdf[4], cmp[0], cmp[1], cmp[2], cmp[3],
-      cmp[4], g->d_pair_blk, g->d_cm_off, g->d_gsl_off, reinterpret_cast<uint32_t*>(g->d_gsl));
+  k_gslice<<<dim3(static_cast<unsigned>(b1 - b0), MODE == 0 ? 1 : 5, z), 256, 0, s>>>(
+      g->view(), b0, g->d_gdf + slot * g->nnz, g->nnz, present, g->d_cm + (slot ? 2 : 0) * g->cm_total, g->cm_total,
+      g->d_pair_blk, g->d_cm_off, g->d_gsl_off, reinterpret_cast<uint32_t*>(g->d_gsl));
   Q4C_CUDA(cudaGetLastError());
   return Q4C_OK;
 }
@@ -732,9 +979,8 @@ q4c_status rowdot_kernel(const q4c_grid* g, int wv, unsigned present, bool weigh
   {
     KernelScope ks(name, s);
     k_split_rowdot<MODE, KS><<<grid, kThreads, Layout<KS>::kSmemTotal, s>>>(
-        g->view(), g->d_rd_items + i0, n_items, reinterpret_cast<const CUtensorMap*>(g->d_tmaps) + g->n_batches,
-        g->d_scr_off, g->d_scratch, g->d_rowexp, g->d_gsl_off, reinterpret_cast<const unsigned char*>(g->d_gsl),
-        g->d_gzero, present, weighted ? 1 : 0, out, g->d_status);
+        g->view(), g->d_rd_items + i0, n_items, g->d_scratch, g->d_rowexp,
+        reinterpret_cast<const unsigned char*>(g->d_gsl), present, weighted ? 1 : 0, out, g->d_status);
   }
   Q4C_CUDA(cudaGetLastError());
   return Q4C_OK;
@@ -748,10 +994,9 @@ q4c_status kernel_ks(const q4c_grid* g, int wv, unsigned present, bool weighted,
 }
 
 template <int MODE>
-q4c_status wave(const q4c_grid* g, int wv, const float2* const mdf[5], unsigned present, bool weighted,
-                double* out, cudaStream_t s) {
+q4c_status wave(const q4c_grid* g, int wv, int slot, unsigned present, bool weighted, double* out, cudaStream_t s) {
   if (g->wave_b0[wv + 1] <= g->wave_b0[wv]) return Q4C_OK;
-  if (q4c_status st = gslice_wave<MODE>(g, wv, mdf, s)) return st;
+  if (q4c_status st = gslice_wave<MODE>(g, wv, slot, present, s)) return st;
   return kernel_ks<MODE>(g, wv, present, weighted, out, s, g->rd_ks, MODE == 0 ? "split_density" : "split_backward");
 }
 
@@ -762,31 +1007,31 @@ q4c_status run(const q4c_tables* t, const q4c_grid* g, const double* const mats[
     set_error("the split density/adjoint need at most 4096 active functions per batch");
     return Q4C_EUNSUPPORTED;
   }
-  const float2* mdf[5];
   unsigned present = 0;
-  if (q4c_status st = prepare(g, mats, 0, mdf, &present, s)) return st;
+  if (q4c_status st = prepare(g, mats, 0, &present, s)) return st;
+  if (g->rd_shares) Q4C_CUDA(cudaMemsetAsync(out, 0, sizeof(double) * g->n_pts, s));
   const int n_waves = static_cast<int>(g->wave_b0.size()) - 1;
   for (int wv = 0; wv < n_waves; ++wv) {
     const int64_t b0 = g->wave_b0[wv], b1 = g->wave_b0[wv + 1];
     if (b1 <= b0) continue;
     if (q4c_status st = launch_fill_idx(t, g, b0, b1, s)) return st;
     if (q4c_status st = launch_basis_df(t, g, b0, b1, nullptr, nullptr, g->d_rowexp, MODE == 0 ? 1 : 4, s)) return st;
-    if (q4c_status st = wave<MODE>(g, wv, mdf, present, weighted, out, s)) return st;
+    if (q4c_status st = wave<MODE>(g, wv, 0, present, weighted, out, s)) return st;
   }
   return Q4C_OK;
 }
 
 }  // namespace rowdot
 
-q4c_status rowdot_prepare(const q4c_grid* g, const double* const mats[5], int slot0, const float2* mdf[5],
-                          unsigned* present, cudaStream_t s) {
-  return rowdot::prepare(g, mats, slot0, mdf, present, s);
+q4c_status rowdot_prepare(const q4c_grid* g, const double* const mats[5], int slot, unsigned* present,
+                          cudaStream_t s) {
+  return rowdot::prepare(g, mats, slot, present, s);
 }
 
-q4c_status rowdot_wave(const q4c_grid* g, int wv, int mode, const float2* const mdf[5], unsigned present,
-                       bool weighted, double* out, cudaStream_t s) {
-  return mode == 0 ? rowdot::wave<0>(g, wv, mdf, present, weighted, out, s)
-                   : rowdot::wave<1>(g, wv, mdf, present, weighted, out, s);
+q4c_status rowdot_wave(const q4c_grid* g, int wv, int mode, int slot, unsigned present, bool weighted, double* out,
+                       cudaStream_t s) {
+  return mode == 0 ? rowdot::wave<0>(g, wv, slot, present, weighted, out, s)
+                   : rowdot::wave<1>(g, wv, slot, present, weighted, out, s);
 }
 
 // the tuner's part for the row-dot kernel: the adjoint kernel of wave 0 with
@@ -799,11 +1044,9 @@ q4c_status autotune_rowdot(q4c_grid* g, double* out, cudaStream_t s) {
   g->rd_tune_ms[0] = g->rd_tune_ms[1] = -1.0;
   if (g->wave_b0.size() < 2 || g->max_nb > rowdot::kMaxNb || g->nnz == 0) return Q4C_OK;
   if (g->wave_b0[1] <= g->wave_b0[0]) return Q4C_OK;
-  const float2* mdf[5];
-  for (int m = 0; m < 5; ++m) mdf[m] = g->d_gdf + (5 + m) * g->nnz;
   Q4C_CUDA(cudaMemsetAsync(g->d_gdf + 5 * g->nnz, 0, sizeof(float2) * 5 * g->nnz, s));
-  Q4C_CUDA(cudaMemsetAsync(g->d_cm + 5 * g->cm_total, 0, sizeof(float) * 5 * g->cm_total, s));
-  if (q4c_status st = rowdot::gslice_wave<1>(g, 0, mdf, s)) return st;
+  Q4C_CUDA(cudaMemsetAsync(g->d_cm + 2 * g->cm_total, 0, sizeof(float) * 2 * g->cm_total, s));
+  if (q4c_status st = rowdot::gslice_wave<1>(g, 0, 5, 31u, s)) return st;
   cudaEvent_t ev[2][3][2] = {};
   q4c_status status = Q4C_OK;
   for (int k = 0; k < 2; ++k)

@@ -223,7 +223,7 @@ __global__ void __launch_bounds__(kThreads, 1)
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(smem + kSmemBar + kNumBars * 8);
   volatile int* s_abort = reinterpret_cast<volatile int*>(smem + kSmemBar + kNumBars * 8 + 4);
 
-  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int tid = threadIdx.x, warp = uniform(tid >> 5), lane = tid & 31;
   if (smem_u32(smem) & 1023u) {  // the swizzled TMA boxes need 1024-byte aligned stages
     if (tid == 0) atomicOr(status, 2u);
     return;
@@ -268,7 +268,7 @@ __global__ void __launch_bounds__(kThreads, 1)
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
-  const uint32_t tmem = *tmem_slot;
+  const uint32_t tmem = uniform(*tmem_slot);
 
   if (warp < kSlicers / 32) {
     // ---------------------------------------------------------- slicers
@@ -375,7 +375,7 @@ __global__ void __launch_bounds__(kThreads, 1)
         bool ok = true;
         for (int s = 0; s < n_steps; ++s, ++g) {
           const int rs = g % kRaw;
-          if (!mbar_wait_abort(rawempty_bar(rs), ((g / kRaw) & 1) ^ 1, s_abort, status, G.wait_ns, 32)) {
+          if (!mbar_wait_abort(rawempty_bar(rs), ((g / kRaw) & 1) ^ 1, s_abort, status, G.wait_ns)) {
             ok = false;
             break;
           }
@@ -401,35 +401,39 @@ __global__ void __launch_bounds__(kThreads, 1)
     __syncwarp();
   } else if (warp == kMmaWarp) {
     // ---------------------------------------------------------- MMA issue
-    if (lane == 0) {
-      int g = 0, k = 0;
-      for (int n = blockIdx.x; n < n_items; n += gridDim.x, ++k) {
-        const int4 item = items[n];
-        const int n_steps = item_stages(item);
-        const int nbB = item_nb(static_cast<int>(G.bat_fn_ptr[item.x + 1] - G.bat_fn_ptr[item.x]), item.w);
-        const int set = k & 1;
-        if (!mbar_wait_abort(accempty_bar(set), ((k >> 1) & 1) ^ 1, s_abort, status, G.wait_ns, 64)) break;
+    // (the whole warp waits, one lane issues, operands uniform: see rowdot.cu)
+    const bool lead = elect_one();
+    const uint32_t smem_st = smem_u32(smem + kSmemStages);
+    int g = 0, k = 0;
+    bool ok = true;
+    for (int n = blockIdx.x; n < n_items && ok; n += gridDim.x, ++k) {
+      const int4 item = items[n];
+      const int n_steps = uniform(item_stages(item));
+      const int nbB = uniform(item_nb(static_cast<int>(G.bat_fn_ptr[item.x + 1] - G.bat_fn_ptr[item.x]), item.w));
+      const int set = k & 1;
+      if (!mbar_wait_abort(accempty_bar(set), ((k >> 1) & 1) ^ 1, s_abort, status, G.wait_ns)) break;
+      tc_fence_after();
+      const uint32_t t0 = uniform(tmem + set * kSetCols);
+      for (int s = 0; s < n_steps; ++s, ++g) {
+        const int st = uniform(g % kStages);
+        if (!mbar_wait_abort(full_bar(st), (g / kStages) & 1, s_abort, status, G.wait_ns)) {
+          ok = false;
+          break;
+        }
         tc_fence_after();
-        const uint32_t t0 = tmem + set * kSetCols;
-        bool ok = true;
-        for (int s = 0; s < n_steps; ++s, ++g) {
-          const int st = g % kStages;
-          if (!mbar_wait_abort(full_bar(st), (g / kStages) & 1, s_abort, status, G.wait_ns, 32)) {
-            ok = false;
-            break;
-          }
-          tc_fence_after();
+        if (lead) {
 #pragma unroll
           for (int h = 0; h < KS; ++h) {
-            const uint32_t a = smem_u32(smem + kSmemStages + st * kStage + h * kHalf), bb = a + kStageA;
+            const uint32_t a = smem_st + st * kStage + h * kHalf, bb = a + kStageA;
             mma_levels(t0, a, bb, (s == 0 && h == 0) ? 0u : 1u, nbB);
           }
           mma_commit(empty_bar(st));
         }
-        if (!ok) break;
-        mma_commit(accfull_bar(set));
       }
-      // every MMA issued by this thread has completed before tensor memory is freed
+      if (ok && lead) mma_commit(accfull_bar(set));
+    }
+    // every MMA issued by this warp has completed before tensor memory is freed
+    if (lead) {
       mma_commit(drain_bar);
       (void)mbar_wait(drain_bar, 0, status);
     }
@@ -443,7 +447,7 @@ __global__ void __launch_bounds__(kThreads, 1)
     int k = 0;
     for (int n = blockIdx.x; n < n_items; n += gridDim.x, ++k) {
       const int set = k & 1;
-      bool ok = mbar_wait_abort(accfull_bar(set), (k >> 1) & 1, s_abort, status, G.wait_ns, 256);
+      bool ok = mbar_wait_abort(accfull_bar(set), (k >> 1) & 1, s_abort, status, G.wait_ns);
       if (bar_red_or(2, kEpiThreads, !ok)) break;
       tc_fence_after();
       const int4 item = items[n];

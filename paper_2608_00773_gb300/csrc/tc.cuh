@@ -35,6 +35,18 @@ __device__ __forceinline__ uint32_t make_idesc(int M, int N) {
          (static_cast<uint32_t>(M >> 4) << 24);
 }
 
+// lane 0's value in every lane (a value the compiler then holds in a uniform
+// register, as the operands of tcgen05.mma are)
+__device__ __forceinline__ int uniform(int x) { return __shfl_sync(0xffffffffu, x, 0); }
+__device__ __forceinline__ uint32_t uniform(uint32_t x) { return __shfl_sync(0xffffffffu, x, 0); }
+
+// true in one lane of the (converged) warp, always the same one
+__device__ __forceinline__ bool elect_one() {
+  uint32_t p;
+  asm volatile("{\n\t.reg .pred P;\n\telect.sync _|P, 0xffffffff;\n\tselp.u32 %0, 1, 0, P;\n\t}\n" : "=r"(p));
+  return p != 0;
+}
+
 __device__ __forceinline__ void mma_bf16(uint32_t tmem_d, uint64_t adesc, uint64_t bdesc, uint32_t idesc,
                                          uint32_t accumulate) {
   asm volatile(
@@ -123,18 +135,24 @@ __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, unsigne
 // bounded wait of a working role (limit_ns of wall clock, the grid's work
 // wait limit) that also gives up as soon as another role of the CTA has set
 // *abort (a role that times out sets it and the status bit); the drain waits
-// before a CTA exits keep the fixed 1 s limit of mbar_wait
-// (sleep_ns > 0: back off between polls, for roles whose waits are long and
-// whose polling would take issue slots from the working warps)
+// before a CTA exits keep the fixed 1 s limit of mbar_wait.  try_wait suspends
+// the thread in hardware, so polling takes few issue slots; the clock is read
+// on every 32nd poll only (each read costs hundreds of clocks, which a
+// handshake between roles would wait for), unless the limit is so short that
+// every poll has to look.
 __device__ __forceinline__ bool mbar_wait_abort(uint32_t bar, uint32_t parity, volatile int* abort,
-                                                unsigned* status, uint64_t limit_ns, unsigned sleep_ns = 0) {
+                                                unsigned* status, uint64_t limit_ns) {
   if (mbar_try_wait(bar, parity)) return true;
-  const uint64_t t0 = global_ns();
-  while (true) {
-    if (sleep_ns) __nanosleep(sleep_ns);
+  const unsigned mask = limit_ns < 1000000ull ? 0u : 31u;
+  uint64_t t0 = mask ? 0 : global_ns();
+  for (unsigned i = 1;; ++i) {
     if (mbar_try_wait(bar, parity)) return true;
     if (*abort) return false;
-    if (global_ns() - t0 > limit_ns) {
+    if (i & mask) continue;
+    const uint64_t t = global_ns();
+    if (!t0) {
+      t0 = t;
+    } else if (t - t0 > limit_ns) {
       *abort = 1;
       atomicOr(status, 1u);
       return false;
@@ -175,6 +193,18 @@ __device__ __forceinline__ void bulk_copy(uint32_t dst, const void* src, uint32_
       "cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(dst),
       "l"(src), "r"(bytes), "r"(bar)
       : "memory");
+}
+
+// one 8-byte read that leaves L1 to the shared memory it is carved from
+__device__ __forceinline__ float2 ldg_stream(const float2* p) {
+  float2 v;
+  asm volatile("ld.global.nc.L1::no_allocate.v2.f32 {%0, %1}, [%2];" : "=f"(v.x), "=f"(v.y) : "l"(p));
+  return v;
+}
+
+// starts fetching `bytes` (a multiple of 16) at a 16-byte aligned address into L2
+__device__ __forceinline__ void prefetch_l2(const void* p, uint32_t bytes) {
+  asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(p), "r"(bytes) : "memory");
 }
 
 // arrive on the mbarrier and add `bytes` to the transactions its phase waits for
@@ -281,6 +311,13 @@ __device__ __forceinline__ float2 add2(float2 a, float2 b) { return __fadd2_rn(a
 __device__ __forceinline__ float2 sub2(float2 a, float2 b) { return __ffma2_rn(b, make_float2(-1.f, -1.f), a); }
 __device__ __forceinline__ float2 mul2(float2 a, float2 b) { return __fmul2_rn(a, b); }
 __device__ __forceinline__ float2 fma2(float2 a, float2 b, float2 c) { return __ffma2_rn(a, b, c); }  // a b + c
+
+// s + e = a + b exactly, per half
+__device__ __forceinline__ void two_sum2(float2 a, float2 b, float2& s, float2& e) {
+  s = add2(a, b);
+  const float2 bb = sub2(s, a);
+  e = add2(sub2(a, sub2(s, bb)), sub2(b, bb));
+}
 
 // BF16 pair (low half = .x) of two FP32 values that are exact in BF16 (their
 // low 16 bits are zero): the upper halves, by byte permute
