@@ -926,6 +926,7 @@ extern "C" q4c_status grid_partition(const q4c_grid_desc* d, const q4c_tables* t
   for (size_t wv = 0; wv + 1 < g->wave_b0.size(); ++wv) {
     struct Key {
       int bucket;
+      bool pair;  // for the pair kernel
       double cost;
       int64_t b;
     };
@@ -934,18 +935,32 @@ extern "C" q4c_status grid_partition(const q4c_grid_desc* d, const q4c_tables* t
       const double np = static_cast<double>(bptr[b + 1] - bptr[b]);
       const int64_t nbi = g->h_bat_fn_ptr[b + 1] - g->h_bat_fn_ptr[b];
       const double nb = static_cast<double>(nbi);
-      bl.push_back({tile_bucket(nbi), np * nb * nb, b});
+      bl.push_back({tile_bucket(nbi), nbi > kPairNb, np * nb * nb, b});
     }
     std::stable_sort(bl.begin(), bl.end(), [](const Key& x, const Key& y) {
-      return x.bucket != y.bucket ? x.bucket < y.bucket : x.cost > y.cost;
+      return x.bucket != y.bucket ? x.bucket < y.bucket : x.pair != y.pair ? x.pair < y.pair : x.cost > y.cost;
     });
     std::vector<int64_t> bw(kTileBuckets + 1, -1);
+    int64_t pair0 = -1;
     for (const Key& x : bl) {
+      if (pair0 < 0 && x.pair) pair0 = static_cast<int64_t>(sitems.size());
       for (int k = 0; k <= x.bucket; ++k)
         if (bw[k] < 0) bw[k] = static_cast<int64_t>(sitems.size());
       const int64_t b = x.b;
       const int nb = static_cast<int>(g->h_bat_fn_ptr[b + 1] - g->h_bat_fn_ptr[b]);
       const int nt = (nb + 63) / 64;
+      if (x.pair) {  // the pair kernel's items (split_pairs.cu: batch, type, tj, ti0 | ti1 << 16)
+        for (int j = 0; j < nt; ++j) {
+          for (int i = 0; i + 1 <= j; i += 2)  // W0 (three products), SO x, y, z (two), V
+            for (int type : {1, 2, 3, 4, 0}) sitems.push_back(make_int4(static_cast<int>(b), type, j, i | (i + 1) << 16));
+          if (j % 2 == 0) {  // the diagonal tile alone
+            sitems.push_back(make_int4(static_cast<int>(b), 6, j, j | j << 16));
+            sitems.push_back(make_int4(static_cast<int>(b), 7, j, j | j << 16));
+            sitems.push_back(make_int4(static_cast<int>(b), 0, j, j | static_cast<int>(0xffff0000u)));
+          }
+        }
+        continue;
+      }
       for (int o : {1, 0, 2, 3, 4})
         for (int i = 0; i < nt; ++i)
           for (int j = i; j < nt; ++j) sitems.push_back(make_int4(static_cast<int>(b), o, i, j));
@@ -953,6 +968,7 @@ extern "C" q4c_status grid_partition(const q4c_grid_desc* d, const q4c_tables* t
     for (int k = 0; k <= kTileBuckets; ++k)
       if (bw[k] < 0) bw[k] = static_cast<int64_t>(sitems.size());
     g->split_bw0.insert(g->split_bw0.end(), bw.begin(), bw.end());
+    g->split_pair0.push_back(pair0 < 0 ? static_cast<int64_t>(sitems.size()) : pair0);
     max_wave_items = std::max(max_wave_items, static_cast<int64_t>(sitems.size()) - g->split_w0.back());
     g->split_w0.push_back(static_cast<int64_t>(sitems.size()));
   }
@@ -962,20 +978,29 @@ extern "C" q4c_status grid_partition(const q4c_grid_desc* d, const q4c_tables* t
   g->col_w0.push_back(0);
   for (size_t wv = 0; wv + 1 < g->wave_b0.size(); ++wv) {
     std::vector<int64_t> bw(kTileBuckets + 1, -1);
-    for (int64_t n = g->split_w0[wv]; n < g->split_w0[wv + 1]; ++n) {
-      const int4 it = sitems[n];
-      if (it.y != 1 || it.z != 0 || it.w != 0) continue;  // once per batch (its first item)
-      const int64_t b = it.x;
+    int64_t pair0 = -1;
+    for (int64_t n = g->split_w0[wv], last = -1; n < g->split_w0[wv + 1]; ++n) {
+      if (sitems[n].x == last) continue;  // once per batch
+      const int64_t b = last = sitems[n].x;
       const int64_t nbi = g->h_bat_fn_ptr[b + 1] - g->h_bat_fn_ptr[b];
       for (int k = 0; k <= tile_bucket(nbi); ++k)
         if (bw[k] < 0) bw[k] = static_cast<int64_t>(citems.size());
       const int nt = static_cast<int>((nbi + 63) / 64);
+      if (nbi > kPairNb) {
+        if (pair0 < 0) pair0 = static_cast<int64_t>(citems.size());
+        for (int j = 0; j < nt; ++j)
+          for (int i = 0; i < nt; i += 2)
+            citems.push_back(make_int4(static_cast<int>(b), 5, j,
+                                       i | (i + 1 < nt ? (i + 1) << 16 : static_cast<int>(0xffff0000u))));
+        continue;
+      }
       for (int i = 0; i < nt; ++i)
         for (int j = 0; j < nt; ++j) citems.push_back(make_int4(static_cast<int>(b), 5, i, j));
     }
     for (int k = 0; k <= kTileBuckets; ++k)
       if (bw[k] < 0) bw[k] = static_cast<int64_t>(citems.size());
     g->col_bw0.insert(g->col_bw0.end(), bw.begin(), bw.end());
+    g->col_pair0.push_back(pair0 < 0 ? static_cast<int64_t>(citems.size()) : pair0);
     max_wave_items = std::max(max_wave_items, static_cast<int64_t>(citems.size()) - g->col_w0.back());
     g->col_w0.push_back(static_cast<int64_t>(citems.size()));
   }

@@ -20,6 +20,10 @@ constexpr int kDPitch = 352;  // points per batch row of the D = w v table (>= 3
 // 128 and above
 constexpr int kTileBuckets = 4;
 constexpr int kBucketNb[kTileBuckets] = {32, 64, 128, 1 << 30};
+// batches above this go to the pair kernel (split_pairs.cu), which takes over
+// where pairs of row tiles make up most of the work: at 129-205 functions (64-atom
+// cluster) 0.74 ms against 0.64 in split.cu, at 700 (304-atom slab) 34.9 against 46.2
+constexpr int kPairNb = 256;
 inline int tile_bucket(int64_t nb) {
   int k = 0;
   while (k + 1 < kTileBuckets && nb > kBucketNb[k]) ++k;
@@ -230,13 +234,15 @@ struct q4c_grid {
   // [n_waves][kTileBuckets+1] item ranges of each batch-size bucket (the
   // items of a wave are grouped by bucket), and the same for d_col_items
   std::vector<int64_t> split_bw0, col_bw0;
+  // [n_waves] first item of a wave's last bucket that is one of the pair kernel
+  std::vector<int64_t> split_pair0, col_pair0;
   int split_ks[4] = {1, 1, 1, 1};          // K-steps of 16 points per pipeline stage, per bucket (tuner)
   double tune_ms[4][2] = {{-1, -1}, {-1, -1}, {-1, -1}, {-1, -1}};  // tuner timings per bucket and shape
   int rd_ks = 1;                           // K-steps per stage of the density/adjoint kernel (tuner)
   double rd_tune_ms[2] = {-1, -1};         // tuner timings of the adjoint with one and two K-steps
   int4* d_split_items = nullptr;
   std::vector<int64_t> col_w0;             // [n_waves+1] ranges into d_col_items
-  int4* d_col_items = nullptr;             // per-column operator: (batch, 5, ti, tj), every tile pair
+  int4* d_col_items = nullptr;             // per-column operator: every tile pair
   float* d_split_mag = nullptr;            // [items of the largest wave][128] rounding constants
   void* d_tmaps = nullptr;                 // [n_batches] 3-D TMA maps (points, functions, quantity) of the
                                            // tiles: boxes of 16 x 64
@@ -301,6 +307,9 @@ q4c_status integrate_split(const q4c_tables* t, const q4c_grid* g, const double*
                            cudaStream_t s);
 q4c_status integrate_columns_split(const q4c_tables* t, const q4c_grid* g, const double* v, double* F,
                                    cudaStream_t s);
+// split_pairs.cu: the products of items of batches above kPairNb functions
+q4c_status launch_pairs(int ks, const q4c_grid* g, const int4* items, int n, double* V, double* W0, double* SOx,
+                        double* SOy, double* SOz, const char* name, cudaStream_t s);
 // per-wave pieces of the split path, for the fused pass (fused.cu)
 q4c_status products_wave(const q4c_grid* g, int wv, const q4c_matrices* out, cudaStream_t s);
 // (slot 0: the density's prepared matrices, 5: the adjoint's)

@@ -457,7 +457,28 @@ __global__ void __launch_bounds__(kThreads, 1)
       const int N = item_nb(nb, item.w);  // accumulator blocks are N columns wide
       const int* idx = G.bat_idx + G.bat_idx_ptr[b];
       double* out = (o == 0 || o == 5) ? V : o == 1 ? W0 : o == 2 ? SOx : o == 3 ? SOy : SOz;
+      const int col = et & 15;
+      // value offsets of this thread's eight elements of columns c0 .. c0 + 15,
+      // all loads at once (a load and its use element by element left the
+      // epilogue 22,000 clocks an item, this 16,700): the element (i, j) itself, for
+      // V and W0 where i <= j, for SO where i != j (a diagonal tile pair holds A_k,
+      // so A_k(i, j) - A_k(j, i) goes to (i, j), i < j; an off-diagonal one holds
+      // SO_k itself), for the per-column operator always
+      int off[8];
+      auto load_off = [&](int c0) {
+        const int j = j0 + c0 + col;
+#pragma unroll
+        for (int qr = 0; qr < 8; ++qr) {
+          const int i = i0 + (et >> 4) + 8 * qr;
+          const bool swap = o >= 2 && o <= 4 && i > j;
+          const int ri = min(swap ? j : i, nb - 1), rj = min(swap ? i : j, nb - 1);
+          const int v = __ldg(idx + ri * nb + rj);
+          const bool use = i < nb && j < nb && (o == 5 || (o <= 1 ? i <= j : i != j));
+          off[qr] = use ? v : -1;
+        }
+      };
       for (int c0 = eg * 16; c0 < N; c0 += 32) {
+        load_off(c0);
 #pragma unroll
         for (int blk = 0; blk < 3; ++blk) {
           float vv[16];
@@ -467,11 +488,10 @@ __global__ void __launch_bounds__(kThreads, 1)
         }
         bar_sync(3 + eg, 128);
         // thread -> (column, rows): a warp covers 16 consecutive columns of two rows
-        const int col = et & 15, j = j0 + c0 + col;
-#pragma unroll 2
+#pragma unroll
         for (int qr = 0; qr < 8; ++qr) {
-          const int r = (et >> 4) + 8 * qr, i = i0 + r;
-          if (i >= nb || j >= nb) continue;
+          if (off[qr] < 0) continue;
+          const int r = (et >> 4) + 8 * qr;
           const float L0 = stg[r * kEpiPitch + col], L1 = stg[(r + 64) * kEpiPitch + col];
           const float L2 = stg[(128 + r) * kEpiPitch + col], L3 = stg[(192 + r) * kEpiPitch + col];
           const float L4 = stg[(256 + r) * kEpiPitch + col], L5 = stg[(320 + r) * kEpiPitch + col];
@@ -485,20 +505,7 @@ __global__ void __launch_bounds__(kThreads, 1)
           const float e2 = (s1 - (sm - bp)) + (L2 - bp);
           const float lo = (e1 + e2) + (L3 + (L4 + L5));
           const double val = static_cast<double>(sm) + static_cast<double>(lo);
-          int ri = i, rj = j;
-          double sgn = 1.0;
-          if (o == 5) {
-            // not symmetric: every (i, j) into its own block
-          } else if (o <= 1) {
-            if (i > j) continue;
-          } else {
-            // SO: a diagonal tile pair holds A_k, so A_k(i, j) - A_k(j, i) goes
-            // to (i, j), i < j; an off-diagonal one holds SO_k itself (i < j)
-            if (i == j) continue;
-            if (i > j) { ri = j; rj = i; sgn = -1.0; }
-          }
-          const int off = __ldg(idx + ri * nb + rj);
-          if (off >= 0) atomicAdd(out + off, sgn * val);
+          atomicAdd(out + off[qr], o >= 2 && o <= 4 && i0 + r > j0 + c0 + col ? -val : val);
         }
         bar_sync(3 + eg, 128);
       }
@@ -535,23 +542,28 @@ q4c_status launch_products(const q4c_grid* g, const int4* items, int n, const fl
   return Q4C_OK;
 }
 
-// items[0, n) with their rounding constants mag[128 n]
-q4c_status launch_products_ks(int ks, const q4c_grid* g, const int4* items, int n, const float* mag, double* V,
-                              double* W0, double* SOx, double* SOy, double* SOz, const char* name, cudaStream_t s) {
-  if (n <= 0) return Q4C_OK;
-  return ks == 2 ? launch_products<2>(g, items, n, mag, V, W0, SOx, SOy, SOz, name, s)
-                 : launch_products<1>(g, items, n, mag, V, W0, SOx, SOy, SOz, name, s);
+// items[0, n) with their rounding constants mag[128 n]; from n_split on they are
+// items of the pair kernel, which needs none
+q4c_status launch_products_ks(int ks, const q4c_grid* g, const int4* items, int n, int n_split, const float* mag,
+                              double* V, double* W0, double* SOx, double* SOy, double* SOz, const char* name,
+                              cudaStream_t s) {
+  n_split = std::max(0, std::min(n_split, n));
+  if (n_split > 0)
+    if (q4c_status st = ks == 2 ? launch_products<2>(g, items, n_split, mag, V, W0, SOx, SOy, SOz, name, s)
+                                : launch_products<1>(g, items, n_split, mag, V, W0, SOx, SOy, SOz, name, s))
+      return st;
+  if (n <= n_split) return Q4C_OK;
+  return launch_pairs(ks, g, items + n_split, n - n_split, V, W0, SOx, SOy, SOz, name, s);
 }
 
 // items of one wave: rounding constants of all of them, then one launch per
 // batch-size bucket with the stage shape chosen for that bucket
-q4c_status products_items(const q4c_grid* g, const int4* d_items, const std::vector<int64_t>& bucket_w0, int wv,
-                          double* V, double* W0, double* SOx, double* SOy, double* SOz, const char* name,
+q4c_status products_items(const q4c_grid* g, const int4* d_items, const std::vector<int64_t>& bucket_w0, int64_t pair0,
+                          int wv, double* V, double* W0, double* SOx, double* SOy, double* SOz, const char* name,
                           cudaStream_t s) {
   const int64_t* r = bucket_w0.data() + static_cast<size_t>(wv) * (kTileBuckets + 1);
-  const int64_t i0 = r[0], i1 = r[kTileBuckets];
-  if (i1 <= i0) return Q4C_OK;
-  {
+  const int64_t i0 = r[0], i1 = pair0;
+  if (i1 > i0) {
     KernelScope ks("split_prep", s);
     split::k_item_prep<<<static_cast<unsigned>(i1 - i0), 128, 0, s>>>(g->view(), d_items + i0, g->d_colexp,
                                                                        g->d_split_mag);
@@ -563,7 +575,7 @@ q4c_status products_items(const q4c_grid* g, const int4* d_items, const std::vec
     const int64_t b0 = r[k], b1 = r[k + 1];
     if (b1 <= b0) continue;
     if (q4c_status st = launch_products_ks(g->split_ks[k], g, d_items + b0, static_cast<int>(b1 - b0),
-                                           g->d_split_mag + (b0 - i0) * 128, V, W0, SOx, SOy, SOz, name, s))
+                                           static_cast<int>(pair0 - b0), g->d_split_mag + (b0 - i0) * 128, V, W0, SOx, SOy, SOz, name, s))
       return st;
   }
   return Q4C_OK;
@@ -575,7 +587,7 @@ q4c_status products_items(const q4c_grid* g, const int4* d_items, const std::vec
 // over the wave's items; the wave's offset tables, basis tiles, column
 // exponents and D row must already be in place
 q4c_status products_wave(const q4c_grid* g, int wv, const q4c_matrices* out, cudaStream_t s) {
-  return products_items(g, g->d_split_items, g->split_bw0, wv, out->V, out->W0, out->SOx, out->SOy, out->SOz,
+  return products_items(g, g->d_split_items, g->split_bw0, g->split_pair0[wv], wv, out->V, out->W0, out->SOx, out->SOy, out->SOz,
                         "split_products", s);
 }
 
@@ -615,7 +627,7 @@ q4c_status integrate_columns_split(const q4c_tables* t, const q4c_grid* g, const
     if (b1 <= b0) continue;
     if (q4c_status st = launch_fill_idx(t, g, b0, b1, s)) return st;
     if (q4c_status st = launch_basis_df(t, g, b0, b1, v, g->d_colexp, nullptr, 2, s, g->d_dpad)) return st;
-    if (q4c_status st = products_items(g, g->d_col_items, g->col_bw0, wv, F, nullptr, nullptr, nullptr, nullptr,
+    if (q4c_status st = products_items(g, g->d_col_items, g->col_bw0, g->col_pair0[wv], wv, F, nullptr, nullptr, nullptr, nullptr,
                                        "split_columns", s))
       return st;
   }
@@ -644,9 +656,10 @@ q4c_status autotune_split(const q4c_tables* t, q4c_grid* g, const double* v, cud
     if (st) return st;
   }
   const int64_t* r = g->split_bw0.data();
-  const int64_t i0 = r[0], i1 = r[kTileBuckets];
-  if (i1 <= i0) return Q4C_OK;
-  split::k_item_prep<<<static_cast<unsigned>(i1 - i0), 128, 0, s>>>(g->view(), g->d_split_items + i0, g->d_colexp,
+  const int64_t i0 = r[0], i1 = g->split_pair0[0];
+  if (r[kTileBuckets] <= i0) return Q4C_OK;
+  if (i1 > i0)
+    split::k_item_prep<<<static_cast<unsigned>(i1 - i0), 128, 0, s>>>(g->view(), g->d_split_items + i0, g->d_colexp,
                                                                      g->d_split_mag);
   Q4C_CUDA(cudaGetLastError());
   double* scratch = nullptr;
@@ -666,14 +679,14 @@ q4c_status autotune_split(const q4c_tables* t, q4c_grid* g, const double* v, cud
     const float* mag = g->d_split_mag + (c0 - i0) * 128;
     for (int ks = 1; ks <= 2 && status == Q4C_OK; ++ks) {
       float ms = 0.f;
-      if (q4c_status st = launch_products_ks(ks, g, g->d_split_items + c0, static_cast<int>(c1 - c0), mag, o[0],
+      if (q4c_status st = launch_products_ks(ks, g, g->d_split_items + c0, static_cast<int>(c1 - c0), static_cast<int>(i1 - c0), mag, o[0],
                                              o[1], o[2], o[3], o[4], "split_tune", s)) {
         fail(st);
         break;
       }
       cudaEventRecord(e0, s);
       for (int rep = 0; rep < 3 && status == Q4C_OK; ++rep)
-        if (q4c_status st = launch_products_ks(ks, g, g->d_split_items + c0, static_cast<int>(c1 - c0), mag, o[0],
+        if (q4c_status st = launch_products_ks(ks, g, g->d_split_items + c0, static_cast<int>(c1 - c0), static_cast<int>(i1 - c0), mag, o[0],
                                                o[1], o[2], o[3], o[4], "split_tune", s))
           fail(st);
       cudaEventRecord(e1, s);

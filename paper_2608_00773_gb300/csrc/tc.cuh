@@ -265,6 +265,42 @@ __device__ __forceinline__ void tmem_ld8x3(uint32_t t0, uint32_t t1, uint32_t t2
   }
 }
 
+// six 8-column loads (levels `step` columns apart) under a single wait
+__device__ __forceinline__ void tmem_ld8x6(uint32_t t, uint32_t step, float (*v)[8]) {
+  uint32_t a[6][8];
+  asm volatile(
+      "tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%48];\n\t"
+      "tcgen05.ld.sync.aligned.32x32b.x8.b32 {%8,%9,%10,%11,%12,%13,%14,%15}, [%49];\n\t"
+      "tcgen05.ld.sync.aligned.32x32b.x8.b32 {%16,%17,%18,%19,%20,%21,%22,%23}, [%50];\n\t"
+      "tcgen05.ld.sync.aligned.32x32b.x8.b32 {%24,%25,%26,%27,%28,%29,%30,%31}, [%51];\n\t"
+      "tcgen05.ld.sync.aligned.32x32b.x8.b32 {%32,%33,%34,%35,%36,%37,%38,%39}, [%52];\n\t"
+      "tcgen05.ld.sync.aligned.32x32b.x8.b32 {%40,%41,%42,%43,%44,%45,%46,%47}, [%53];\n\t"
+      "tcgen05.wait::ld.sync.aligned;"
+      : "=r"(a[0][0]), "=r"(a[0][1]), "=r"(a[0][2]), "=r"(a[0][3]), "=r"(a[0][4]), "=r"(a[0][5]), "=r"(a[0][6]),
+        "=r"(a[0][7]), "=r"(a[1][0]), "=r"(a[1][1]), "=r"(a[1][2]), "=r"(a[1][3]), "=r"(a[1][4]), "=r"(a[1][5]),
+        "=r"(a[1][6]), "=r"(a[1][7]), "=r"(a[2][0]), "=r"(a[2][1]), "=r"(a[2][2]), "=r"(a[2][3]), "=r"(a[2][4]),
+        "=r"(a[2][5]), "=r"(a[2][6]), "=r"(a[2][7]), "=r"(a[3][0]), "=r"(a[3][1]), "=r"(a[3][2]), "=r"(a[3][3]),
+        "=r"(a[3][4]), "=r"(a[3][5]), "=r"(a[3][6]), "=r"(a[3][7]), "=r"(a[4][0]), "=r"(a[4][1]), "=r"(a[4][2]),
+        "=r"(a[4][3]), "=r"(a[4][4]), "=r"(a[4][5]), "=r"(a[4][6]), "=r"(a[4][7]), "=r"(a[5][0]), "=r"(a[5][1]),
+        "=r"(a[5][2]), "=r"(a[5][3]), "=r"(a[5][4]), "=r"(a[5][5]), "=r"(a[5][6]), "=r"(a[5][7])
+      : "r"(t), "r"(t + step), "r"(t + 2 * step), "r"(t + 3 * step), "r"(t + 4 * step), "r"(t + 5 * step)
+      : "memory");
+#pragma unroll
+  for (int l = 0; l < 6; ++l)
+#pragma unroll
+    for (int i = 0; i < 8; ++i) v[l][i] = __uint_as_float(a[l][i]);
+}
+
+// x as a double on the integer pipes (the FP64 units, where a conversion would
+// run, take 16 clocks a warp instruction)
+__device__ __forceinline__ double widen(float x) {
+  const uint32_t u = __float_as_uint(x);
+  const uint32_t e = (u >> 23) & 0xffu;
+  if (e == 0u || e == 255u) return static_cast<double>(x);  // zero, subnormal, infinite, NaN
+  return __hiloint2double(static_cast<int>((u & 0x80000000u) | (((u & 0x7fffffffu) >> 3) + 0x38000000u)),
+                          static_cast<int>(u << 29));
+}
+
 // ------------------------------------------------------------ slicing
 // The split of a value x against a column exponent e (|x| <= 2^e):
 //   x = sum_s d_s 2^(e - 6 - 8 s) + O(2^(e - 47)),  s = 0..5,
@@ -354,6 +390,37 @@ __device__ __forceinline__ void slice6x2(float2 h, float2 l, float m0, float2 d[
     d[s] = t;
     if (s + 1 < kSlices) x = sub2(x, t);
     m = __fmul_rn(m, 0x1p-8f);
+  }
+}
+
+// slice6x2 on N pairs side by side (pair n against m0[n]): w[n][s] is digit s of
+// pair n in BF16.  The digits of one pair are a chain of 18 dependent operations;
+// N chains in lockstep keep the FP32 pipes busy from a single warp.
+template <int N>
+__device__ __forceinline__ void slice_pairs(float2 (&x)[N], const float2 (&l)[N], const float (&m0)[N],
+                                            uint32_t (&w)[N][kSlices]) {
+  float m[N];
+#pragma unroll
+  for (int n = 0; n < N; ++n) m[n] = m0[n];
+#pragma unroll
+  for (int s = 0; s < kSlices; ++s) {
+    float2 t[N];
+    if (s == 3) {
+#pragma unroll
+      for (int n = 0; n < N; ++n) x[n] = add2(x[n], l[n]);
+    }
+#pragma unroll
+    for (int n = 0; n < N; ++n) t[n] = add2(x[n], pk2(m[n], m[n]));
+#pragma unroll
+    for (int n = 0; n < N; ++n) t[n] = sub2(t[n], pk2(m[n], m[n]));
+    if (s + 1 < kSlices) {
+#pragma unroll
+      for (int n = 0; n < N; ++n) x[n] = sub2(x[n], t[n]);
+#pragma unroll
+      for (int n = 0; n < N; ++n) m[n] = __fmul_rn(m[n], 0x1p-8f);
+    }
+#pragma unroll
+    for (int n = 0; n < N; ++n) w[n][s] = bf16x2_exact(t[n]);
   }
 }
 
