@@ -233,8 +233,18 @@ __device__ __forceinline__ void harmonics_s(df x, df y, df z, int lmax, df* S) {
   }
 }
 
+// What bounds it: instruction issue and the loads of the harmonics, kept in
+// indexed local arrays (the values leave at half the HBM rate).  64 registers for
+// 32 warps an SM: 48, 56, 80 and 96 are slower by 4 to 17 %; the same with the
+// harmonics unrolled per l (45 KB of code) waits for instructions three times as
+// long as it issues.  A function's column maxima go to shared memory with one
+// atomic over the lanes that hold them; a warp none of whose points lies inside
+// the centre's cutoff writes zeros and goes on.  64-atom cluster, 70M
+// function-point pairs, four quantities (3.4 GB): 1.25 ms with an atomic per
+// maximum and every warp evaluated, 1.11 with the one atomic, 1.00 with both; Phi
+// and Psi 0.68 -> 0.56; 304-atom slab 4.25 -> 2.81.
 template <int NQ, int LM>
-__global__ void __launch_bounds__(256, 4) k_basis_df(DevBasis B, DevGrid G, DfTables T, int64_t b0,
+__global__ void __launch_bounds__(512, 2) k_basis_df(DevBasis B, DevGrid G, DfTables T, int64_t b0,
                                                   const int64_t* __restrict__ scr_off, float2* __restrict__ scratch,
                                                   const double* __restrict__ v, int* __restrict__ colexp,
                                                   int* __restrict__ rowexp, float2* __restrict__ dpad,
@@ -276,6 +286,7 @@ __global__ void __launch_bounds__(256, 4) k_basis_df(DevBasis B, DevGrid G, DfTa
       in = r64 < B.r_c;
       below = r64 < B.r_min;
     }
+    const bool any = __any_sync(0xffffffffu, in);
     int eD = -30000;
     if (colexp && live) {
       const double Dp = NQ == 2 ? G.w[p0 + p] : G.w[p0 + p] * v[p0 + p];
@@ -286,6 +297,15 @@ __global__ void __launch_bounds__(256, 4) k_basis_df(DevBasis B, DevGrid G, DfTa
       }
     } else if (dpad && a == 0 && p < ((np + 31) & ~31)) {
       dpad[b * kDPitch + p] = make_float2(0.f, 0.f);  // stages of 16 or 32 points read zeros past n_p
+    }
+    if (!any) {  // no point of the warp inside the centre's cutoff: its functions are zero there
+      int nf = 0;
+      for (int q = 0; q < nr; ++q) nf += 2 * __ldg(B.rad_l + r0 + q) + 1;
+      float2* o = base + static_cast<int64_t>(f0) * ldp + p;
+      if (live)
+        for (int c = 0; c < NQ; ++c)
+          for (int i = 0; i < nf; ++i) o[c * plane + static_cast<int64_t>(i) * ldp] = make_float2(0.f, 0.f);
+      continue;
     }
     const df vdf = (NQ == 2 && live) ? split_d(v[p0 + p]) : df{0.f, 0.f};
     int lmax = 0;
@@ -366,6 +386,9 @@ __global__ void __launch_bounds__(256, 4) k_basis_df(DevBasis B, DevGrid G, DfTa
 #pragma unroll
         for (int c = 0; c < NQ; ++c) rmax[c] = fmaxf(rmax[c], fabsf(vals[c].hi));
         if (colexp) {
+          // lane i keeps maximum i of the 2 NQ (with D, then without) and the lanes
+          // add them to the column's with one shared atomic
+          int mine = -30000;
 #pragma unroll
           for (int c = 0; c < NQ; ++c) {
             const float h = vals[c].hi;
@@ -373,11 +396,9 @@ __global__ void __launch_bounds__(256, 4) k_basis_df(DevBasis B, DevGrid G, DfTa
             const int ea = (e > -30000 && eD > -30000) ? e + eD : -30000;
             const int mb = __reduce_max_sync(0xffffffffu, e);
             const int ma = __reduce_max_sync(0xffffffffu, ea);
-            if (lane == 0) {
-              if (mb > -30000) atomicMax(&s_col[(4 + c) * nb + f], mb);
-              if (ma > -30000) atomicMax(&s_col[c * nb + f], ma);
-            }
+            mine = lane == c ? ma : lane == NQ + c ? mb : mine;
           }
+          if (mine > -30000) atomicMax(&s_col[(lane < NQ ? lane : 4 + lane - NQ) * nb + f], mine);
         }
       }
     }
@@ -424,7 +445,12 @@ q4c_status launch_basis_df(const q4c_tables* t, const q4c_grid* g, int64_t b0, i
   T.pts = g->d_pts_df;
   T.atoms = g->d_atoms_df;
   KernelScope ks("basis_df", s);
-  kern<<<static_cast<unsigned>(b1 - b0), 256, smem, s>>>(t->view(), g->view(), T, b0, g->d_scr_off,
+  // a wave with no more batches than SMs: 16 warps a batch instead of 8 (one
+  // molecule of 3 atoms, 60 batches: 26 us with 8, 16 with 16)
+  int dev = 0, n_sm = 0;
+  cudaGetDevice(&dev);
+  cudaDeviceGetAttribute(&n_sm, cudaDevAttrMultiProcessorCount, dev);
+  kern<<<static_cast<unsigned>(b1 - b0), b1 - b0 <= n_sm ? 512 : 256, smem, s>>>(t->view(), g->view(), T, b0, g->d_scr_off,
                                                                      reinterpret_cast<float2*>(g->d_scratch), v,
                                                                      colexp, rowexp, dpad, t->d_col_coef_df,
                                                                      t->d_col_eps);
