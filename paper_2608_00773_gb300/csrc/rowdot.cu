@@ -157,88 +157,113 @@ __host__ __device__ __forceinline__ int jt_chunks(int m, int n_ic, int jt) {
   return m < 2 && n < n_ic ? n : n_ic;
 }
 
-// Pre-pass: CTAs (batch, matrix, share of the j-tiles).  Per j-tile the column
-// exponents e_j (|G'_ij| < 2^e_j over the batch's i), then the six digits of
-// every G'_ij written as the B operand of the main kernel: block (jt, ic) = six
-// tiles of jt_width rows (j) x 16 K (i), 32 bytes a row, in the no-swizzle
-// K-major layout, back to back, at (jt * n_ic) * 6 KB + ic * 192 * jt_width;
-// padding rows and columns, and for V and W i > j, are 0.
+// Pre-pass: CTAs (batch, share of the j-tiles), all NM matrices (V alone or the
+// five).  Per j-tile the column exponents e_j (|G'_ij| < 2^e_j over the batch's i),
+// then the six digits of every G'_ij written as the B operand of the main kernel:
+// block (jt, ic) = six tiles of jt_width rows (j) x 16 K (i), 32 bytes a row, in
+// the no-swizzle K-major layout, back to back, at (jt * n_ic) * 6 KB + ic * 192 *
+// jt_width; padding rows and columns, and for V and W i > j, are 0.
 // The column bound is the largest column bound (k_prepare_blocks) of the blocks
 // (a, c) of column j's centre c over the batch's active centres a, whose
 // functions are exactly the batch's i.
+// What bounds it: the stores (12 bytes an element and matrix; 5 TB/s with the reads
+// on batches of 900 functions).  A warp takes units of 8 j x 8 i (32 words of a tile, an
+// element pair each), so a unit's place needs no division and its offsets are read
+// once for all matrices.  One matrix a CTA with offsets and divisions of its own:
+// 24 molecules 6.8 ms -> 4.4, 64-atom cluster 0.60 -> 0.43; the slab's large
+// batches, already at the memory's rate, 12.1 and 12.5.
+template <int NM>
 __global__ void __launch_bounds__(256) k_gslice(DevGrid G, int64_t b0, const float2* __restrict__ prep, int64_t nnz,
                                                 unsigned present, const float* __restrict__ cm, int64_t cm_total,
                                                 const int* __restrict__ pair_blk, const int64_t* __restrict__ cm_off,
                                                 const int64_t* __restrict__ gsl_off, uint32_t* __restrict__ gsl) {
-  __shared__ unsigned sMax[kTileJ];  // bits of the columns' bounds
+  constexpr int kB = NM > 1 ? 2 : 1;      // column bounds: of V, of the other matrices
+  __shared__ unsigned sMax[kB][kTileJ];  // their bits
   const int64_t b = b0 + blockIdx.x;
-  const int m = blockIdx.y;
-  if (!(present >> m & 1u)) return;
-  const float2* M = prep + m * nnz;
-  const float* CM = cm + (m ? cm_total : 0);
   const int64_t f0 = G.bat_fn_ptr[b];
   const int nb = static_cast<int>(G.bat_fn_ptr[b + 1] - f0);
   const int* idx = G.bat_idx + G.bat_idx_ptr[b];
   const int n_jt = (nb + kTileJ - 1) / kTileJ, n_ic = (nb + kKc - 1) / kKc;
   const int na = G.bat_atom_ptr[b + 1] - G.bat_atom_ptr[b];
   const int* pb = pair_blk + G.bat_pair_ptr[b];
-  uint32_t* out = gsl + (gsl_off[b] + static_cast<int64_t>(m) * n_jt * n_ic * kBlockB) / 4;
-  for (int jt = blockIdx.z; jt < n_jt; jt += gridDim.z) {
+  uint32_t* out = gsl + gsl_off[b] / 4;
+  const int64_t mstride = static_cast<int64_t>(n_jt) * n_ic * (kBlockB / 4);  // words of one matrix
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, nwarps = blockDim.x >> 5;
+  const int r8 = lane >> 2, kp = lane & 3;
+  for (int jt = blockIdx.y; jt < n_jt; jt += gridDim.y) {
     __syncthreads();
-    if (threadIdx.x < kTileJ) sMax[threadIdx.x] = 0u;
+    if (threadIdx.x < kB * kTileJ) sMax[threadIdx.x / kTileJ][threadIdx.x % kTileJ] = 0u;
     __syncthreads();
     {  // column bounds: eight threads a column over the batch's centres
-      const int j = jt * kTileJ + (threadIdx.x >> 3);
+      const int jl = threadIdx.x >> 3, j = jt * kTileJ + jl;
       if (j < nb) {
         const int info = G.fn_info[f0 + j], c = info >> 16, jj = info & 0xffff;
-        float mx = 0.f;
+        float mx[kB] = {};
         for (int a = threadIdx.x & 7; a < na; a += 8) {
           const int q = pb[a * na + c];  // block (a, c): its column jj
-          if (q >= 0) mx = fmaxf(mx, __ldg(CM + cm_off[q] + jj));
+          if (q >= 0) {
+            const int64_t o = cm_off[q] + jj;
+#pragma unroll
+            for (int k = 0; k < kB; ++k) mx[k] = fmaxf(mx[k], __ldg(cm + k * cm_total + o));
+          }
         }
-        atomicMax(&sMax[threadIdx.x >> 3], __float_as_uint(mx));
+#pragma unroll
+        for (int k = 0; k < kB; ++k) atomicMax(&sMax[k][jl], __float_as_uint(mx[k]));
       }
     }
     __syncthreads();
     const int w = jt_width(nb, jt), tw = w * 8;  // words of one tile (one per element pair)
-    const int words = jt_chunks(m, n_ic, jt) * tw;
+    const int sh = w == kTileJ ? 3 : 2;          // log2 of a block's units, w / 4
+    const int n_low = jt_chunks(0, n_ic, jt) << sh;  // units that V and W have
+    const int units = (present & ~3u) ? n_ic << sh : n_low;
     uint32_t* oj = out + static_cast<int64_t>(jt) * n_ic * (kBlockB / 4);
-    // a thread takes kU words (element pairs) at a time and issues all their
-    // offset loads, then all their value loads, before slicing any
-    constexpr int kU = 4;
-    for (int w0 = threadIdx.x; w0 < words; w0 += kU * blockDim.x) {
+    // a warp takes kU units at a time and issues all their loads (addresses
+    // clamped, so that none depends on a condition) before slicing any
+    constexpr int kU = NM > 1 ? 2 : 4;
+    for (int u0 = warp; u0 < units; u0 += kU * nwarps) {
       int i_[kU], j_[kU], o0[kU], o1[kU];
 #pragma unroll
       for (int u = 0; u < kU; ++u) {
-        const int wd = w0 + u * blockDim.x;
-        const int ic = wd / tw, pos = wd - ic * tw;
-        // pos -> byte offset rg*SBO + kq*LBO + r8*16 + kp*4
-        const int rg = pos >> 6, kq = (pos >> 5) & 1, r8 = (pos >> 2) & 7, kp = pos & 3;
-        j_[u] = jt * kTileJ + rg * 8 + r8;
-        i_[u] = ic * kKc + kq * 8 + kp * 2;
-        const bool ok = wd < words && j_[u] < nb;
-        const int last = m < 2 ? j_[u] : nb - 1;  // last i of this column
-        o0[u] = ok && i_[u] <= last ? __ldg(idx + i_[u] * nb + j_[u]) : -1;
-        o1[u] = ok && i_[u] + 1 <= last ? __ldg(idx + (i_[u] + 1) * nb + j_[u]) : -1;
+        const int un = u0 + u * nwarps, r = un & ((1 << sh) - 1);
+        i_[u] = (un >> sh) * kKc + (r & 1) * 8 + kp * 2;
+        j_[u] = (r >> 1) * 8 + r8;
+        const int j = min(jt * kTileJ + j_[u], nb - 1);
+        o0[u] = __ldg(idx + min(i_[u], nb - 1) * nb + j);
+        o1[u] = __ldg(idx + min(i_[u] + 1, nb - 1) * nb + j);
       }
-      float2 x0[kU], x1[kU];
+      bool ok0[kU], ok1[kU];
 #pragma unroll
       for (int u = 0; u < kU; ++u) {
-        x0[u] = o0[u] < 0 ? make_float2(0.f, 0.f) : __ldg(M + o0[u]);
-        x1[u] = o1[u] < 0 ? make_float2(0.f, 0.f) : __ldg(M + o1[u]);
+        const bool jin = jt * kTileJ + j_[u] < nb;
+        ok0[u] = jin && i_[u] < nb && o0[u] >= 0;
+        ok1[u] = jin && i_[u] + 1 < nb && o1[u] >= 0;
+        o0[u] = ok0[u] ? o0[u] : 0;
+        o1[u] = ok1[u] ? o1[u] : 0;
       }
 #pragma unroll
-      for (int u = 0; u < kU; ++u) {
-        const int wd = w0 + u * blockDim.x;
-        if (wd >= words) break;
-        const int ic = wd / tw, pos = wd - ic * tw;
-        const unsigned mb = sMax[j_[u] - jt * kTileJ];
-        float2 d[kSlices];
-        slice6x2(pk2(x0[u].x, x1[u].x), pk2(x0[u].y, x1[u].y),
-                 magic0((mb ? fexp(__uint_as_float(mb)) : -30000) - kFine), d);
-        uint32_t* o = oj + ic * (kSlices * tw) + pos;
+      for (int m = 0; m < NM; ++m) {
+        if (!(present >> m & 1u)) continue;
+        const float2* M = prep + m * nnz;
+        float2 x0[kU], x1[kU];
 #pragma unroll
-        for (int t = 0; t < kSlices; ++t) o[t * tw] = bf16x2_exact(d[t]);
+        for (int u = 0; u < kU; ++u) {
+          x0[u] = __ldg(M + o0[u]);
+          x1[u] = __ldg(M + o1[u]);
+        }
+#pragma unroll
+        for (int u = 0; u < kU; ++u) {
+          const int un = u0 + u * nwarps;
+          if (un >= (m < 2 ? n_low : units)) break;
+          const int j = jt * kTileJ + j_[u];
+          const bool a0 = ok0[u] && (m >= 2 || i_[u] <= j), a1 = ok1[u] && (m >= 2 || i_[u] + 1 <= j);
+          const unsigned mb = sMax[m ? kB - 1 : 0][j_[u]];
+          float2 d[kSlices];
+          slice6x2(pk2(a0 ? x0[u].x : 0.f, a1 ? x1[u].x : 0.f), pk2(a0 ? x0[u].y : 0.f, a1 ? x1[u].y : 0.f),
+                   magic0((mb ? fexp(__uint_as_float(mb)) : -30000) - kFine), d);
+          uint32_t* o = oj + m * mstride + (un >> sh) * (kSlices * tw) + ((un & ((1 << sh) - 1)) << 5) + lane;
+#pragma unroll
+          for (int t = 0; t < kSlices; ++t) o[t * tw] = bf16x2_exact(d[t]);
+        }
       }
     }
   }
@@ -926,11 +951,11 @@ q4c_status prepare(const q4c_grid* g, const double* const mats[5], int slot, uns
 template <int MODE>
 q4c_status gslice_wave(const q4c_grid* g, int wv, int slot, unsigned present, cudaStream_t s) {
   const int64_t b0 = g->wave_b0[wv], b1 = g->wave_b0[wv + 1];
-  if (b1 <= b0) return Q4C_OK;
-  // four j-tiles a CTA: the batches of a wave differ widely in n_b
-  const unsigned z = static_cast<unsigned>(std::max(1, (g->max_nb + 4 * kTileJ - 1) / (4 * kTileJ)));
+  if (b1 <= b0 || present == 0) return Q4C_OK;
+  // two j-tiles a CTA: the batches of a wave differ widely in n_b
+  const unsigned y = static_cast<unsigned>(std::max(1, (g->max_nb + 2 * kTileJ - 1) / (2 * kTileJ)));
   KernelScope ks("split_gslice", s);
-  k_gslice<<<dim3(static_cast<unsigned>(b1 - b0), MODE == 0 ? 1 : 5, z), 256, 0, s>>>(
+  k_gslice<MODE == 0 ? 1 : 5><<<dim3(static_cast<unsigned>(b1 - b0), y), 256, 0, s>>>(
       g->view(), b0, g->d_gdf + slot * g->nnz, g->nnz, present, g->d_cm + (slot ? 2 : 0) * g->cm_total, g->cm_total,
       g->d_pair_blk, g->d_cm_off, g->d_gsl_off, reinterpret_cast<uint32_t*>(g->d_gsl));
   Q4C_CUDA(cudaGetLastError());
