@@ -308,7 +308,7 @@ q4c_status integrate_split(const q4c_tables* t, const q4c_grid* g, const double*
 q4c_status integrate_columns_split(const q4c_tables* t, const q4c_grid* g, const double* v, double* F,
                                    cudaStream_t s);
 // split_pairs.cu: the products of items of batches above kPairNb functions
-q4c_status launch_pairs(int ks, const q4c_grid* g, const int4* items, int n, double* V, double* W0, double* SOx,
+q4c_status launch_pairs(const q4c_grid* g, const int4* items, int n, double* V, double* W0, double* SOx,
                         double* SOy, double* SOz, const char* name, cudaStream_t s);
 // per-wave pieces of the split path, for the fused pass (fused.cu)
 q4c_status products_wave(const q4c_grid* g, int wv, const q4c_matrices* out, cudaStream_t s);

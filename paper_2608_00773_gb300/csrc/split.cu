@@ -57,14 +57,10 @@ constexpr int kTile = 64;                    // functions per tile (rows of one 
 constexpr int kKc = 16;                      // points per step (one K = 16 MMA step)
 constexpr int kTileBytes = kTile * kKc * 2;  // 2 KB
 constexpr int kSBO = (kKc / 8) * 128;        // 256 B between 8-row groups
-constexpr int kSlicers = 256;                // warps 0-7 slice the operands
-constexpr int kEpiWarp0 = 8;                 // warps 8-15 drain tensor memory (two groups of four)
+constexpr int kSlicers = 256;                // threads of a slicer group (8 warps, a whole stage)
 constexpr int kEpiThreads = 256;
-constexpr int kMmaWarp = 16;                 // warp 16 owns tensor memory and issues the MMAs
-constexpr int kProdWarp = 17;                // warp 17 issues the TMA loads of the raw operands
-constexpr int kThreads = 18 * 32;
-constexpr int kEpiPitch = 17;                // floats per staged TMEM lane (16 columns + pad)
-constexpr int kEpiStage = 3 * 128 * kEpiPitch * 4;  // one group's staging, 26 KB
+constexpr int kEpiPitch = kTile + 1;         // (hi, lo) pairs per staged row
+constexpr int kEpiStage = kTile * kEpiPitch * 12;  // one item's elements and a third level, 49 KB
 constexpr int kStageA = (kSlices + 1) * kTileBytes;  // [Z, A0..A5] of one K-step
 constexpr int kStageB = kSlices * kTileBytes;        // [B0..B5] of one K-step
 constexpr int kHalf = kStageA + kStageB;             // one K-step's operands, 26 KB
@@ -74,26 +70,33 @@ constexpr uint32_t kSetCols = 256;
 
 // Shared-memory layout of the kernel with KS K-steps of 16 points per
 // pipeline stage (the stage shape the tuner chooses per batch-size bucket):
-// KS = 1 keeps four operand and four raw stages, KS = 2 two of each (twice
-// the points per handshake, the same points in flight).
+// KS = 1 keeps four operand and four raw stages and two slicer groups that take
+// alternate stages (one group's waits and loads run beside the other's arithmetic:
+// 64-atom cluster 4.14 ms with one group, 3.84 with two; a group for each operand
+// instead 4.96, the handshakes of a stage doubled); KS = 2 two of each (twice the
+// points per handshake, the same points in flight) and one group (two: 4.55 ms, the
+// ring too shallow for both).
 //   raw stage:     per K-step h the A and B boxes (64 functions x 16 points
-//                  of (hi, lo), 128-byte rows, swizzled) at h * 16 KB, the
-//                  stage's D values (KS x 16 x 8 B) and, on an item's first
-//                  stage, the item's 128 rounding constants;
+//                  of (hi, lo), 128-byte rows, swizzled) at h * 16 KB and the
+//                  stage's D values (KS x 16 x 8 B);
 //   operand stage: per K-step h the six A digit tiles after a zero tile and
 //                  the six B digit tiles, at h * 26 KB.
 template <int KS>
 struct Layout {
+  static constexpr int kGroups = KS == 1 ? 2 : 1;       // slicer groups: warps 0 .. 8 kGroups - 1
+  static constexpr int kEpiWarp0 = 8 * kGroups;         // eight warps that drain tensor memory (two groups of four)
+  static constexpr int kMmaWarp = kEpiWarp0 + 8;        // owns tensor memory and issues the MMAs
+  static constexpr int kProdWarp = kMmaWarp + 1;        // issues the TMA loads of the raw operands
+  static constexpr int kThreads = 32 * (kProdWarp + 1);
   static constexpr int kStages = KS == 1 ? 4 : 2;  // ring depth of sliced operands
   static constexpr int kRaw = KS == 1 ? 4 : 2;     // ring depth of raw boxes
   static constexpr int kStage = KS * kHalf;
   static constexpr int kRawD = KS * 2 * kRawTile;              // offset of D
-  static constexpr int kRawMag = kRawD + KS * kKc * 8;         // offset of the rounding constants
-  static constexpr int kRawStage = ((kRawMag + 128 * 4 + 1023) / 1024) * 1024;  // 1024-aligned (swizzle atoms)
+  static constexpr int kRawStage = ((kRawD + KS * kKc * 8 + 1023) / 1024) * 1024;  // 1024-aligned (swizzle atoms)
   static constexpr int kSmemRaw = 0;
   static constexpr int kSmemStages = kSmemRaw + kRaw * kRawStage;
-  static constexpr int kSmemEpi = kSmemStages + kStages * kStage;  // epilogue staging, 2 x 26 KB
-  static constexpr int kSmemBar = kSmemEpi + 2 * kEpiStage;
+  static constexpr int kSmemEpi = kSmemStages + kStages * kStage;  // epilogue staging
+  static constexpr int kSmemBar = kSmemEpi + kEpiStage;
   // full, empty, accfull[2], accempty[2], drain, raw full/empty
   static constexpr int kNumBars = 2 * kStages + 5 + 2 * kRaw;
   static constexpr int kSmemTotal = kSmemBar + kNumBars * 8 + 16;
@@ -176,40 +179,42 @@ __device__ __forceinline__ void sts64(unsigned char* p, uint32_t a, uint32_t b) 
 // exponents; the subtracted SO product slices -D).
 //
 // Warp roles (one CTA per SM, items strided over the CTAs):
-//   warp 17     (one thread) loads step g's raw operands into raw stage
-//               g mod 4 once the slicers have read it (raw_empty): two TMA
-//               boxes (A and B rows of the step's quantities, zeros past n_p
-//               and n_b), the step's 16 D values and, on an item's first
-//               step, the item's rounding constants; one mbarrier (raw_full)
-//               counts the bytes;
-//   warps 0-7   thread (row r, points 4q..4q+3) reads its raw values, forms
+//   producer    (one thread) loads stage g's raw operands into raw stage
+//               g mod kRaw once the slicers have read it (raw_empty): two TMA
+//               boxes a K-step (A and B rows of the step's quantities, zeros
+//               past n_p and n_b) and the stage's D values; one mbarrier
+//               (raw_full) counts the bytes;
+//   slicers     thread (row r, points 4q..4q+3) reads its raw values, forms
 //               the D-scaled A values in double-float, slices both sides
 //               (the B side only on the item's B rows) into six BF16 digits
 //               and stores them (8 bytes per slice and side) into operand
-//               stage g mod 4 once the MMAs that last read it have completed
-//               (empty[stage], a tcgen05.commit), arrives on full[stage] and
-//               frees the raw stage;
-//   warp 16     (one thread) waits full[stage], issues the six MMAs into the
+//               stage g mod kStages once the MMAs that last read it have
+//               completed (empty[stage], a tcgen05.commit), arrives on
+//               full[stage] and frees the raw stage;
+//   MMA warp    waits full[stage], issues the six MMAs a K-step into the
 //               item's accumulator set (items alternate between two sets of
 //               up to 192 TMEM columns), commits empty[stage], and after an item's
 //               last step commits accfull[set];
-//   warps 8-15  wait accfull[set], read the six levels, combine and scatter
-//               (two groups of four warps take alternate 16-column chunks;
-//               the scatter offsets come from the batch's dense offset
-//               table), then arrive on accempty[set] so the set can take
-//               item k + 2.
+//   epilogue    (eight warps) wait accfull[set], combine the six levels of
+//               every element into an FP32 pair in shared memory (two groups of
+//               four warps take alternate 16-column chunks; levels 1, 3 and 5 lie 64 lanes below
+//               0, 2 and 4 and reach them there), arrive on accempty[set] so the
+//               set can take item k + 2, and scatter the pairs (offsets from the
+//               batch's dense offset table) while the next item runs.
 // Every wait is bounded; a role that times out sets the status bit and an
 // abort flag that ends the other roles' waits, and the MMA thread drains its
 // outstanding MMAs (bounded) before tensor memory is freed.
 template <int KS>
-__global__ void __launch_bounds__(kThreads, 1)
+__global__ void __launch_bounds__(Layout<KS>::kThreads, 1)
     k_split_products(DevGrid G, const int4* __restrict__ items, int n_items,
                      const CUtensorMap* __restrict__ maps, const float2* __restrict__ dpad,
                      const float* __restrict__ mag, double* V, double* W0, double* SOx, double* SOy, double* SOz,
                      unsigned* status) {
   using L = Layout<KS>;
   constexpr int kStages = L::kStages, kRaw = L::kRaw, kStage = L::kStage, kRawStage = L::kRawStage;
-  constexpr int kRawD = L::kRawD, kRawMag = L::kRawMag, kSmemRaw = L::kSmemRaw, kSmemStages = L::kSmemStages;
+  constexpr int kGroups = L::kGroups, kEpiWarp0 = L::kEpiWarp0, kMmaWarp = L::kMmaWarp, kProdWarp = L::kProdWarp;
+  constexpr int kThreads = L::kThreads;
+  constexpr int kRawD = L::kRawD, kSmemRaw = L::kSmemRaw, kSmemStages = L::kSmemStages;
   constexpr int kSmemEpi = L::kSmemEpi, kSmemBar = L::kSmemBar, kNumBars = L::kNumBars;
   // stages of KS x 16 points per item: the batch's points, times the products
   // the item K-concatenates
@@ -218,7 +223,7 @@ __global__ void __launch_bounds__(kThreads, 1)
     return (np + KS * kKc - 1) / (KS * kKc) * item_products(it).n;
   };
   extern __shared__ __align__(1024) unsigned char smem[];
-  float* stage = reinterpret_cast<float*>(smem + kSmemEpi);
+  float2* stg = reinterpret_cast<float2*>(smem + kSmemEpi);
   uint64_t* bars = reinterpret_cast<uint64_t*>(smem + kSmemBar);
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(smem + kSmemBar + kNumBars * 8);
   volatile int* s_abort = reinterpret_cast<volatile int*>(smem + kSmemBar + kNumBars * 8 + 4);
@@ -270,13 +275,14 @@ __global__ void __launch_bounds__(kThreads, 1)
   tc_fence_after();
   const uint32_t tmem = uniform(*tmem_slot);
 
-  if (warp < kSlicers / 32) {
+  if (warp < kEpiWarp0) {
     // ---------------------------------------------------------- slicers
     // row, points 4q..4q+3 of the step.  A quarter warp takes one q on rows
     // 0-7 (its 16-byte raw chunks 2q ^ row are then eight distinct banks
     // groups) and a half warp one K-half on rows 0-7 (its 8-byte digit slots
     // fill one 128-byte core-matrix pair without a bank conflict).
-    const int r = warp * 8 + (lane & 7), q = lane >> 3;
+    const int grp = warp >> 3;
+    const int r = (warp & 7) * 8 + (lane & 7), q = lane >> 3;
     // byte offsets: swizzled 16-byte chunks 2q, 2q+1 of row r in a raw box;
     // the 8-byte slot of (r, 4q) in a K-major core-matrix operand tile
     const int rc0 = r * 128 + (((2 * q) ^ (r & 7)) << 4), rc1 = r * 128 + (((2 * q + 1) ^ (r & 7)) << 4);
@@ -288,19 +294,16 @@ __global__ void __launch_bounds__(kThreads, 1)
       const int nbB = item_nb(static_cast<int>(G.bat_fn_ptr[item.x + 1] - G.bat_fn_ptr[item.x]), item.w);
       const int n_prod = item_products(item).n;
       const bool b_row = r < nbB;  // this warp's rows of the B tile exist (nbB is a multiple of 16)
-      float mA = 0.f, mB = 0.f;
+      const float mA = __ldg(mag + static_cast<int64_t>(n) * 128 + r), mB = __ldg(mag + static_cast<int64_t>(n) * 128 + 64 + r);
       bool ok = true;
       for (int s = 0, pr = 0; s < n_steps; ++s, ++g, pr = (pr + 1 == n_prod) ? 0 : pr + 1) {
+        if (kGroups > 1 && (g & 1) != grp) continue;
         const int rs = g % kRaw, st = g % kStages;
         if (!mbar_wait_abort(rawfull_bar(rs), (g / kRaw) & 1, s_abort, status, G.wait_ns)) {
           ok = false;
           break;
         }
         const unsigned char* raw = smem + kSmemRaw + rs * kRawStage;
-        if (s == 0) {
-          mA = reinterpret_cast<const float*>(raw + kRawMag)[r];
-          mB = reinterpret_cast<const float*>(raw + kRawMag)[64 + r];
-        }
         float4 a01[KS], a23[KS], b01[KS], b23[KS], d01[KS], d23[KS];
 #pragma unroll
         for (int h = 0; h < KS; ++h) {
@@ -359,7 +362,7 @@ __global__ void __launch_bounds__(kThreads, 1)
         if (lane == 0) mbar_arrive(rawempty_bar(rs));
       }
       // agree on stopping (a wait that gave up in one warp ends every role)
-      if (bar_red_or(1, kSlicers, !ok || *s_abort)) break;
+      if (bar_red_or(1 + 4 * grp, kSlicers, !ok || *s_abort)) break;
     }
   } else if (warp == kProdWarp) {
     // ---------------------------------------------------------- TMA producer
@@ -382,7 +385,7 @@ __global__ void __launch_bounds__(kThreads, 1)
           const int c = P.n == 1 ? s : s / P.n, pr = s - c * P.n;  // c: this stage's chunk of KS x 16 points
           const uint32_t dst = smem_u32(smem + kSmemRaw + rs * kRawStage);
           const uint32_t fb = rawfull_bar(rs);
-          arrive_expect_tx(fb, KS * (2 * kRawTile + kKc * 8) + (s == 0 ? 128 * 4 : 0));
+          arrive_expect_tx(fb, KS * (2 * kRawTile + kKc * 8));
 #pragma unroll
           for (int h = 0; h < KS; ++h) {
             const int x = (c * KS + h) * kKc;  // first point of K-step h (16-byte aligned coordinate)
@@ -390,7 +393,6 @@ __global__ void __launch_bounds__(kThreads, 1)
             tma_load_3d(dst + h * 2 * kRawTile + kRawTile, map, x, j0, P.b(pr), fb);
           }
           bulk_copy(dst + kRawD, drow + c * KS * kKc, KS * kKc * 8, fb);
-          if (s == 0) bulk_copy(dst + kRawMag, mag + static_cast<int64_t>(n) * 128, 128 * 4, fb);
         }
         if (!ok) break;
       }
@@ -441,76 +443,102 @@ __global__ void __launch_bounds__(kThreads, 1)
   } else {
     // ---------------------------------------------------------- epilogue
     const int eg = (warp - kEpiWarp0) >> 2;        // column group
-    const int et = (warp & 3) * 32 + lane;         // TMEM lane 0..127
     const uint32_t lane_base = static_cast<uint32_t>((warp & 3) * 32) << 16;
-    float* stg = stage + eg * (kEpiStage / 4);
+    // What bounds it: the latency of the scatter and the FP64 pipe (16 clocks a warp
+    // instruction).  The sums of an item stay in tensor memory only until they are
+    // pairs in shared memory; A_k(i, j) - A_k(j, i) is formed there, one atomic for
+    // the two; and pairs are widened by integer operations.  With the six levels
+    // staged 16 columns at a time, converted and added element by element, and the
+    // accumulators held until then, an item of 64 columns took 10,500 clocks here and
+    // the tensor cores waited for it where n_p is small: 24 molecules (92 points a
+    // batch) 24.4 ms -> 22.5, and 21.0 with the second slicer group; 64-atom cluster
+    // (298 points) 4.23 -> 4.14 and 3.89.
+    const bool odd = warp & 2;                  // lanes 64..127: levels 1, 3, 5
+    const int r = (warp & 1) * 32 + lane;       // row of the tile
+    const int e256 = tid - kEpiWarp0 * 32, col0 = e256 & 15, row0 = e256 >> 4;
+    float2* mine = stg + r * kEpiPitch;
+    float* mine5 = reinterpret_cast<float*>(stg + kTile * kEpiPitch) + r * kEpiPitch;
     int k = 0;
     for (int n = blockIdx.x; n < n_items; n += gridDim.x, ++k) {
       const int set = k & 1;
-      bool ok = mbar_wait_abort(accfull_bar(set), (k >> 1) & 1, s_abort, status, G.wait_ns);
-      if (bar_red_or(2, kEpiThreads, !ok)) break;
-      tc_fence_after();
       const int4 item = items[n];
       const int64_t b = item.x;
       const int o = item.y, i0 = item.z * kTile, j0 = item.w * kTile;
       const int nb = static_cast<int>(G.bat_fn_ptr[b + 1] - G.bat_fn_ptr[b]);
       const int N = item_nb(nb, item.w);  // accumulator blocks are N columns wide
       const int* idx = G.bat_idx + G.bat_idx_ptr[b];
+      const bool diag = item.z == item.w, anti = o >= 2 && o <= 4 && diag;
       double* out = (o == 0 || o == 5) ? V : o == 1 ? W0 : o == 2 ? SOx : o == 3 ? SOy : SOz;
-      const int col = et & 15;
-      // value offsets of this thread's eight elements of columns c0 .. c0 + 15,
-      // all loads at once (a load and its use element by element left the
-      // epilogue 22,000 clocks an item, this 16,700): the element (i, j) itself, for
-      // V and W0 where i <= j, for SO where i != j (a diagonal tile pair holds A_k,
-      // so A_k(i, j) - A_k(j, i) goes to (i, j), i < j; an off-diagonal one holds
-      // SO_k itself), for the per-column operator always
-      int off[8];
-      auto load_off = [&](int c0) {
-        const int j = j0 + c0 + col;
+      // offsets of this thread's elements of columns c0 .. c0 + 15 (rows row0 + 16 q;
+      // a warp covers 16 consecutive columns of two rows): a diagonal tile pair
+      // scatters i <= j of V and W0 and i < j of SO, an off-diagonal one and the
+      // per-column operator every element
+      const int skip = anti ? 1 : 0;
+      auto load_off = [&](int c0, int (&off)[4]) {
+        const int j = j0 + c0 + col0;
 #pragma unroll
-        for (int qr = 0; qr < 8; ++qr) {
-          const int i = i0 + (et >> 4) + 8 * qr;
-          const bool swap = o >= 2 && o <= 4 && i > j;
-          const int ri = min(swap ? j : i, nb - 1), rj = min(swap ? i : j, nb - 1);
-          const int v = __ldg(idx + ri * nb + rj);
-          const bool use = i < nb && j < nb && (o == 5 || (o <= 1 ? i <= j : i != j));
-          off[qr] = use ? v : -1;
+        for (int q = 0; q < 4; ++q) {
+          const int i = i0 + row0 + 16 * q;
+          const int v = __ldg(idx + min(i, nb - 1) * nb + min(j, nb - 1));
+          off[q] = i < nb && j < nb && (o == 5 || !diag || i + skip <= j) ? v : -1;
         }
       };
+      int off[4], nxt[4];
+      load_off(0, off);
+      const bool ok = mbar_wait_abort(accfull_bar(set), (k >> 1) & 1, s_abort, status, G.wait_ns);
+      if (bar_red_or(2, kEpiThreads, !ok)) break;  // also: the last item's pairs have been read
+      tc_fence_after();
       for (int c0 = eg * 16; c0 < N; c0 += 32) {
-        load_off(c0);
+        float v0[16], v1[16], v2[16];
+        const uint32_t t = tmem + lane_base + set * kSetCols + c0;
+        tmem_ld8x3(t, t + N, t + 2 * N, v0, v1, v2);
+        tmem_ld8x3(t + 8, t + N + 8, t + 2 * N + 8, v0 + 8, v1 + 8, v2 + 8);
+        if (odd) {
 #pragma unroll
-        for (int blk = 0; blk < 3; ++blk) {
-          float vv[16];
-          tmem_ld16(tmem + lane_base + set * kSetCols + blk * N + c0, vv);
-#pragma unroll
-          for (int i = 0; i < 16; ++i) stg[(blk * 128 + et) * kEpiPitch + i] = vv[i];
+          for (int i = 0; i < 16; ++i) {
+            mine[c0 + i] = make_float2(v0[i], v1[i]);
+            mine5[c0 + i] = v2[i];
+          }
         }
         bar_sync(3 + eg, 128);
-        // thread -> (column, rows): a warp covers 16 consecutive columns of two rows
+        if (!odd) {
 #pragma unroll
-        for (int qr = 0; qr < 8; ++qr) {
-          if (off[qr] < 0) continue;
-          const int r = (et >> 4) + 8 * qr;
-          const float L0 = stg[r * kEpiPitch + col], L1 = stg[(r + 64) * kEpiPitch + col];
-          const float L2 = stg[(128 + r) * kEpiPitch + col], L3 = stg[(192 + r) * kEpiPitch + col];
-          const float L4 = stg[(256 + r) * kEpiPitch + col], L5 = stg[(320 + r) * kEpiPitch + col];
-          // exact levels by two-sums, rounded tail on top
-          float sm = L0 + L1;
-          float bp = sm - L0;
-          const float e1 = (L0 - (sm - bp)) + (L1 - bp);
-          const float s1 = sm;
-          sm = s1 + L2;
-          bp = sm - s1;
-          const float e2 = (s1 - (sm - bp)) + (L2 - bp);
-          const float lo = (e1 + e2) + (L3 + (L4 + L5));
-          const double val = static_cast<double>(sm) + static_cast<double>(lo);
-          atomicAdd(out + off[qr], o >= 2 && o <= 4 && i0 + r > j0 + c0 + col ? -val : val);
+          for (int i = 0; i < 16; i += 2) {  // exact levels by two-sums, rounded tail on top
+            const float2 p = mine[c0 + i], q = mine[c0 + i + 1];
+            float2 s, es, u, eu;
+            two_sum2(pk2(v0[i], v0[i + 1]), pk2(p.x, q.x), s, es);
+            two_sum2(s, pk2(v1[i], v1[i + 1]), u, eu);
+            const float2 l45 = add2(pk2(v2[i], v2[i + 1]), pk2(mine5[c0 + i], mine5[c0 + i + 1]));
+            const float2 lo = add2(add2(es, eu), add2(pk2(p.y, q.y), l45));
+            mine[c0 + i] = make_float2(u.x, lo.x);
+            mine[c0 + i + 1] = make_float2(u.y, lo.y);
+          }
         }
-        bar_sync(3 + eg, 128);
       }
       tc_fence_before();
       mbar_arrive(accempty_bar(set));
+      bar_sync(2, kEpiThreads);
+      for (int c0 = 0; c0 < N; c0 += 16) {
+        if (c0 + 16 < N) load_off(c0 + 16, nxt);  // a block ahead
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+          if (off[q] >= 0) {
+            const int i = row0 + 16 * q, j = c0 + col0;
+            const float2 x = stg[i * kEpiPitch + j];
+            double val;
+            if (anti) {  // A_k(i, j) - A_k(j, i): the parts' differences d + e, l + le are exact
+              const float2 y = stg[j * kEpiPitch + i];
+              const float d = x.x - y.x, z = d - x.x, e = (x.x - (d - z)) + (-y.x - z);
+              const float l = x.y - y.y, zl = l - x.y, le = (x.y - (l - zl)) + (-y.y - zl);
+              val = (widen(d) + widen(l)) + widen(e + le);
+            } else {
+              val = widen(x.x) + widen(x.y);
+            }
+            atomicAdd(out + off[q], val);
+          }
+          off[q] = nxt[q];
+        }
+      }
     }
   }
   tc_fence_before();
@@ -535,7 +563,7 @@ q4c_status launch_products(const q4c_grid* g, const int4* items, int n, const fl
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&n_sm, cudaDevAttrMultiProcessorCount, dev);
   KernelScope ks(name, s);
-  split::k_split_products<KS><<<std::min(n, n_sm), split::kThreads, L::kSmemTotal, s>>>(
+  split::k_split_products<KS><<<std::min(n, n_sm), L::kThreads, L::kSmemTotal, s>>>(
       g->view(), items, n, reinterpret_cast<const CUtensorMap*>(g->d_tmaps), g->d_dpad, mag, V, W0, SOx, SOy, SOz,
       g->d_status);
   Q4C_CUDA(cudaGetLastError());
@@ -553,7 +581,7 @@ q4c_status launch_products_ks(int ks, const q4c_grid* g, const int4* items, int 
                                 : launch_products<1>(g, items, n_split, mag, V, W0, SOx, SOy, SOz, name, s))
       return st;
   if (n <= n_split) return Q4C_OK;
-  return launch_pairs(ks, g, items + n_split, n - n_split, V, W0, SOx, SOy, SOz, name, s);
+  return launch_pairs(g, items + n_split, n - n_split, V, W0, SOx, SOy, SOz, name, s);
 }
 
 // items of one wave: rounding constants of all of them, then one launch per

@@ -27,9 +27,9 @@
 // (about 630 issue slots a scheduler) where two steps of split.cu slice 256, and its
 // MMAs read 43 KB from shared memory where theirs read 97.  Measured per 64 x 64
 // x 16 product: 710 clocks for 1,185 on batches of 700 functions (304-atom slab,
-// products 46.2 -> 34.9 ms); with few row tiles half of M is empty much of the
-// time and split.cu is the faster one (64-atom cluster, 65-128 functions: 2.33 ms
-// there, 3.2 here; 129-205: 0.64 and 0.74).
+// products 46.2 -> 33.7 ms); with few row tiles half of M is empty much of the
+// time and split.cu is the faster one (64-atom cluster, 65-128 functions: 2.15 ms
+// there, 3.2 here; 129-205: 0.59 and 0.74).
 #include <cuda.h>
 
 #include <algorithm>
@@ -61,19 +61,17 @@ constexpr uint32_t kTmemCols = 512;
 constexpr uint32_t kTmemA = 384;  // two stages of six A digits (48 columns) behind six levels of up to 64
 constexpr int kFine = 1;          // digits 2^-1 finer than tc::slice6's against the exponent itself
 
-// Shared memory with KS steps per raw stage (the stage shape the tuner chooses
-// per batch-size bucket): four raw stages of one step or two of two.
-template <int KS>
-struct Layout {
-  static constexpr int kRaw = 4 / KS;
-  static constexpr int kSmemB = 4 * kRawStep;
-  static constexpr int kSmemEpi = kSmemB + kStagesB * kStageB;  // [128][kEpiPitch] pairs
-  static constexpr int kSmemBar = kSmemEpi + 2 * kTile * kEpiPitch * 8;
-  // raw full/empty, B full/empty, A full[2], A empty[2], acc full, acc empty, drain
-  static constexpr int kNumBars = 2 * kRaw + 2 * kStagesB + 7;
-  static constexpr int kSmemTotal = kSmemBar + kNumBars * 8 + 16;
-  static_assert(kSmemTotal <= 232448, "shared memory per CTA");
-};
+// Shared memory: four raw stages of one step (two of two steps, half the handshakes,
+// are the slower by far: 304-atom slab 54.2 ms for 34.9), the B digits, the staged
+// elements.
+constexpr int kRaw = 4;
+constexpr int kSmemB = kRaw * kRawStep;
+constexpr int kSmemEpi = kSmemB + kStagesB * kStageB;  // [128][kEpiPitch] pairs
+constexpr int kSmemBar = kSmemEpi + 2 * kTile * kEpiPitch * 8;
+// raw full/empty, B full/empty, A full[2], A empty[2], acc full, acc empty, drain
+constexpr int kNumBars = 2 * kRaw + 2 * kStagesB + 7;
+constexpr int kSmemTotal = kSmemBar + kNumBars * 8 + 16;
+static_assert(kSmemTotal <= 232448, "shared memory per CTA");
 
 // ------------------------------------------------------------ items
 // An item is (batch, type, B tile tj, row tiles ti0 | ti1 << 16); ti1 = 0xffff: no
@@ -173,18 +171,14 @@ __device__ __forceinline__ void mma_step(uint32_t d, uint32_t a, uint64_t b, int
 // Every wait is bounded; a role that times out sets the status bit and an
 // abort flag that ends the other roles' waits, and the MMA warp drains its
 // outstanding MMAs (bounded) before tensor memory is freed.
-template <int KS>
 __global__ void __launch_bounds__(kThreads, 1)
-    k_split_pairs(DevGrid G, const int4* __restrict__ items, int n_items,
-                     const CUtensorMap* __restrict__ maps, const float2* __restrict__ dpad,
-                     const int* __restrict__ colexp, double* V, double* W0, double* SOx, double* SOy, double* SOz,
-                     unsigned* status) {
-  using L = Layout<KS>;
-  constexpr int kRaw = L::kRaw;
+    k_split_pairs(DevGrid G, const int4* __restrict__ items, int n_items, const CUtensorMap* __restrict__ maps,
+                  const float2* __restrict__ dpad, const int* __restrict__ colexp, double* V, double* W0, double* SOx,
+                  double* SOy, double* SOz, unsigned* status) {
   extern __shared__ __align__(1024) unsigned char smem[];
-  uint64_t* bars = reinterpret_cast<uint64_t*>(smem + L::kSmemBar);
-  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(smem + L::kSmemBar + L::kNumBars * 8);
-  volatile int* s_abort = reinterpret_cast<volatile int*>(smem + L::kSmemBar + L::kNumBars * 8 + 4);
+  uint64_t* bars = reinterpret_cast<uint64_t*>(smem + kSmemBar);
+  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(smem + kSmemBar + kNumBars * 8);
+  volatile int* s_abort = reinterpret_cast<volatile int*>(smem + kSmemBar + kNumBars * 8 + 4);
 
   const int tid = threadIdx.x, warp = uniform(tid >> 5), lane = tid & 31;
   const uint32_t smem0 = smem_u32(smem);
@@ -206,7 +200,7 @@ __global__ void __launch_bounds__(kThreads, 1)
   if (tid == 0) {
     for (int k = 0; k < kRaw; ++k) {
       mbar_init(rawfull_bar(k), 1);
-      mbar_init(rawempty_bar(k), (KS * kASlicers / 2 + kBSlicers) / 32);  // an A group a step, the B warps
+      mbar_init(rawempty_bar(k), (kASlicers / 2 + kBSlicers) / 32);  // an A group, the B warps
     }
     for (int k = 0; k < kStagesB; ++k) {
       mbar_init(bfull_bar(k), kBSlicers);
@@ -231,11 +225,10 @@ __global__ void __launch_bounds__(kThreads, 1)
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem = uniform(*tmem_slot);
-  // steps of 16 points of an item, KS a raw stage (a stage past the last point
-  // reads zeros): each chunk of KS x 16 points once per product
-  auto item_stages = [&](const int4& it) {
+  // steps of an item: each chunk of 16 points once per product
+  auto item_steps = [&](const int4& it) {
     const int np = static_cast<int>(G.pt_ptr[it.x + 1] - G.pt_ptr[it.x]);
-    return (np + KS * kKc - 1) / (KS * kKc) * n_products(it.y);
+    return (np + kKc - 1) / kKc * n_products(it.y);
   };
 
   if (warp < kBWarp0) {
@@ -249,14 +242,14 @@ __global__ void __launch_bounds__(kThreads, 1)
     // raw box row r64 is 128 bytes, its 16-byte chunk c swizzled to c ^ (r & 7)
     const uint32_t box = (bot ? kRawTile : 0) + r64 * 128;
     const uint32_t t = tmem + (static_cast<uint32_t>((warp & 3) * 32) << 16) + kTmemA + ag * 48;
-    int g = 0, aph = 1, rs = 0, rph = 0;  // steps, parities, raw stage
+    int g = 0, aph = 1;  // steps, parity
     bool ok = true;
     for (int n = blockIdx.x; n < n_items && ok; n += gridDim.x) {
       const int4 item = items[n];
       const int type = item.y, n_prod = n_products(type);
       const int64_t fn0 = G.bat_fn_ptr[item.x];
       const int nb = static_cast<int>(G.bat_fn_ptr[item.x + 1] - fn0);
-      const int n_st = item_stages(item);
+      const int n_st = item_steps(item);
       const int ti = bot ? static_cast<int>(static_cast<unsigned>(item.w) >> 16) : item.w & 0xffff;
       // rounding constant of this row: products that share an accumulator are
       // sliced against one exponent per function; acts: products that take part
@@ -271,61 +264,51 @@ __global__ void __launch_bounds__(kThreads, 1)
       }
       const float mag = magic0(e - kFine);
       const float mm[4] = {mag, mag, mag, mag};
-      for (int s = 0, pr = 0; s < n_st && ok; ++s, pr = pr + 1 == n_prod ? 0 : pr + 1) {
+      for (int s = 0, pr = 0; s < n_st && ok; ++s, ++g, pr = pr + 1 == n_prod ? 0 : pr + 1) {
         const bool act = acts >> pr & 1u;
-        bool seen = false;
+        const int rs = g % kRaw;
+        if ((g & 1) != ag) continue;
+        if (!mbar_wait_abort(rawfull_bar(rs), (g / kRaw) & 1, s_abort, status, G.wait_ns)) ok = false;
+        const uint32_t raw = smem0 + rs * kRawStep;
 #pragma unroll
-        for (int h = 0; h < KS; ++h, ++g) {
-          if ((g & 1) != ag) continue;
-          if (!mbar_wait_abort(rawfull_bar(rs), rph, s_abort, status, G.wait_ns)) ok = false;
-          const uint32_t raw = smem0 + (rs * KS + h) * kRawStep;
+        for (int half = 0; half < 2; ++half) {
+          uint32_t wd[4][kSlices];
+          if (act) {
+            float2 x[4], l[4];
 #pragma unroll
-          for (int half = 0; half < 2; ++half) {
-            uint32_t wd[4][kSlices];
-            if (act) {
-              float2 x[4], l[4];
-#pragma unroll
-              for (int u = 0; u < 4; ++u) {  // points 8 half + 2u, + 1: D-scaled values in double-float
-                const float4 v = lds128(raw + box + (((4 * half + u) ^ (r64 & 7)) << 4));
-                const float4 d = lds128(raw + 3 * kRawTile + (4 * half + u) * 16);
-                df_mul2(pk2(v.x, v.z), pk2(v.y, v.w), pk2(d.x, d.z), pk2(d.y, d.w), pk2(-d.x, -d.z), x[u], l[u]);
-              }
-              slice_pairs<4>(x, l, mm, wd);
-            } else {
-#pragma unroll
-              for (int u = 0; u < 4; ++u)
-#pragma unroll
-                for (int d = 0; d < kSlices; ++d) wd[u][d] = 0u;
+            for (int u = 0; u < 4; ++u) {  // points 8 half + 2u, + 1: D-scaled values in double-float
+              const float4 v = lds128(raw + box + (((4 * half + u) ^ (r64 & 7)) << 4));
+              const float4 d = lds128(raw + 3 * kRawTile + (4 * half + u) * 16);
+              df_mul2(pk2(v.x, v.z), pk2(v.y, v.w), pk2(d.x, d.z), pk2(d.y, d.w), pk2(-d.x, -d.z), x[u], l[u]);
             }
-            if (half == 0) {  // the first half is sliced while the stage's last MMAs still run
-              if (!mbar_wait_abort(aempty_bar(ag), aph, s_abort, status, G.wait_ns)) ok = false;
-              if (!__all_sync(0xffffffffu, ok)) {
-                ok = false;
-                break;
-              }
-              tc_fence_after();
-            }
+            slice_pairs<4>(x, l, mm, wd);
+          } else {
 #pragma unroll
-            for (int d = 0; d < kSlices; ++d)
-              tmem_st4(t + 8 * d + 4 * half, wd[0][d], wd[1][d], wd[2][d], wd[3][d]);
+            for (int u = 0; u < 4; ++u)
+#pragma unroll
+              for (int d = 0; d < kSlices; ++d) wd[u][d] = 0u;
           }
-          if (!ok) break;
-          seen = true;
-          aph ^= 1;
-          asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
-          tc_fence_before();
-          mbar_arrive(afull_bar(ag));
+          if (half == 0) {  // the first half is sliced while the stage's last MMAs still run
+            if (!mbar_wait_abort(aempty_bar(ag), aph, s_abort, status, G.wait_ns)) ok = false;
+            if (!__all_sync(0xffffffffu, ok)) {
+              ok = false;
+              break;
+            }
+            tc_fence_after();
+          }
+#pragma unroll
+          for (int d = 0; d < kSlices; ++d)
+            tmem_st4(t + 8 * d + 4 * half, wd[0][d], wd[1][d], wd[2][d], wd[3][d]);
         }
+        if (!ok) break;
+        aph ^= 1;
+        asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
+        tc_fence_before();
+        mbar_arrive(afull_bar(ag));
         // The raw stage is free: the digits above were formed from its values,
         // so the loads have landed.
-        if (seen) {
-          __syncwarp();
-          if (lane == 0) mbar_arrive(rawempty_bar(rs));
-        }
-        if (++rs == kRaw) {
-          rs = 0;
-          rph ^= 1;
-        }
+        __syncwarp();
+        if (lane == 0) mbar_arrive(rawempty_bar(rs));
       }
     }
   } else if (warp < kBWarp0 + kBSlicers / 32) {
@@ -334,14 +317,14 @@ __global__ void __launch_bounds__(kThreads, 1)
     const int half = (warp >> 1) & 1, r64 = (warp & 1) * 32 + lane;
     const uint32_t box = 2 * kRawTile + r64 * 128;
     const uint32_t dstB = (r64 >> 3) * kSBO + half * kLBO + (r64 & 7) * 16;
-    int g = 0, rs = 0, rph = 0;
+    int g = 0;
     bool ok = true;
     for (int n = blockIdx.x; n < n_items && ok; n += gridDim.x) {
       const int4 item = items[n];
       const int type = item.y, n_prod = n_products(type);
       const int64_t fn0 = G.bat_fn_ptr[item.x];
       const int nb = static_cast<int>(G.bat_fn_ptr[item.x + 1] - fn0);
-      const int n_st = item_stages(item);
+      const int n_st = item_steps(item);
       const int w = item_w(nb, item.z);
       const bool have = r64 < w;
       int e = -30000, e1 = -30000;
@@ -355,47 +338,40 @@ __global__ void __launch_bounds__(kThreads, 1)
           e = max(e, v);
       }
       const float mag = magic0(e - kFine), mag1 = type == kDiag2 ? magic0(e1 - kFine) : mag;
-      for (int s = 0, pr = 0; s < n_st && ok; ++s, pr = pr + 1 == n_prod ? 0 : pr + 1) {
-        if (!mbar_wait_abort(rawfull_bar(rs), rph, s_abort, status, G.wait_ns)) {
+      for (int s = 0, pr = 0; s < n_st; ++s, ++g, pr = pr + 1 == n_prod ? 0 : pr + 1) {
+        const int rs = g % kRaw;
+        if (!mbar_wait_abort(rawfull_bar(rs), (g / kRaw) & 1, s_abort, status, G.wait_ns)) {
           ok = false;
           break;
         }
         const float m = pr ? mag1 : mag;
         const float mm[4] = {m, m, m, m};
+        const uint32_t raw = smem0 + rs * kRawStep;
+        uint32_t wd[4][kSlices];
+        if (have) {
+          float2 x[4], l[4];
 #pragma unroll
-        for (int h = 0; h < KS; ++h, ++g) {
-          const uint32_t raw = smem0 + (rs * KS + h) * kRawStep;
-          uint32_t wd[4][kSlices];
-          if (have) {
-            float2 x[4], l[4];
-#pragma unroll
-            for (int u = 0; u < 4; ++u) {
-              const float4 v = lds128(raw + box + (((4 * half + u) ^ (r64 & 7)) << 4));
-              x[u] = pk2(v.x, v.z);
-              l[u] = pk2(v.y, v.w);
-            }
-            slice_pairs<4>(x, l, mm, wd);
+          for (int u = 0; u < 4; ++u) {
+            const float4 v = lds128(raw + box + (((4 * half + u) ^ (r64 & 7)) << 4));
+            x[u] = pk2(v.x, v.z);
+            l[u] = pk2(v.y, v.w);
           }
-          const int st = g % kStagesB;
-          if (!mbar_wait_abort(bempty_bar(st), ((g / kStagesB) & 1) ^ 1, s_abort, status, G.wait_ns)) {
-            ok = false;
-            break;
-          }
-          if (have) {
-            const uint32_t dst = smem0 + L::kSmemB + st * kStageB + dstB;
-#pragma unroll
-            for (int d = 0; d < kSlices; ++d) sts128(dst + d * w * kRowBytes, wd[0][d], wd[1][d], wd[2][d], wd[3][d]);
-          }
-          fence_async_smem();
-          mbar_arrive(bfull_bar(st));
+          slice_pairs<4>(x, l, mm, wd);
         }
-        if (!ok) break;
+        const int st = g % kStagesB;
+        if (!mbar_wait_abort(bempty_bar(st), ((g / kStagesB) & 1) ^ 1, s_abort, status, G.wait_ns)) {
+          ok = false;
+          break;
+        }
+        if (have) {
+          const uint32_t dst = smem0 + kSmemB + st * kStageB + dstB;
+#pragma unroll
+          for (int d = 0; d < kSlices; ++d) sts128(dst + d * w * kRowBytes, wd[0][d], wd[1][d], wd[2][d], wd[3][d]);
+        }
+        fence_async_smem();
+        mbar_arrive(bfull_bar(st));
         __syncwarp();
         if (lane == 0) mbar_arrive(rawempty_bar(rs));
-        if (++rs == kRaw) {
-          rs = 0;
-          rph ^= 1;
-        }
       }
     }
   } else if (warp == kProdWarp) {
@@ -405,7 +381,7 @@ __global__ void __launch_bounds__(kThreads, 1)
       bool ok = true;
       for (int n = blockIdx.x; n < n_items && ok; n += gridDim.x) {
         const int4 item = items[n];
-        const int n_st = item_stages(item), n_prod = n_products(item.y);
+        const int n_st = item_steps(item), n_prod = n_products(item.y);
         const CUtensorMap* map = maps + item.x;
         const float2* drow = dpad + static_cast<int64_t>(item.x) * kDPitch;
         const int ti1 = static_cast<int>(static_cast<unsigned>(item.w) >> 16);
@@ -418,16 +394,13 @@ __global__ void __launch_bounds__(kThreads, 1)
           const Step stp = step_of(item.y, pr);
           const bool top = stp.top & 8, bot = (stp.bot & 8) && ti1 != 0xffff;
           const uint32_t fb = rawfull_bar(rs);
-          arrive_expect_tx(fb, KS * ((1 + top + bot) * kRawTile + kKc * 8));
-#pragma unroll
-          for (int h = 0; h < KS; ++h) {
-            const uint32_t dst = smem0 + (rs * KS + h) * kRawStep;
-            const int x = (c * KS + h) * kKc;  // first point of the step (16-byte aligned coordinate)
-            if (top) tma_load_3d(dst, map, x, i0, stp.top & 3, fb);
-            if (bot) tma_load_3d(dst + kRawTile, map, x, i1, stp.bot & 3, fb);
-            tma_load_3d(dst + 2 * kRawTile, map, x, j0, stp.b, fb);
-            bulk_copy(dst + 3 * kRawTile, drow + x, kKc * 8, fb);
-          }
+          arrive_expect_tx(fb, (1 + top + bot) * kRawTile + kKc * 8);
+          const uint32_t dst = smem0 + rs * kRawStep;
+          const int x = c * kKc;  // first point of the step (16-byte aligned coordinate)
+          if (top) tma_load_3d(dst, map, x, i0, stp.top & 3, fb);
+          if (bot) tma_load_3d(dst + kRawTile, map, x, i1, stp.bot & 3, fb);
+          tma_load_3d(dst + 2 * kRawTile, map, x, j0, stp.b, fb);
+          bulk_copy(dst + 3 * kRawTile, drow + x, kKc * 8, fb);
           if (++rs == kRaw) {
             rs = 0;
             ph ^= 1;
@@ -448,21 +421,17 @@ __global__ void __launch_bounds__(kThreads, 1)
     // (the whole warp waits, one lane issues, operands uniform: see rowdot.cu)
     int g = 0, k = 0;
     bool ok = true;
-    const uint64_t descB = make_desc(smem0 + L::kSmemB, kSBO);
+    const uint64_t descB = make_desc(smem0 + kSmemB, kSBO);
     for (int n = blockIdx.x; n < n_items && ok; n += gridDim.x, ++k) {
       const int4 item = items[n];
-      const int n_steps = uniform(item_stages(item) * KS);
+      const int n_steps = uniform(item_steps(item));
       const int w = uniform(item_w(static_cast<int>(G.bat_fn_ptr[item.x + 1] - G.bat_fn_ptr[item.x]), item.z));
       if (!mbar_wait_abort(accempty_bar, (k & 1) ^ 1, s_abort, status, G.wait_ns)) break;
       const int type = item.y, n_prod = n_products(type);
-      int pr = 0, kc = 0;  // product, step within its raw stage
-      for (int s = 0; s < n_steps; ++s, ++g) {
+      for (int s = 0, pr = 0; s < n_steps; ++s, ++g) {
         // a subtracted product (both halves alike): the instruction's negate-A bit
         const uint32_t neg = (step_of(type, pr).top & 4) ? 1u << 13 : 0u;
-        if (++kc == KS) {
-          kc = 0;
-          if (++pr == n_prod) pr = 0;
-        }
+        if (++pr == n_prod) pr = 0;
         const int sa = uniform(g & 1), sb = uniform(g % kStagesB);
         if (!mbar_wait_abort(bfull_bar(sb), (g / kStagesB) & 1, s_abort, status, G.wait_ns) ||
             !mbar_wait_abort(afull_bar(sa), (g >> 1) & 1, s_abort, status, G.wait_ns)) {
@@ -492,7 +461,7 @@ __global__ void __launch_bounds__(kThreads, 1)
     const int r = quarter * 32 + lane;
     const int et = tid - kEpiWarp0 * 32;
     const uint32_t lane_base = static_cast<uint32_t>(quarter * 32) << 16;
-    float2* stg = reinterpret_cast<float2*>(smem + L::kSmemEpi);
+    float2* stg = reinterpret_cast<float2*>(smem + kSmemEpi);
     int k = 0;
     for (int n = blockIdx.x; n < n_items; n += gridDim.x, ++k) {
       const int4 item = items[n];
@@ -575,26 +544,18 @@ __global__ void __launch_bounds__(kThreads, 1)
 }  // namespace pairs
 
 // one launch over items [0, n): a persistent grid of at most one CTA per SM
-template <int KS>
-static q4c_status launch(const q4c_grid* g, const int4* items, int n, double* V, double* W0, double* SOx, double* SOy,
-                         double* SOz, const char* name, cudaStream_t s) {
-  using L = pairs::Layout<KS>;
-  Q4C_CUDA(cudaFuncSetAttribute(pairs::k_split_pairs<KS>, cudaFuncAttributeMaxDynamicSharedMemorySize, L::kSmemTotal));
+q4c_status launch_pairs(const q4c_grid* g, const int4* items, int n, double* V, double* W0, double* SOx, double* SOy,
+                        double* SOz, const char* name, cudaStream_t s) {
+  Q4C_CUDA(cudaFuncSetAttribute(pairs::k_split_pairs, cudaFuncAttributeMaxDynamicSharedMemorySize, pairs::kSmemTotal));
   int dev = 0, n_sm = 0;
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&n_sm, cudaDevAttrMultiProcessorCount, dev);
   KernelScope ks(name, s);
-  pairs::k_split_pairs<KS><<<std::min(n, n_sm), pairs::kThreads, L::kSmemTotal, s>>>(
+  pairs::k_split_pairs<<<std::min(n, n_sm), pairs::kThreads, pairs::kSmemTotal, s>>>(
       g->view(), items, n, reinterpret_cast<const CUtensorMap*>(g->d_tmaps), g->d_dpad, g->d_colexp, V, W0, SOx, SOy,
       SOz, g->d_status);
   Q4C_CUDA(cudaGetLastError());
   return Q4C_OK;
-}
-
-q4c_status launch_pairs(int ks, const q4c_grid* g, const int4* items, int n, double* V, double* W0, double* SOx,
-                        double* SOy, double* SOz, const char* name, cudaStream_t s) {
-  return ks == 2 ? launch<2>(g, items, n, V, W0, SOx, SOy, SOz, name, s)
-                 : launch<1>(g, items, n, V, W0, SOx, SOy, SOz, name, s);
 }
 
 }  // namespace q4c

@@ -292,13 +292,14 @@ __device__ __forceinline__ void tmem_ld8x6(uint32_t t, uint32_t step, float (*v)
 }
 
 // x as a double on the integer pipes (the FP64 units, where a conversion would
-// run, take 16 clocks a warp instruction)
+// run, take 16 clocks a warp instruction), without a branch (one for zeros and
+// subnormals ran the conversion for a warp with any zero: 24 molecules, products
+// 22.2 ms against 21.0)
 __device__ __forceinline__ double widen(float x) {
-  const uint32_t u = __float_as_uint(x);
-  const uint32_t e = (u >> 23) & 0xffu;
-  if (e == 0u || e == 255u) return static_cast<double>(x);  // zero, subnormal, infinite, NaN
-  return __hiloint2double(static_cast<int>((u & 0x80000000u) | (((u & 0x7fffffffu) >> 3) + 0x38000000u)),
-                          static_cast<int>(u << 29));
+  const bool small = (__float_as_uint(x) & 0x7fffffffu) < 0x800000u;  // subnormal or zero: scaled by 2^32 first
+  const uint32_t u = __float_as_uint(small ? x * 0x1p32f : x), a = u & 0x7fffffffu;
+  const uint32_t bias = a >= 0x7f800000u ? 0x70000000u : small ? 0x36000000u : 0x38000000u;  // infinite and NaN stay so
+  return a == 0u ? 0.0 : __hiloint2double(static_cast<int>((u & 0x80000000u) | ((a >> 3) + bias)), static_cast<int>(u << 29));
 }
 
 // ------------------------------------------------------------ slicing
