@@ -240,27 +240,39 @@ __global__ void __launch_bounds__(256, 3) k_products_fp64(DevBasis B, DevGrid G,
 // transposed into their partner (B, A, -T) (negated for SO); a block that is
 // its own partner (A = B, T = 0; role 2) fills i > j from (j, i); role 0
 // blocks are the copy targets.
+// SPINOR: also the spinor blocks of both (k_spinor), from the same read.
+template <bool SPINOR>
 __global__ void k_mirror(const int* __restrict__ blk_row, const int* __restrict__ blk_col,
                          const int* __restrict__ blk_T, const int* __restrict__ blk_role,
                          const int64_t* __restrict__ blk_off, const int* atom_sp, const int* sp_nfn, double* V,
-                         double* W0, double* SOx, double* SOy, double* SOz) {
+                         double* W0, double* SOx, double* SOy, double* SOz, double2* __restrict__ SS) {
   const int q = blockIdx.x;
-  const int role = blk_role[q];
+  const int role = blk_role[q], A = blk_row[q], Bc = blk_col[q];
+  const int64_t o = blk_off[q], oT = role ? blk_off[blk_T[q]] : 0;
   if (role == 0) return;
-  const int A = blk_row[q], Bc = blk_col[q];
   const int nfA = sp_nfn[atom_sp[A]], nfB = sp_nfn[atom_sp[Bc]];
   const bool self = role == 2;
-  const int64_t o = blk_off[q], oT = blk_off[blk_T[q]];
+  auto spinor = [&](int64_t off, int nf, int i, int j, double w, double x, double y, double z) {
+    double2* r0 = SS + 4 * off + static_cast<int64_t>(2 * i) * (2 * nf) + 2 * j;
+    double2* r1 = r0 + 2 * nf;
+    r0[0] = make_double2(w, z);
+    r0[1] = make_double2(y, x);
+    r1[0] = make_double2(-y, x);
+    r1[1] = make_double2(w, -z);
+  };
   for (int e = threadIdx.x; e < nfA * nfB; e += blockDim.x) {
     const int i = e / nfB, j = e - i * nfB;
-    if (self && i <= j) continue;
-    const int64_t src = self ? o + static_cast<int64_t>(j) * nfB + i : o + e;
-    const int64_t dst = self ? o + e : oT + static_cast<int64_t>(j) * nfA + i;
-    V[dst] = V[src];
-    W0[dst] = W0[src];
-    SOx[dst] = -SOx[src];
-    SOy[dst] = -SOy[src];
-    SOz[dst] = -SOz[src];
+    if (self && i > j) continue;
+    const double v = V[o + e], w = W0[o + e], x = SOx[o + e], y = SOy[o + e], z = SOz[o + e];
+    if (SPINOR) spinor(o, nfB, i, j, w, x, y, z);
+    if (self && i == j) continue;
+    const int64_t dst = oT + static_cast<int64_t>(j) * nfA + i;  // oT = o where the block is its own partner
+    V[dst] = v;
+    W0[dst] = w;
+    SOx[dst] = -x;
+    SOy[dst] = -y;
+    SOz[dst] = -z;
+    if (SPINOR) spinor(oT, nfA, j, i, w, -x, -y, -z);
   }
 }
 
@@ -288,13 +300,22 @@ __global__ void k_spinor(const int* __restrict__ blk_row, const int* __restrict_
 q4c_status mirror_and_spinor(const q4c_grid* g, const q4c_matrices* out, cudaStream_t s) {
   const q4c_tables* t = g->tables;
   if (g->n_blocks == 0) return Q4C_OK;
-  {
-  KernelScope ks("mirror", s);
-  k_mirror<<<static_cast<unsigned>(g->n_blocks), 128, 0, s>>>(g->d_blk_row, g->d_blk_col, g->d_blk_T,
-                                                             g->d_blk_role, g->d_blk_off, g->d_atom_sp,
-                                                             t->d_sp_nfn, out->V,
-                                                             out->W0, out->SOx, out->SOy, out->SOz);
+  auto launch = [&](auto kern) {
+    KernelScope ks("mirror", s);
+    kern<<<static_cast<unsigned>(g->n_blocks), 128, 0, s>>>(
+        g->d_blk_row, g->d_blk_col, g->d_blk_T, g->d_blk_role, g->d_blk_off, g->d_atom_sp, t->d_sp_nfn, out->V,
+        out->W0, out->SOx, out->SOy, out->SOz, reinterpret_cast<double2*>(out->spinor_SS));
+  };
+  // The transposed block's spinors leave 32 bytes at a time: with everything in the
+  // L2 cache that is cheaper than a second launch and read (one molecule of 3 atoms:
+  // 8 us for 14; 64-atom cluster, 0.2M elements: 19 us for 29), with a pattern of 19M
+  // elements it is not (304-atom slab: 1.12 ms for 0.85).
+  if (out->spinor_SS && g->nnz <= 1 << 20) {
+    launch(k_mirror<true>);
+    Q4C_CUDA(cudaGetLastError());
+    return Q4C_OK;
   }
+  launch(k_mirror<false>);
   Q4C_CUDA(cudaGetLastError());
   if (out->spinor_SS) {
     KernelScope ks("spinor", s);
