@@ -166,14 +166,15 @@ __host__ __device__ __forceinline__ int jt_chunks(int m, int n_ic, int jt) {
 // The column bound is the largest column bound (k_prepare_blocks) of the blocks
 // (a, c) of column j's centre c over the batch's active centres a, whose
 // functions are exactly the batch's i.
-// What bounds it: the stores (12 bytes an element and matrix; 5 TB/s with the reads
+// What bounds it: the stores (12 bytes an element and matrix; 5.5 TB/s with the reads
 // on batches of 900 functions).  A warp takes units of 8 j x 8 i (32 words of a tile, an
 // element pair each), so a unit's place needs no division and its offsets are read
 // once for all matrices.  One matrix a CTA with offsets and divisions of its own:
-// 24 molecules 6.8 ms -> 4.4, 64-atom cluster 0.60 -> 0.43; the slab's large
-// batches, already at the memory's rate, 12.1 and 12.5.
+// 24 molecules 6.8 ms -> 4.0, 64-atom cluster 0.60 -> 0.39, 304-atom slab 12.1 ->
+// 10.7.  Forty warps an SM with one unit's ten values in flight each: two units a
+// turn 4.4, 0.43 and 12.5 ms at 32 warps, 3.8, 0.38 and 11.6 at 48.
 template <int NM>
-__global__ void __launch_bounds__(256) k_gslice(DevGrid G, int64_t b0, const float2* __restrict__ prep, int64_t nnz,
+__global__ void __launch_bounds__(256, 5) k_gslice(DevGrid G, int64_t b0, const float2* __restrict__ prep, int64_t nnz,
                                                 unsigned present, const float* __restrict__ cm, int64_t cm_total,
                                                 const int* __restrict__ pair_blk, const int64_t* __restrict__ cm_off,
                                                 const int64_t* __restrict__ gsl_off, uint32_t* __restrict__ gsl) {
@@ -218,8 +219,8 @@ __global__ void __launch_bounds__(256) k_gslice(DevGrid G, int64_t b0, const flo
     const int units = (present & ~3u) ? n_ic << sh : n_low;
     uint32_t* oj = out + static_cast<int64_t>(jt) * n_ic * (kBlockB / 4);
     // a warp takes kU units at a time and issues all their loads (addresses
-    // clamped, so that none depends on a condition) before slicing any
-    constexpr int kU = NM > 1 ? 2 : 4;
+    // clamped, conditions the same for the whole warp) before slicing any
+    constexpr int kU = NM > 1 ? 1 : 4;
     for (int u0 = warp; u0 < units; u0 += kU * nwarps) {
       int i_[kU], j_[kU], o0[kU], o1[kU];
 #pragma unroll
@@ -240,25 +241,28 @@ __global__ void __launch_bounds__(256) k_gslice(DevGrid G, int64_t b0, const flo
         o0[u] = ok0[u] ? o0[u] : 0;
         o1[u] = ok1[u] ? o1[u] : 0;
       }
+      float2 x0[NM][kU], x1[NM][kU];
+#pragma unroll
+      for (int m = 0; m < NM; ++m)
+#pragma unroll
+        for (int u = 0; u < kU; ++u) {
+          if (!(present >> m & 1u) || u0 + u * nwarps >= (m < 2 ? n_low : units)) continue;
+          x0[m][u] = __ldg(prep + m * nnz + o0[u]);
+          x1[m][u] = __ldg(prep + m * nnz + o1[u]);
+        }
 #pragma unroll
       for (int m = 0; m < NM; ++m) {
         if (!(present >> m & 1u)) continue;
-        const float2* M = prep + m * nnz;
-        float2 x0[kU], x1[kU];
-#pragma unroll
-        for (int u = 0; u < kU; ++u) {
-          x0[u] = __ldg(M + o0[u]);
-          x1[u] = __ldg(M + o1[u]);
-        }
 #pragma unroll
         for (int u = 0; u < kU; ++u) {
           const int un = u0 + u * nwarps;
           if (un >= (m < 2 ? n_low : units)) break;
           const int j = jt * kTileJ + j_[u];
           const bool a0 = ok0[u] && (m >= 2 || i_[u] <= j), a1 = ok1[u] && (m >= 2 || i_[u] + 1 <= j);
+          const float2 y0 = x0[m][u], y1 = x1[m][u];
           const unsigned mb = sMax[m ? kB - 1 : 0][j_[u]];
           float2 d[kSlices];
-          slice6x2(pk2(a0 ? x0[u].x : 0.f, a1 ? x1[u].x : 0.f), pk2(a0 ? x0[u].y : 0.f, a1 ? x1[u].y : 0.f),
+          slice6x2(pk2(a0 ? y0.x : 0.f, a1 ? y1.x : 0.f), pk2(a0 ? y0.y : 0.f, a1 ? y1.y : 0.f),
                    magic0((mb ? fexp(__uint_as_float(mb)) : -30000) - kFine), d);
           uint32_t* o = oj + m * mstride + (un >> sh) * (kSlices * tw) + ((un & ((1 << sh) - 1)) << 5) + lane;
 #pragma unroll
