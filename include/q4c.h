@@ -409,9 +409,11 @@ Q4C_API q4c_status q4c_scf_pass(const q4c_tables* tables, const q4c_grid* grid, 
  * bucket (the active functions n_b of a batch: <= 32, <= 64, <= 128, more;
  * Q4C_TILE_BUCKETS buckets).  A shape is the number of 16-point K-steps one
  * pipeline stage of the tensor-core kernel carries: 1 (four stages in
- * flight) or 2 (two stages of twice the points, half the handshakes per
- * point); the 64-function tiles and their N width (the functions of the B
- * tile rounded up to 16) follow from the batch.  A new grid uses 1 for every
+ * flight, two groups of warps that slice alternate ones) or 2 (two stages of
+ * twice the points, half the handshakes per point, one group); the 64-function
+ * tiles and their N width (the functions of the B tile rounded up to 16) follow
+ * from the batch.  Batches of more than 256 functions run two row tiles a step
+ * in the one-step shape, whatever their bucket's.  A new grid uses 1 for every
  * bucket.  Not in the paper: a library control of the kernels.
  *
  * q4c_autotune times both shapes on the grid's first wave of batches with
@@ -422,7 +424,7 @@ Q4C_API q4c_status q4c_scf_pass(const q4c_tables* tables, const q4c_grid* grid, 
  * (q4c_integrate, q4c_integrate_columns, q4c_scf_pass) on the grid; results
  * do not depend on it beyond the order of FP64 additions.
  * The density/adjoint kernel (row-dot products over 16-function K-steps)
- * has one such shape per grid, tuned on the same wave with its adjoint; it is
+ * has one such shape per grid (the K-steps whose G' digits one copy brings), tuned on the same wave with its adjoint; it is
  * addressed as bucket Q4C_TILE_BUCKETS below.
  * q4c_grid_tiling reports a bucket: its largest n_b (4096 for the row-dot
  * kernel), the shape in use, the grid's batches in it (all for the row-dot

@@ -21,8 +21,9 @@ constexpr int kDPitch = 352;  // points per batch row of the D = w v table (>= 3
 constexpr int kTileBuckets = 4;
 constexpr int kBucketNb[kTileBuckets] = {32, 64, 128, 1 << 30};
 // batches above this go to the pair kernel (split_pairs.cu), which takes over
-// where pairs of row tiles make up most of the work: at 129-205 functions (64-atom
-// cluster) 0.74 ms against 0.64 in split.cu, at 700 (304-atom slab) 34.9 against 46.2
+// where pairs of row tiles make up most of the work.  Products with the line at
+// 192, 256, 384, 512 functions and nowhere: 304-atom slab (125-2,475 functions) 33.6,
+// 33.7, 33.9, 34.6 and 44.0 ms; 64-atom cluster (up to 205) 3.94 at 192, 3.89 beyond
 constexpr int kPairNb = 256;
 inline int tile_bucket(int64_t nb) {
   int k = 0;

@@ -72,7 +72,7 @@ constexpr uint32_t kSetCols = 256;
 // pipeline stage (the stage shape the tuner chooses per batch-size bucket):
 // KS = 1 keeps four operand and four raw stages and two slicer groups that take
 // alternate stages (one group's waits and loads run beside the other's arithmetic:
-// 64-atom cluster 4.14 ms with one group, 3.84 with two; a group for each operand
+// 64-atom cluster 4.14 ms with one group, 3.89 with two; a group for each operand
 // instead 4.96, the handshakes of a stage doubled); KS = 2 two of each (twice the
 // points per handshake, the same points in flight) and one group (two: 4.55 ms, the
 // ring too shallow for both).

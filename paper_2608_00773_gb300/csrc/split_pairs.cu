@@ -27,7 +27,7 @@
 // (about 630 issue slots a scheduler) where two steps of split.cu slice 256, and its
 // MMAs read 43 KB from shared memory where theirs read 97.  Measured per 64 x 64
 // x 16 product: 710 clocks for 1,185 on batches of 700 functions (304-atom slab,
-// products 46.2 -> 33.7 ms); with few row tiles half of M is empty much of the
+// products 44.0 -> 33.7 ms); with few row tiles half of M is empty much of the
 // time and split.cu is the faster one (64-atom cluster, 65-128 functions: 2.15 ms
 // there, 3.2 here; 129-205: 0.59 and 0.74).
 #include <cuda.h>
@@ -62,7 +62,7 @@ constexpr uint32_t kTmemA = 384;  // two stages of six A digits (48 columns) beh
 constexpr int kFine = 1;          // digits 2^-1 finer than tc::slice6's against the exponent itself
 
 // Shared memory: four raw stages of one step (two of two steps, half the handshakes,
-// are the slower by far: 304-atom slab 54.2 ms for 34.9), the B digits, the staged
+// are the slower by far: 304-atom slab 54.2 ms for 33.7), the B digits, the staged
 // elements.
 constexpr int kRaw = 4;
 constexpr int kSmemB = kRaw * kRawStep;
