@@ -628,7 +628,7 @@ __global__ void __launch_bounds__(kThreads, 1)
     bool more = W.next();
     if (more) load();
     while (more) {
-      if (!mbar_wait_abort(slotempty_bar(slot), ph, s_abort, status, G.wait_ns)) break;
+      if (!mbar_wait_warp(slotempty_bar(slot), ph, s_abort, status, G.wait_ns)) break;
       const uint32_t dst = dst0 + slot * kSlot;
       const bool store = __any_sync(0xffffffffu, live);  // a warp with no point leaves its rows as they are
       const float m = mag;
@@ -748,7 +748,7 @@ __global__ void __launch_bounds__(kThreads, 1)
     const uint32_t t0 = uniform(tmem + set * kSetCols);
     auto see = [&](int e) {  // every entry up to e is in place
       for (; known <= e; ++known)
-        if (!mbar_wait_abort(slotfull_bar(known % kSlots), (known / kSlots) & 1, s_abort, status, G.wait_ns))
+        if (!mbar_wait_warp(slotfull_bar(known % kSlots), (known / kSlots) & 1, s_abort, status, G.wait_ns))
           return false;
       return true;
     };
@@ -763,7 +763,7 @@ __global__ void __launch_bounds__(kThreads, 1)
           }
           continue;
         }
-        if (!mbar_wait_abort(accempty_bar(set), ((k >> 1) & 1) ^ 1, s_abort, status, G.wait_ns)) {
+        if (!mbar_wait_warp(accempty_bar(set), ((k >> 1) & 1) ^ 1, s_abort, status, G.wait_ns)) {
           ok = false;
           break;
         }
@@ -780,7 +780,7 @@ __global__ void __launch_bounds__(kThreads, 1)
         Run R = W.A;
         for (int run = 0; run < 2 && ok; ++run, R = W.B)
           for (int c = 0; c < R.n && ok; c += KS) {
-            if (!mbar_wait_abort(gfull_bar(set, st), ph, s_abort, status, G.wait_ns)) {
+            if (!mbar_wait_warp(gfull_bar(set, st), ph, s_abort, status, G.wait_ns)) {
               ok = false;
               break;
             }
@@ -859,11 +859,8 @@ __global__ void __launch_bounds__(kThreads, 1)
         const int set = k & 1, w = jt_width(I.nb, W.jt);
         have = W.next();
         if (have && busy) load_R(Rn);
-        ok = mbar_wait_abort(accfull_bar(set), (k >> 1) & 1, s_abort, status, G.wait_ns);
-        if (!__all_sync(0xffffffffu, ok)) {
-          ok = false;
-          break;
-        }
+        ok = mbar_wait_warp(accfull_bar(set), (k >> 1) & 1, s_abort, status, G.wait_ns);
+        if (!ok) break;
         tc_fence_after();
         // this group's sum yh + yl, even and odd columns apart (packed
         // instructions: the issue slots are shared with the slicers): per column

@@ -299,7 +299,7 @@ __global__ void __launch_bounds__(Layout<KS>::kThreads, 1)
       for (int s = 0, pr = 0; s < n_steps; ++s, ++g, pr = (pr + 1 == n_prod) ? 0 : pr + 1) {
         if (kGroups > 1 && (g & 1) != grp) continue;
         const int rs = g % kRaw, st = g % kStages;
-        if (!mbar_wait_abort(rawfull_bar(rs), (g / kRaw) & 1, s_abort, status, G.wait_ns)) {
+        if (!mbar_wait_warp(rawfull_bar(rs), (g / kRaw) & 1, s_abort, status, G.wait_ns)) {
           ok = false;
           break;
         }
@@ -322,7 +322,7 @@ __global__ void __launch_bounds__(Layout<KS>::kThreads, 1)
             d23[h] = make_float4(-d23[h].x, -d23[h].y, -d23[h].z, -d23[h].w);
           }
         }
-        if (!mbar_wait_abort(empty_bar(st), ((g / kStages) & 1) ^ 1, s_abort, status, G.wait_ns)) {
+        if (!mbar_wait_warp(empty_bar(st), ((g / kStages) & 1) ^ 1, s_abort, status, G.wait_ns)) {
           ok = false;
           break;
         }
@@ -413,12 +413,12 @@ __global__ void __launch_bounds__(Layout<KS>::kThreads, 1)
       const int n_steps = uniform(item_stages(item));
       const int nbB = uniform(item_nb(static_cast<int>(G.bat_fn_ptr[item.x + 1] - G.bat_fn_ptr[item.x]), item.w));
       const int set = k & 1;
-      if (!mbar_wait_abort(accempty_bar(set), ((k >> 1) & 1) ^ 1, s_abort, status, G.wait_ns)) break;
+      if (!mbar_wait_warp(accempty_bar(set), ((k >> 1) & 1) ^ 1, s_abort, status, G.wait_ns)) break;
       tc_fence_after();
       const uint32_t t0 = uniform(tmem + set * kSetCols);
       for (int s = 0; s < n_steps; ++s, ++g) {
         const int st = uniform(g % kStages);
-        if (!mbar_wait_abort(full_bar(st), (g / kStages) & 1, s_abort, status, G.wait_ns)) {
+        if (!mbar_wait_warp(full_bar(st), (g / kStages) & 1, s_abort, status, G.wait_ns)) {
           ok = false;
           break;
         }
@@ -485,7 +485,7 @@ __global__ void __launch_bounds__(Layout<KS>::kThreads, 1)
       };
       int off[4], nxt[4];
       load_off(0, off);
-      const bool ok = mbar_wait_abort(accfull_bar(set), (k >> 1) & 1, s_abort, status, G.wait_ns);
+      const bool ok = mbar_wait_warp(accfull_bar(set), (k >> 1) & 1, s_abort, status, G.wait_ns);
       if (bar_red_or(2, kEpiThreads, !ok)) break;  // also: the last item's pairs have been read
       tc_fence_after();
       for (int c0 = eg * 16; c0 < N; c0 += 32) {

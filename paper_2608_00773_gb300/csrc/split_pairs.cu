@@ -268,7 +268,10 @@ __global__ void __launch_bounds__(kThreads, 1)
         const bool act = acts >> pr & 1u;
         const int rs = g % kRaw;
         if ((g & 1) != ag) continue;
-        if (!mbar_wait_abort(rawfull_bar(rs), (g / kRaw) & 1, s_abort, status, G.wait_ns)) ok = false;
+        if (!mbar_wait_warp(rawfull_bar(rs), (g / kRaw) & 1, s_abort, status, G.wait_ns)) {
+          ok = false;
+          break;
+        }
         const uint32_t raw = smem0 + rs * kRawStep;
 #pragma unroll
         for (int half = 0; half < 2; ++half) {
@@ -289,8 +292,7 @@ __global__ void __launch_bounds__(kThreads, 1)
               for (int d = 0; d < kSlices; ++d) wd[u][d] = 0u;
           }
           if (half == 0) {  // the first half is sliced while the stage's last MMAs still run
-            if (!mbar_wait_abort(aempty_bar(ag), aph, s_abort, status, G.wait_ns)) ok = false;
-            if (!__all_sync(0xffffffffu, ok)) {
+            if (!mbar_wait_warp(aempty_bar(ag), aph, s_abort, status, G.wait_ns)) {
               ok = false;
               break;
             }
@@ -340,7 +342,7 @@ __global__ void __launch_bounds__(kThreads, 1)
       const float mag = magic0(e - kFine), mag1 = type == kDiag2 ? magic0(e1 - kFine) : mag;
       for (int s = 0, pr = 0; s < n_st; ++s, ++g, pr = pr + 1 == n_prod ? 0 : pr + 1) {
         const int rs = g % kRaw;
-        if (!mbar_wait_abort(rawfull_bar(rs), (g / kRaw) & 1, s_abort, status, G.wait_ns)) {
+        if (!mbar_wait_warp(rawfull_bar(rs), (g / kRaw) & 1, s_abort, status, G.wait_ns)) {
           ok = false;
           break;
         }
@@ -359,7 +361,7 @@ __global__ void __launch_bounds__(kThreads, 1)
           slice_pairs<4>(x, l, mm, wd);
         }
         const int st = g % kStagesB;
-        if (!mbar_wait_abort(bempty_bar(st), ((g / kStagesB) & 1) ^ 1, s_abort, status, G.wait_ns)) {
+        if (!mbar_wait_warp(bempty_bar(st), ((g / kStagesB) & 1) ^ 1, s_abort, status, G.wait_ns)) {
           ok = false;
           break;
         }
@@ -426,15 +428,15 @@ __global__ void __launch_bounds__(kThreads, 1)
       const int4 item = items[n];
       const int n_steps = uniform(item_steps(item));
       const int w = uniform(item_w(static_cast<int>(G.bat_fn_ptr[item.x + 1] - G.bat_fn_ptr[item.x]), item.z));
-      if (!mbar_wait_abort(accempty_bar, (k & 1) ^ 1, s_abort, status, G.wait_ns)) break;
+      if (!mbar_wait_warp(accempty_bar, (k & 1) ^ 1, s_abort, status, G.wait_ns)) break;
       const int type = item.y, n_prod = n_products(type);
       for (int s = 0, pr = 0; s < n_steps; ++s, ++g) {
         // a subtracted product (both halves alike): the instruction's negate-A bit
         const uint32_t neg = (step_of(type, pr).top & 4) ? 1u << 13 : 0u;
         if (++pr == n_prod) pr = 0;
         const int sa = uniform(g & 1), sb = uniform(g % kStagesB);
-        if (!mbar_wait_abort(bfull_bar(sb), (g / kStagesB) & 1, s_abort, status, G.wait_ns) ||
-            !mbar_wait_abort(afull_bar(sa), (g >> 1) & 1, s_abort, status, G.wait_ns)) {
+        if (!mbar_wait_warp(bfull_bar(sb), (g / kStagesB) & 1, s_abort, status, G.wait_ns) ||
+            !mbar_wait_warp(afull_bar(sa), (g >> 1) & 1, s_abort, status, G.wait_ns)) {
           ok = false;
           break;
         }
@@ -470,7 +472,7 @@ __global__ void __launch_bounds__(kThreads, 1)
       const int w = item_w(nb, item.z);  // accumulator levels are w columns wide
       const int ti0 = item.w & 0xffff, ti1 = static_cast<int>(static_cast<unsigned>(item.w) >> 16);
       const int* idx = G.bat_idx + G.bat_idx_ptr[b];
-      const bool ok = mbar_wait_abort(accfull_bar, k & 1, s_abort, status, G.wait_ns);
+      const bool ok = mbar_wait_warp(accfull_bar, k & 1, s_abort, status, G.wait_ns);
       if (bar_red_or(2, kEpiThreads, !ok)) break;  // also: the last item's pairs have been read
       tc_fence_after();
       if (quarter < 2 || ti1 != 0xffff) {

@@ -160,6 +160,29 @@ __device__ __forceinline__ bool mbar_wait_abort(uint32_t bar, uint32_t parity, v
   }
 }
 
+// the same by all lanes of a converged warp, which agree on every step by votes:
+// lane by lane, one might see the phase complete at a time-out and another give
+// up, and what follows a wait (votes, shuffles, elect.sync, barriers over whole
+// warps) would wait for ever for the lanes that had left.
+__device__ __forceinline__ bool mbar_wait_warp(uint32_t bar, uint32_t parity, volatile int* abort, unsigned* status,
+                                               uint64_t limit_ns) {
+  if (__all_sync(0xffffffffu, mbar_try_wait(bar, parity))) return true;
+  const unsigned mask = limit_ns < 1000000ull ? 0u : 31u;
+  uint64_t t0 = mask ? 0 : global_ns();
+  for (unsigned i = 1;; ++i) {
+    if (__all_sync(0xffffffffu, mbar_try_wait(bar, parity))) return true;
+    if (__any_sync(0xffffffffu, *abort)) return false;
+    if (i & mask) continue;
+    const uint64_t t = global_ns();
+    if (!t0) t0 = t;
+    if (__any_sync(0xffffffffu, t - t0 > limit_ns)) {
+      *abort = 1;
+      atomicOr(status, 1u);
+      return false;
+    }
+  }
+}
+
 __device__ __forceinline__ void mbar_arrive(uint32_t bar) {
   asm volatile("{\n\t.reg .b64 st;\n\tmbarrier.arrive.shared::cta.b64 st, [%0];\n\t}" ::"r"(bar) : "memory");
 }
