@@ -1,12 +1,15 @@
 // Split-precision batch products for batches of more than 256 functions: two
 // 64-function row tiles per step against one B operand.
 //
-// The slices, their levels and the outputs are those of split.cu (|d_0| up to 128
-// here: the digits resolve 2^-47 of the column's largest value, and levels 0-2
-// are sums of at most 3 2^14 units per term, exact for K <= 341 terms, the most
-// points of a batch; products that share an accumulator add their terms, and
-// where a sum then passed 2^24 units a rounding of L2 would sit ~2^-40 below the
-// column scale).
+// The slices, their levels and the outputs are those of split.cu.  An accumulator
+// of at most 341 terms (points times the products that share it) takes digits one
+// bit finer: |d_0| <= 128, resolving 2^-47 of the column's largest value, with
+// levels 0-2 sums of at most 2^14, 2^15 and 3 2^14 units per term, exact.  A longer
+// one keeps split.cu's |d_0| <= 64: level 1 is then exact for every batch (2^14
+// units a term, at most 1,023 terms) and level 2 for 512 terms, beyond which a
+// rounding of L2 sits ~2^-40 below the column scale.  With the finer digits there
+// level 1 itself would pass 2^24 and lose its last bits ~2^-32 below the column
+// scale: W0 of 340 points with digits of one sign 1e-9 off, 1e-15 so.
 //
 // Layout: M = 128 rows are two halves of 64 functions with a product each, both
 // against the same B operand: two row tiles of one output, or two outputs of
@@ -59,7 +62,6 @@ constexpr int kRawStep = 3 * kRawTile + 1024;        // A top, A bottom and B bo
 constexpr int kEpiPitch = kTile + 1;                 // (hi, lo) pairs per staged row
 constexpr uint32_t kTmemCols = 512;
 constexpr uint32_t kTmemA = 384;  // two stages of six A digits (48 columns) behind six levels of up to 64
-constexpr int kFine = 1;          // digits 2^-1 finer than tc::slice6's against the exponent itself
 
 // Shared memory: four raw stages of one step (two of two steps, half the handshakes,
 // are the slower by far: 304-atom slab 54.2 ms for 33.7), the B digits, the staged
@@ -101,6 +103,12 @@ __device__ __forceinline__ Step step_of(int type, int s) {
   }
   p >>= 10 * s;
   return {static_cast<int>(p & 3u), static_cast<int>((p >> 2) & 15u), static_cast<int>((p >> 6) & 15u)};
+}
+// bits by which the digits of an item of n_p points are finer than tc::slice6x2's
+// against the exponent itself: one where the terms of an accumulator stay at 341
+__device__ __forceinline__ int fine_of(int type, int np) {
+  const int k = type == kW0 || type == kDiag1 ? 3 : type >= kSOx && type <= kSOz ? 2 : 1;  // products in an accumulator
+  return k * np <= 341 ? 1 : 0;
 }
 // output of a half: 0 V (or F), 1 W0, 2-4 SO
 __device__ __forceinline__ int output_of(int type, bool bot) {
@@ -226,10 +234,8 @@ __global__ void __launch_bounds__(kThreads, 1)
   tc_fence_after();
   const uint32_t tmem = uniform(*tmem_slot);
   // steps of an item: each chunk of 16 points once per product
-  auto item_steps = [&](const int4& it) {
-    const int np = static_cast<int>(G.pt_ptr[it.x + 1] - G.pt_ptr[it.x]);
-    return (np + kKc - 1) / kKc * n_products(it.y);
-  };
+  auto item_np = [&](const int4& it) { return static_cast<int>(G.pt_ptr[it.x + 1] - G.pt_ptr[it.x]); };
+  auto item_steps = [&](const int4& it) { return (item_np(it) + kKc - 1) / kKc * n_products(it.y); };
 
   if (warp < kBWarp0) {
     // ---------------------------------------------------------- A slicers
@@ -262,7 +268,7 @@ __global__ void __launch_bounds__(kThreads, 1)
         acts |= 1u << s;
         if (ti * kTile + r64 < nb) e = max(e, __ldg(colexp + 8 * fn0 + (a & 3) * nb + ti * kTile + r64));
       }
-      const float mag = magic0(e - kFine);
+      const float mag = magic0(e - fine_of(type, item_np(item)));
       const float mm[4] = {mag, mag, mag, mag};
       for (int s = 0, pr = 0; s < n_st && ok; ++s, ++g, pr = pr + 1 == n_prod ? 0 : pr + 1) {
         const bool act = acts >> pr & 1u;
@@ -339,7 +345,8 @@ __global__ void __launch_bounds__(kThreads, 1)
         else
           e = max(e, v);
       }
-      const float mag = magic0(e - kFine), mag1 = type == kDiag2 ? magic0(e1 - kFine) : mag;
+      const int fine = fine_of(type, item_np(item));
+      const float mag = magic0(e - fine), mag1 = type == kDiag2 ? magic0(e1 - fine) : mag;
       for (int s = 0, pr = 0; s < n_st; ++s, ++g, pr = pr + 1 == n_prod ? 0 : pr + 1) {
         const int rs = g % kRaw;
         if (!mbar_wait_warp(rawfull_bar(rs), (g / kRaw) & 1, s_abort, status, G.wait_ns)) {
