@@ -990,9 +990,9 @@ extern "C" q4c_status grid_partition(const q4c_grid_desc* d, const q4c_tables* t
           for (int i = 0; i + 1 <= j; i += 2)  // W0 (three products), SO x, y, z (two), V
             for (int type : {1, 2, 3, 4, 0}) sitems.push_back(make_int4(static_cast<int>(b), type, j, i | (i + 1) << 16));
           if (j % 2 == 0) {  // the diagonal tile alone
+            sitems.push_back(make_int4(static_cast<int>(b), 1, j, j | static_cast<int>(0xffff0000u)));
             sitems.push_back(make_int4(static_cast<int>(b), 6, j, j | j << 16));
             sitems.push_back(make_int4(static_cast<int>(b), 7, j, j | j << 16));
-            sitems.push_back(make_int4(static_cast<int>(b), 0, j, j | static_cast<int>(0xffff0000u)));
           }
         }
         continue;

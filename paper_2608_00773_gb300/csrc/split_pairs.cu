@@ -23,8 +23,9 @@
 // sliced against a common exponent per function) and SO_x = (D Y)^T Z - (D Z)^T Y
 // etc. (two products).  A last single one is the diagonal tile, whose SO come
 // from A_yz = (D Y)^T Z etc. alone (SO_x = A_yz - A_yz^T, applied while
-// scattering), one beside W0, two beside each other.  The per-column operator is
-// Phi against Psi on every tile pair.
+// scattering), one beside V, two beside each other, each step's B operand sliced
+// against its own exponents; its W0 runs alone.  The per-column operator is Phi
+// against Psi on every tile pair.
 //
 // What bounds it: slicing.  A step of two products slices 192 rows of 16 values
 // (about 630 issue slots a scheduler) where two steps of split.cu slice 256, and its
@@ -80,14 +81,15 @@ static_assert(kSmemTotal <= 232448, "shared memory per CTA");
 // bottom half.  Its program is up to three products K-concatenated step by step:
 // per product the B quantity and for each half the A quantity (0 Phi, 1 X, 2 Y,
 // 3 Z; + 4: subtracted, D negated; + 8: present).
-enum Type { kV = 0, kW0 = 1, kSOx = 2, kSOy = 3, kSOz = 4, kCol = 5, kDiag1 = 6, kDiag2 = 7 };
+// kDiagV, kDiagA: the halves are different outputs of a diagonal tile, a step each.
+enum Type { kV = 0, kW0 = 1, kSOx = 2, kSOy = 3, kSOz = 4, kCol = 5, kDiagV = 6, kDiagA = 7 };
 struct Step {
   int b, top, bot;
 };
 constexpr unsigned step_code(int b, int top, int bot) { return static_cast<unsigned>(b | top << 2 | bot << 6); }
 constexpr unsigned program(unsigned s0, unsigned s1 = 0, unsigned s2 = 0) { return s0 | s1 << 10 | s2 << 20; }
 __device__ __forceinline__ int n_products(int type) {
-  return static_cast<int>((0x23122231u >> (4 * type)) & 15u);  // types 7 .. 0
+  return static_cast<int>((0x22122231u >> (4 * type)) & 15u);  // types 7 .. 0
 }
 __device__ __forceinline__ Step step_of(int type, int s) {
   unsigned p;
@@ -98,8 +100,8 @@ __device__ __forceinline__ Step step_of(int type, int s) {
     case kSOy: p = program(step_code(1, 11, 11), step_code(3, 13, 13)); break;  // Z X - X Z
     case kSOz: p = program(step_code(2, 9, 9), step_code(1, 14, 14)); break;    // X Y - Y X
     case kCol: p = program(step_code(1, 8, 8)); break;                          // Phi Psi
-    case kDiag1: p = program(step_code(1, 9, 11), step_code(2, 10, 0), step_code(3, 11, 0)); break;  // W0; A_zx
-    default: p = program(step_code(2, 9, 0), step_code(3, 0, 10)); break;                             // A_xy; A_yz
+    case kDiagV: p = program(step_code(1, 11, 0), step_code(0, 0, 8)); break;   // A_zx; V
+    default: p = program(step_code(2, 9, 0), step_code(3, 0, 10)); break;       // A_xy; A_yz
   }
   p >>= 10 * s;
   return {static_cast<int>(p & 3u), static_cast<int>((p >> 2) & 15u), static_cast<int>((p >> 6) & 15u)};
@@ -107,12 +109,12 @@ __device__ __forceinline__ Step step_of(int type, int s) {
 // bits by which the digits of an item of n_p points are finer than tc::slice6x2's
 // against the exponent itself: one where the terms of an accumulator stay at 341
 __device__ __forceinline__ int fine_of(int type, int np) {
-  const int k = type == kW0 || type == kDiag1 ? 3 : type >= kSOx && type <= kSOz ? 2 : 1;  // products in an accumulator
+  const int k = type == kW0 ? 3 : type >= kSOx && type <= kSOz ? 2 : 1;  // products in an accumulator
   return k * np <= 341 ? 1 : 0;
 }
 // output of a half: 0 V (or F), 1 W0, 2-4 SO
 __device__ __forceinline__ int output_of(int type, bool bot) {
-  return type <= kSOz ? type : type == kCol ? 0 : type == kDiag1 ? (bot ? 3 : 1) : (bot ? 2 : 4);
+  return type <= kSOz ? type : type == kCol ? 0 : type == kDiagV ? (bot ? 0 : 3) : (bot ? 2 : 4);
 }
 
 // B-tile width of an item: the functions of tile tj rounded up to 16 (the
@@ -340,13 +342,13 @@ __global__ void __launch_bounds__(kThreads, 1)
         const int f = item.z * kTile + r64;
         if (f >= nb) break;
         const int v = __ldg(colexp + 8 * fn0 + (4 + step_of(type, s).b) * nb + f);
-        if (type == kDiag2 && s == 1)
+        if (type >= kDiagV && s == 1)
           e1 = v;  // its two products go to different accumulators
         else
           e = max(e, v);
       }
       const int fine = fine_of(type, item_np(item));
-      const float mag = magic0(e - fine), mag1 = type == kDiag2 ? magic0(e1 - fine) : mag;
+      const float mag = magic0(e - fine), mag1 = type >= kDiagV ? magic0(e1 - fine) : mag;
       for (int s = 0, pr = 0; s < n_st; ++s, ++g, pr = pr + 1 == n_prod ? 0 : pr + 1) {
         const int rs = g % kRaw;
         if (!mbar_wait_warp(rawfull_bar(rs), (g / kRaw) & 1, s_abort, status, G.wait_ns)) {
@@ -509,7 +511,7 @@ __global__ void __launch_bounds__(kThreads, 1)
       auto load_off = [&](int blk, int (&off)[4]) {
         const int hb = halves == 2 ? blk & 1 : 0, c0 = (halves == 2 ? blk >> 1 : blk) * 16;
         const int o = output_of(item.y, hb != 0);
-        const bool sym = item.y != kCol && o <= 1, anti = item.y >= kDiag1 && o >= 2;
+        const bool sym = item.y != kCol && o <= 1, anti = item.y >= kDiagV && o >= 2;
         const int i0 = (hb ? ti1 : ti0) * kTile, j = item.z * kTile + c0 + col0;
 #pragma unroll
         for (int q = 0; q < 4; ++q) {
@@ -529,7 +531,7 @@ __global__ void __launch_bounds__(kThreads, 1)
         if (blk + 1 < n_blk) load_off(blk + 1, nxt);  // a block ahead
         const int hb = halves == 2 ? blk & 1 : 0, c0 = (halves == 2 ? blk >> 1 : blk) * 16;
         const int o = output_of(item.y, hb != 0);
-        const bool anti = item.y >= kDiag1 && o >= 2;
+        const bool anti = item.y >= kDiagV && o >= 2;
         double* out = o == 0 ? V : o == 1 ? W0 : o == 2 ? SOx : o == 3 ? SOy : SOz;
         const int i0 = (hb ? ti1 : ti0) * kTile, j = item.z * kTile + c0 + col0;
 #pragma unroll
