@@ -13,14 +13,11 @@
 // of one adjoint are (F, G', R) = (Phi, V, Phi), (Q, W, Q), (Y, x, Z), (Z, y, X),
 // (X, z, Y).
 //
-// Each U is computed from six BF16 slices of F (per-point exponents, one for
-// Phi and one for the three gradient quantities) and of G' (per-column
-// exponents, one for V and one for the other four matrices) in six FP32
-// accumulators, one per level s + t (see split.cu): levels 0-2 are exact
-// integer sums for K <= 512 terms (here at most 112), levels 3-5 are rounded
-// 2^-24 below.  The exponents are shared so that two products can be added up
-// in one accumulator set; a quantity's digits then resolve 2^-46 of the largest
-// of the three, which is what their sum resolves.
+// Each U is computed from six BF16 slices of F (an exponent per point and
+// quantity) and of G' (per-column exponents, one for V and one for the other
+// four matrices) in six FP32 accumulators, one per level s + t (see split.cu):
+// levels 0-2 are exact integer sums for K <= 512 terms (here at most 112),
+// levels 3-5 are rounded 2^-24 below.
 //
 // G' does not depend on the points, so a pre-pass slices every batch's G' once
 // into BF16 digit tiles laid out exactly as the MMA reads them (per matrix,
@@ -279,26 +276,24 @@ __global__ void __launch_bounds__(256, 5) k_gslice(DevGrid G, int64_t b0, const 
 //
 // Chunks of F digits stay in shared memory while every product that reads them
 // runs: an item is a list of segments, a segment fills up to seven slots and
-// then runs its groups, and a group (j-tile, R, one or two runs of chunks) is
-// one accumulation drained by the epilogue.
-//   fused items (n_ic <= 2): segment Phi; then one segment with all of X, Y, Z,
-//     whose groups add both products with the same R (W with F = R and an SO
-//     matrix) into one accumulation;
-//   other items: K segments of up to seven chunks, in each one segment per
-//     quantity, whose groups are single products (the row-dot with R is linear
-//     in U, so K segments add up in the point's running sum).
+// then runs its groups, and a group (j-tile, R, a run of chunks) is one
+// accumulation drained by the epilogue.
+// An item has K segments of up to seven chunks, in each one segment per quantity,
+// whose groups are single products (the row-dot with R is linear in U, so K
+// segments add up in the point's running sum).  Two products that are dotted with
+// the same R (W with F = R and an SO matrix) would share an accumulation only at
+// the price of one exponent for X, Y and Z of a point: on points along an axis,
+// X 2e4 times smaller than Z, the adjoint of SO_z alone then lost 14 bits of F.
 struct Item {
   int64_t bp0, scr, gsl, plane;
   int pt, np, ldp, nb, n_jt, n_ic;
   int jt0, jt1;  // the item's j-tiles
   int seg_len, nq;  // chunks of a K segment, segments in one
   unsigned qlist;  // quantities of a K segment, two bits each
-  bool fused;
 };
 
-constexpr int kPhi = 0, kOne = 1, kGrad = 2;  // kinds of segment
 struct Seg {
-  int kind, q, c0, c1, n;  // quantity and chunks [c0, c1); n: entries (slots)
+  int q, c0, c1, n;  // quantity and chunks [c0, c1); n: entries (slots)
 };
 
 // the SO matrix that multiplies F = quantity q (X: z, Y: x, Z: y) and the
@@ -325,18 +320,13 @@ __device__ __forceinline__ Item item_of(const RdItem* __restrict__ it, unsigned 
   I.plane = static_cast<int64_t>(I.nb) * I.ldp;
   const int n_kseg = max((I.n_ic + kSlots - 1) / kSlots, 1);
   I.seg_len = n_kseg == 1 ? I.n_ic : (I.n_ic + n_kseg - 1) / n_kseg;
-  I.fused = MODE == 1 && 3 * I.n_ic <= kSlots;
   I.qlist = 0;
   I.nq = 0;
   if (MODE == 0 || (present & 1u)) ++I.nq;  // Phi (two zero bits)
   if (MODE == 1) {
-    if (I.fused) {
-      if (present & 0x1eu) ++I.nq;
-    } else {
 #pragma unroll
-      for (int q = 1; q < 4; ++q)
-        if (present & (2u | 1u << so_matrix(q))) I.qlist |= static_cast<unsigned>(q) << (2 * I.nq++);
-    }
+    for (int q = 1; q < 4; ++q)
+      if (present & (2u | 1u << so_matrix(q))) I.qlist |= static_cast<unsigned>(q) << (2 * I.nq++);
   }
   if (I.n_ic == 0) I.nq = 0;
   return I;
@@ -345,15 +335,11 @@ __device__ __forceinline__ Item item_of(const RdItem* __restrict__ it, unsigned 
 // segment qi of the K segment that starts at chunk c0
 template <int MODE>
 __device__ __forceinline__ Seg seg_of(const Item& I, int qi, int c0, unsigned present) {
-  if (MODE == 1 && I.fused) {
-    if (qi == 0 && (present & 1u)) return {kPhi, 0, 0, I.n_ic, I.n_ic};
-    return {kGrad, 1, 0, I.n_ic, 3 * I.n_ic};
-  }
   const int q = MODE == 0 ? 0 : static_cast<int>((I.qlist >> (2 * qi)) & 3u);
   // a symmetric matrix alone needs the chunks up to the last j-tile's end only
   const bool sym = q == 0 || !(present >> so_matrix(q) & 1u);
   const int c1 = min(sym ? min(I.n_ic, 2 * I.jt1) : I.n_ic, c0 + I.seg_len);
-  return {q ? kOne : kPhi, q, c0, c1, max(0, c1 - c0)};
+  return {q, c0, c1, max(0, c1 - c0)};
 }
 // the segment after (qi, c0); false past the item's last one
 __device__ __forceinline__ bool next_seg(const Item& I, int& qi, int& c0) {
@@ -363,72 +349,46 @@ __device__ __forceinline__ bool next_seg(const Item& I, int& qi, int& c0) {
   return c0 < I.n_ic;
 }
 
-// one run of chunks of a group: chunks [c, c + n) of the segment's entries
-// from `ent` on, times matrix m
-struct Run {
-  int m, ent, c, n;
-};
-
 // The groups of one item in order: open() an item, then next() until it
-// returns false.  Run B follows run A in the same accumulation (B.n = 0: none).
+// returns false.
 template <int MODE>
 struct GroupWalk {
   Item I;
   Seg S;
   unsigned present;
-  int ent = 0;       // first entry of the segment in the CTA's sequence
-  int qi, c0, part, jt, r;  // qi = -1: before the item's first segment
-  int qr;            // quantity of the dot
-  Run A, B;
-  bool last;         // last group of its segment
+  int ent = 0;          // first entry of the segment in the CTA's sequence
+  int qi, c0, part, jt;  // qi = -1: before the item's first segment
+  int qr;               // quantity of the dot
+  int m, n;             // matrix, chunks (the segment's first n)
+  bool last;            // last group of its segment: it reads every chunk
   __device__ __forceinline__ explicit GroupWalk(unsigned pr) : present(pr) { S.n = 0; }
   __device__ __forceinline__ void open(const RdItem* it) {
     I = item_of<MODE>(it, present);
     qi = -1;
     c0 = 0;
-    B.n = 0;
   }
-  __device__ __forceinline__ bool has(int m) const { return present >> m & 1u; }
+  __device__ __forceinline__ bool has(int k) const { return present >> k & 1u; }
   __device__ __forceinline__ bool next() {
     for (;;) {
-      if (MODE == 1 && qi >= 0 && S.kind == kGrad) {
-        if (++r > 3) {
-          r = 1;
-          ++jt;
-        }
-        if (jt < I.jt1) {
-          const int q = r == 1 ? 3 : r - 1;  // the quantity whose SO product is dotted with r
-          const bool w = has(1), so = has(so_matrix(q));
-          if (!w && !so) continue;
-          const Run ra = {1, (r - 1) * I.n_ic, 0, jt_chunks(1, I.n_ic, jt)};
-          const Run rb = {so_matrix(q), (q - 1) * I.n_ic, 0, I.n_ic};
-          A = w ? ra : rb;
-          B = rb;
-          B.n = w && so ? I.n_ic : 0;
-          qr = r;
-          // a later r of the last j-tile has a group: through W, or X.z -> 2, Y.x -> 3
-          const bool more = r < 3 && (w || (r == 1 && has(4)) || has(2));
-          last = jt + 1 == I.jt1 && !more;
-          return true;
-        }
-      } else if (qi >= 0 && part < 2) {
+      if (qi >= 0 && part < 2) {
         ++jt;
-        const int mt = S.kind == kPhi ? 0 : 1;  // the symmetric matrix
-        const bool so = MODE == 1 && S.kind == kOne && has(so_matrix(S.q));
+        const int mt = S.q ? 1 : 0;  // the symmetric matrix
+        const bool so = MODE == 1 && S.q && has(so_matrix(S.q));
         if (jt >= I.jt1) {
           ++part;
           jt = I.jt0 - 1;
           continue;
         }
         if (part == 0) {
-          const int n = min(S.c1, jt_chunks(mt, I.n_ic, jt)) - S.c0;
+          n = min(S.c1, jt_chunks(mt, I.n_ic, jt)) - S.c0;
           if (n <= 0 || !(MODE == 0 || has(mt))) continue;
-          A = {mt, 0, S.c0, n};
+          m = mt;
           qr = S.q;
           last = !so && jt + 1 == I.jt1;
         } else {
           if (!so) continue;
-          A = {so_matrix(S.q), 0, S.c0, S.n};
+          m = so_matrix(S.q);
+          n = S.n;
           qr = so_dot(S.q);
           last = jt + 1 == I.jt1;
         }
@@ -440,13 +400,7 @@ struct GroupWalk {
       if (I.nq == 0 || !next_seg(I, qi, c0)) return false;
       S = seg_of<MODE>(I, qi, c0, present);
       part = 0;
-      B.n = 0;
-      if (MODE == 1 && S.kind == kGrad) {
-        jt = I.jt0;
-        r = 0;
-      } else {
-        jt = I.jt0 - 1;
-      }
+      jt = I.jt0 - 1;
     }
   }
 };
@@ -457,8 +411,7 @@ struct EntryWalk {
   const RdItem* items;
   int n_items;
   unsigned present;
-  int n, qi, c0, e;  // item, segment, entry within it
-  int q, c;          // quantity and chunk of the entry
+  int n, qi, c0, e;  // item, segment, entry within it: chunk S.c0 + e of quantity S.q
   Item I;
   Seg S;
   __device__ __forceinline__ EntryWalk(const RdItem* it, int ni, unsigned pr)
@@ -470,17 +423,11 @@ struct EntryWalk {
     qi = c0 = 0;
     S.n = 0;
     if (I.nq) S = seg_of<MODE>(I, 0, 0, present);
-    c = S.c0 - 1;
-    q = S.q;
   }
   // advances to the next entry; false at the end
   __device__ __forceinline__ bool next() {
     if (n >= n_items) return false;
     ++e;
-    if (++c >= S.c1) {  // the next quantity of a segment with all three
-      c = S.c0;
-      ++q;
-    }
     while (e >= S.n) {
       e = 0;
       if (I.nq && next_seg(I, qi, c0)) {
@@ -490,8 +437,6 @@ struct EntryWalk {
         if (n >= n_items) return false;
         open();
       }
-      c = S.c0;
-      q = S.q;
     }
     return true;
   }
@@ -600,7 +545,7 @@ __global__ void __launch_bounds__(kThreads, 1)
     bool live = false;
     int left = 0;  // functions from the chunk's first on
     int item = -1;
-    float mPhi = 0.f, mGrad = 0.f;  // rounding constants of the walk's current item
+    float mq[MODE == 0 ? 1 : 4];  // rounding constants of the walk's current item per quantity
     // raw values of the walk's entry (zeros past the batch's functions and points)
     auto load = [&]() {
       const Item& I = W.I;
@@ -608,15 +553,18 @@ __global__ void __launch_bounds__(kThreads, 1)
       live = p < I.np;
       if (item != W.n) {
         item = W.n;
-        mPhi = mGrad = 0.f;
-        if (live) {
-          const int4 e = *reinterpret_cast<const int4*>(rowexp + 4 * (I.bp0 + p));
-          mPhi = magic0(e.x - kFine);
-          mGrad = magic0(max(e.y, max(e.z, e.w)) - kFine);
+        int4 e = make_int4(-30000, -30000, -30000, -30000);
+        if (live) e = *reinterpret_cast<const int4*>(rowexp + 4 * (I.bp0 + p));
+        mq[0] = magic0(e.x - kFine);
+        if constexpr (MODE == 1) {
+          mq[1] = magic0(e.y - kFine);
+          mq[2] = magic0(e.z - kFine);
+          mq[3] = magic0(e.w - kFine);
         }
       }
-      const int q = W.q, f0 = W.c * kKc;
-      mag = q ? mGrad : mPhi;
+      const int q = W.S.q, f0 = (W.S.c0 + W.e) * kKc;
+      mag = mq[0];
+      if constexpr (MODE == 1) mag = q == 0 ? mag : q == 1 ? mq[1] : q == 2 ? mq[2] : mq[3];
       // no load is conditional: functions past the batch's read the last one and
       // are cleared below, points past n_p the row's end (their rows are dropped)
       const float2* src = reinterpret_cast<const float2*>(scratch) + I.scr + q * I.plane + min(p, I.ldp - 1);
@@ -696,24 +644,21 @@ __global__ void __launch_bounds__(kThreads, 1)
         for (; ok && W.next(); ++k) {
           if ((k & 1) != set) continue;
           const uint32_t blk = kSlices * kRowBytes * jt_width(W.I.nb, W.jt);
-          Run R = W.A;
-          for (int run = 0; run < 2 && ok; ++run, R = W.B) {
-            const unsigned char* src = gb + (static_cast<int64_t>(R.m) * W.I.n_jt + W.jt) * W.I.n_ic * kBlockB +
-                                       static_cast<int64_t>(R.c) * blk;
-            for (int c = 0; c < R.n; c += KS) {
-              if (!mbar_wait_abort(gempty_bar(set, st), ph, s_abort, status, G.wait_ns)) {
-                ok = false;
-                break;
-              }
-              const uint32_t bytes = min(KS, R.n - c) * blk;
-              arrive_expect_tx(gfull_bar(set, st), bytes);
-              bulk_copy(ring + st * L::kStage, src, bytes, gfull_bar(set, st));
-              src += bytes;
-              ++filled;
-              if (++st == kStages) {
-                st = 0;
-                ph ^= 1;
-              }
+          const unsigned char* src = gb + (static_cast<int64_t>(W.m) * W.I.n_jt + W.jt) * W.I.n_ic * kBlockB +
+                                     static_cast<int64_t>(W.S.c0) * blk;
+          for (int c = 0; c < W.n; c += KS) {
+            if (!mbar_wait_abort(gempty_bar(set, st), ph, s_abort, status, G.wait_ns)) {
+              ok = false;
+              break;
+            }
+            const uint32_t bytes = min(KS, W.n - c) * blk;
+            arrive_expect_tx(gfull_bar(set, st), bytes);
+            bulk_copy(ring + st * L::kStage, src, bytes, gfull_bar(set, st));
+            src += bytes;
+            ++filled;
+            if (++st == kStages) {
+              st = 0;
+              ph ^= 1;
             }
           }
         }
@@ -768,48 +713,37 @@ __global__ void __launch_bounds__(kThreads, 1)
           break;
         }
         tc_fence_after();
-        // every entry the group reads (the last one is in its last run)
-        if (!see(W.ent + (W.B.n ? max(W.A.ent + W.A.n, W.B.ent + W.B.n) : W.A.ent + W.A.n) - 1)) {
+        if (!see(W.ent + W.n - 1)) {  // every entry the group reads
           ok = false;
           break;
         }
         tc_fence_after();
         const int w = uniform(jt_width(W.I.nb, W.jt));
-        const bool release = W.last && W.S.kind != kGrad;  // the last group reads every chunk of its segment in order
-        bool first = true;
-        Run R = W.A;
-        for (int run = 0; run < 2 && ok; ++run, R = W.B)
-          for (int c = 0; c < R.n && ok; c += KS) {
-            if (!mbar_wait_warp(gfull_bar(set, st), ph, s_abort, status, G.wait_ns)) {
-              ok = false;
-              break;
-            }
-            tc_fence_after();
+        for (int c = 0; c < W.n; c += KS) {
+          if (!mbar_wait_warp(gfull_bar(set, st), ph, s_abort, status, G.wait_ns)) {
+            ok = false;
+            break;
+          }
+          tc_fence_after();
 #pragma unroll
-            for (int h = 0; h < KS; ++h) {
-              if (c + h >= R.n) break;
-              const int slot = uniform((W.ent + R.ent + c + h) % kSlots);
-              const uint64_t a = descA + static_cast<uint32_t>(slot * (kSlot >> 4));
-              const uint64_t bd = descB + static_cast<uint32_t>((st * L::kStage + h * kSlices * kRowBytes * w) >> 4);
-              if (elect_one()) {
-                mma_row_levels(t0, a, bd, w, first);
-                if (release) mma_commit(slotempty_bar(slot));
-              }
-              first = false;
-            }
-            if (ok && elect_one()) mma_commit(gempty_bar(set, st));
-            if (++st == kStages) {
-              st = 0;
-              ph ^= 1;
+          for (int h = 0; h < KS; ++h) {
+            if (c + h >= W.n) break;
+            const int slot = uniform((W.ent + c + h) % kSlots);
+            const uint64_t a = descA + static_cast<uint32_t>(slot * (kSlot >> 4));
+            const uint64_t bd = descB + static_cast<uint32_t>((st * L::kStage + h * kSlices * kRowBytes * w) >> 4);
+            if (elect_one()) {
+              mma_row_levels(t0, a, bd, w, c + h == 0);
+              if (W.last) mma_commit(slotempty_bar(slot));
             }
           }
-        if (ok && W.last && !release) ok = see(W.ent + W.S.n - 1);
-        if (!ok) break;
-        if (elect_one()) {
-          mma_commit(accfull_bar(set));
-          if (W.last && !release)
-            for (int e = W.ent; e < W.ent + W.S.n; ++e) mma_commit(slotempty_bar(e % kSlots));
+          if (elect_one()) mma_commit(gempty_bar(set, st));
+          if (++st == kStages) {
+            st = 0;
+            ph ^= 1;
+          }
         }
+        if (!ok) break;
+        if (elect_one()) mma_commit(accfull_bar(set));
       }
     }
     // every MMA issued by this warp has completed before tensor memory is freed
