@@ -262,9 +262,9 @@ struct q4c_grid {
   unsigned* d_status = nullptr;            // bit 0: a bounded wait expired
   float2* d_gdf = nullptr;                 // [10][nnz] FP32-pair copies of the density (0-4) and adjoint (5-9) matrices
   // per pattern block q, at cm_off[q]: a bound of each of its nf_B columns
-  // (FP32, rounded up), for V and for the largest of the other four matrices,
-  // of the density's and of the adjoint's ([4][cm_total]); the G' pre-pass
-  // bounds a batch column's largest element from them
+  // (FP32, rounded up) for each matrix of the density and of the adjoint
+  // ([10][cm_total]); the G' pre-pass bounds a batch column's largest element
+  // from them
   int64_t* d_cm_off = nullptr;             // [n_blocks + 1]
   int64_t cm_total = 0;
   float* d_cm = nullptr;

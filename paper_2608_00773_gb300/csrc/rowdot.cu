@@ -14,10 +14,9 @@
 // (X, z, Y).
 //
 // Each U is computed from six BF16 slices of F (an exponent per point and
-// quantity) and of G' (per-column exponents, one for V and one for the other
-// four matrices) in six FP32 accumulators, one per level s + t (see split.cu):
-// levels 0-2 are exact integer sums for K <= 512 terms (here at most 112),
-// levels 3-5 are rounded 2^-24 below.
+// quantity) and of G' (an exponent per column and matrix) in six FP32
+// accumulators, one per level s + t (see split.cu): levels 0-2 are exact integer
+// sums for K <= 512 terms (here at most 112), levels 3-5 are rounded 2^-24 below.
 //
 // G' does not depend on the points, so a pre-pass slices every batch's G' once
 // into BF16 digit tiles laid out exactly as the MMA reads them (per matrix,
@@ -86,8 +85,7 @@ struct Mats {
 // a block that is its own partner) and G - G^T for the SO matrices, formed in
 // FP64, G^T read from the partner block (B, A, -T) through shared memory where
 // both sides have at most 64 functions, else straight from memory; and at
-// cm_off[q] an FP32 bound of each of its nf_B columns, cm[0] for V and cm[1]
-// for the largest of the other four.
+// cm_off[q] an FP32 bound of each of its nf_B columns, cm[m] for matrix m.
 __global__ void __launch_bounds__(128) k_prepare_blocks(DevBasis B, DevGrid G, Mats M, int64_t n_blocks,
                                                        const int* __restrict__ blk_row,
                                                        const int* __restrict__ blk_col,
@@ -96,14 +94,14 @@ __global__ void __launch_bounds__(128) k_prepare_blocks(DevBasis B, DevGrid G, M
                                                        const int64_t* __restrict__ cm_off, float2* __restrict__ out,
                                                        int64_t nnz, float* __restrict__ cm, int64_t cm_total) {
   __shared__ double sT[64 * 65];      // G^T of the block: sT[i * 65 + j] = partner (j, i)
-  extern __shared__ unsigned s_cm[];  // [2][nf_B] bits of the column bounds (non-negative floats order as integers)
+  extern __shared__ unsigned s_cm[];  // [5][nf_B] bits of the column bounds (non-negative floats order as integers)
   for (int64_t q = blockIdx.x; q < n_blocks; q += gridDim.x) {
     const int nfA = __ldg(B.sp_nfn + G.atom_sp[blk_row[q]]), nfB = __ldg(B.sp_nfn + G.atom_sp[blk_col[q]]);
     const int64_t o0 = blk_off[q];
     const int ne = nfA * nfB, qt = blk_T[q];
     const bool tile = qt >= 0 && nfA <= 64 && nfB <= 64;
     __syncthreads();
-    for (int j = threadIdx.x; j < 2 * nfB; j += blockDim.x) s_cm[j] = 0u;
+    for (int j = threadIdx.x; j < 5 * nfB; j += blockDim.x) s_cm[j] = 0u;
 #pragma unroll
     for (int m = 0; m < 5; ++m) {
       if (M.m[m] == nullptr) continue;
@@ -125,14 +123,14 @@ __global__ void __launch_bounds__(128) k_prepare_blocks(DevBasis B, DevGrid G, M
         const double x = m >= 2 ? g - xt : (qt == q && i == j) ? g : g + xt;
         const float h = __double2float_rn(x), l = __double2float_rn(x - static_cast<double>(h));
         o[e] = make_float2(h, l);
-        atomicMax(&s_cm[(m ? nfB : 0) + j], __float_as_uint(__fadd_ru(fabsf(h), fabsf(l))));
+        atomicMax(&s_cm[m * nfB + j], __float_as_uint(__fadd_ru(fabsf(h), fabsf(l))));
       }
     }
     __syncthreads();
-    for (int j = threadIdx.x; j < nfB; j += blockDim.x) {
-      cm[cm_off[q] + j] = __uint_as_float(s_cm[j]);
-      cm[cm_total + cm_off[q] + j] = __uint_as_float(s_cm[nfB + j]);
-    }
+    for (int j = threadIdx.x; j < nfB; j += blockDim.x)
+#pragma unroll
+      for (int m = 0; m < 5; ++m)
+        if (M.m[m]) cm[m * cm_total + cm_off[q] + j] = __uint_as_float(s_cm[m * nfB + j]);
   }
 }
 
@@ -175,8 +173,7 @@ __global__ void __launch_bounds__(256, 5) k_gslice(DevGrid G, int64_t b0, const 
                                                 unsigned present, const float* __restrict__ cm, int64_t cm_total,
                                                 const int* __restrict__ pair_blk, const int64_t* __restrict__ cm_off,
                                                 const int64_t* __restrict__ gsl_off, uint32_t* __restrict__ gsl) {
-  constexpr int kB = NM > 1 ? 2 : 1;      // column bounds: of V, of the other matrices
-  __shared__ unsigned sMax[kB][kTileJ];  // their bits
+  __shared__ unsigned sMax[NM][kTileJ];  // column bounds per matrix (bits)
   const int64_t b = b0 + blockIdx.x;
   const int64_t f0 = G.bat_fn_ptr[b];
   const int nb = static_cast<int>(G.bat_fn_ptr[b + 1] - f0);
@@ -190,23 +187,24 @@ __global__ void __launch_bounds__(256, 5) k_gslice(DevGrid G, int64_t b0, const 
   const int r8 = lane >> 2, kp = lane & 3;
   for (int jt = blockIdx.y; jt < n_jt; jt += gridDim.y) {
     __syncthreads();
-    if (threadIdx.x < kB * kTileJ) sMax[threadIdx.x / kTileJ][threadIdx.x % kTileJ] = 0u;
+    if (threadIdx.x < NM * kTileJ) sMax[threadIdx.x / kTileJ][threadIdx.x % kTileJ] = 0u;
     __syncthreads();
     {  // column bounds: eight threads a column over the batch's centres
       const int jl = threadIdx.x >> 3, j = jt * kTileJ + jl;
       if (j < nb) {
         const int info = G.fn_info[f0 + j], c = info >> 16, jj = info & 0xffff;
-        float mx[kB] = {};
+        float mx[NM] = {};
         for (int a = threadIdx.x & 7; a < na; a += 8) {
           const int q = pb[a * na + c];  // block (a, c): its column jj
           if (q >= 0) {
             const int64_t o = cm_off[q] + jj;
 #pragma unroll
-            for (int k = 0; k < kB; ++k) mx[k] = fmaxf(mx[k], __ldg(cm + k * cm_total + o));
+            for (int m = 0; m < NM; ++m)
+              if (present >> m & 1u) mx[m] = fmaxf(mx[m], __ldg(cm + m * cm_total + o));
           }
         }
 #pragma unroll
-        for (int k = 0; k < kB; ++k) atomicMax(&sMax[k][jl], __float_as_uint(mx[k]));
+        for (int m = 0; m < NM; ++m) atomicMax(&sMax[m][jl], __float_as_uint(mx[m]));
       }
     }
     __syncthreads();
@@ -257,7 +255,7 @@ __global__ void __launch_bounds__(256, 5) k_gslice(DevGrid G, int64_t b0, const 
           const int j = jt * kTileJ + j_[u];
           const bool a0 = ok0[u] && (m >= 2 || i_[u] <= j), a1 = ok1[u] && (m >= 2 || i_[u] + 1 <= j);
           const float2 y0 = x0[m][u], y1 = x1[m][u];
-          const unsigned mb = sMax[m ? kB - 1 : 0][j_[u]];
+          const unsigned mb = sMax[m][j_[u]];
           float2 d[kSlices];
           slice6x2(pk2(a0 ? y0.x : 0.f, a1 ? y1.x : 0.f), pk2(a0 ? y0.y : 0.f, a1 ? y1.y : 0.f),
                    magic0((mb ? fexp(__uint_as_float(mb)) : -30000) - kFine), d);
@@ -857,7 +855,7 @@ __global__ void __launch_bounds__(kThreads, 1)
 }
 
 // the prepared matrices of one call: FP32-pair copies in slots [slot, slot + 5)
-// of the grid's buffer and two column bounds per block; slot 0 for the density,
+// of the grid's buffer and their column bounds per block; slot 0 for the density,
 // 5 for the adjoint.  Returns the mask of present matrices.
 q4c_status prepare(const q4c_grid* g, const double* const mats[5], int slot, unsigned* present, cudaStream_t s) {
   int dev = 0, n_sm = 0;
@@ -870,14 +868,14 @@ q4c_status prepare(const q4c_grid* g, const double* const mats[5], int slot, uns
     M.m[m] = mats[m];
     if (mats[m]) *present |= 1u << m;
   }
-  const size_t smem = sizeof(unsigned) * 2 * *std::max_element(g->tables->nfn.begin(), g->tables->nfn.end());
+  const size_t smem = sizeof(unsigned) * 5 * *std::max_element(g->tables->nfn.begin(), g->tables->nfn.end());
   if (smem > 12 * 1024)
     Q4C_CUDA(cudaFuncSetAttribute(k_prepare_blocks, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem)));
   KernelScope ks("split_gslice", s);
   const unsigned nblk = static_cast<unsigned>(std::min<int64_t>(g->n_blocks, 64 * n_sm));
   k_prepare_blocks<<<nblk, 128, smem, s>>>(g->tables->view(), g->view(), M, g->n_blocks, g->d_blk_row, g->d_blk_col,
                                            g->d_blk_off, g->d_blk_T, g->d_cm_off, g->d_gdf + slot * g->nnz, g->nnz,
-                                           g->d_cm + (slot ? 2 : 0) * g->cm_total, g->cm_total);
+                                           g->d_cm + slot * g->cm_total, g->cm_total);
   Q4C_CUDA(cudaGetLastError());
   return Q4C_OK;
 }
@@ -891,7 +889,7 @@ q4c_status gslice_wave(const q4c_grid* g, int wv, int slot, unsigned present, cu
   const unsigned y = static_cast<unsigned>(std::max(1, (g->max_nb + 2 * kTileJ - 1) / (2 * kTileJ)));
   KernelScope ks("split_gslice", s);
   k_gslice<MODE == 0 ? 1 : 5><<<dim3(static_cast<unsigned>(b1 - b0), y), 256, 0, s>>>(
-      g->view(), b0, g->d_gdf + slot * g->nnz, g->nnz, present, g->d_cm + (slot ? 2 : 0) * g->cm_total, g->cm_total,
+      g->view(), b0, g->d_gdf + slot * g->nnz, g->nnz, present, g->d_cm + slot * g->cm_total, g->cm_total,
       g->d_pair_blk, g->d_cm_off, g->d_gsl_off, reinterpret_cast<uint32_t*>(g->d_gsl));
   Q4C_CUDA(cudaGetLastError());
   return Q4C_OK;
@@ -979,7 +977,7 @@ q4c_status autotune_rowdot(q4c_grid* g, double* out, cudaStream_t s) {
   if (g->wave_b0.size() < 2 || g->max_nb > rowdot::kMaxNb || g->nnz == 0) return Q4C_OK;
   if (g->wave_b0[1] <= g->wave_b0[0]) return Q4C_OK;
   Q4C_CUDA(cudaMemsetAsync(g->d_gdf + 5 * g->nnz, 0, sizeof(float2) * 5 * g->nnz, s));
-  Q4C_CUDA(cudaMemsetAsync(g->d_cm + 2 * g->cm_total, 0, sizeof(float) * 2 * g->cm_total, s));
+  Q4C_CUDA(cudaMemsetAsync(g->d_cm + 5 * g->cm_total, 0, sizeof(float) * 5 * g->cm_total, s));
   if (q4c_status st = rowdot::gslice_wave<1>(g, 0, 5, 31u, s)) return st;
   cudaEvent_t ev[2][3][2] = {};
   q4c_status status = Q4C_OK;
