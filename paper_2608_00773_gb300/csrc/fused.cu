@@ -49,10 +49,6 @@ q4c_status scf_pass(const q4c_tables* t, const q4c_grid* g, const double* v, con
     const double* mats[5] = {Gm->V, Gm->W0, Gm->SOx, Gm->SOy, Gm->SOz};
     if (q4c_status st = rowdot_prepare(g, mats, 5, &presentG, s)) return st;
   }
-  if (split && g->rd_shares) {
-    if (do_n) Q4C_CUDA(cudaMemsetAsync(n, 0, sizeof(double) * g->n_pts, s));
-    if (do_g) Q4C_CUDA(cudaMemsetAsync(dLdv, 0, sizeof(double) * g->n_pts, s));
-  }
   const int n_waves = static_cast<int>(g->wave_b0.size()) - 1;
   for (int wv = 0; wv < n_waves; ++wv) {
     const int64_t b0 = g->wave_b0[wv], b1 = g->wave_b0[wv + 1];

@@ -1058,21 +1058,32 @@ extern "C" q4c_status grid_partition(const q4c_grid_desc* d, const q4c_tables* t
   // first.  Eight j-tiles (256 functions) an item at most: an item of a batch
   // of 1,918 functions would be 7 times the average SM's share of a wave (the
   // 304-atom slab: adjoint 47.6 ms with whole batches, 37.0 with shares), while
-  // a share still reads each sliced chunk of F about 16 times.
+  // a share still reads each sliced chunk of F about 16 times.  The shares of a
+  // tile leave partial sums that are added up in order, so that a call repeats
+  // bit for bit.
   std::vector<RdItem> rditems;
+  std::vector<RdSum> rdsums;
+  int64_t rd_slots = 0;  // of the largest wave
   g->rd_w0.push_back(0);
+  g->rd_s0.push_back(0);
   for (size_t wv = 0; wv + 1 < g->wave_b0.size(); ++wv) {
     const size_t first = rditems.size();
+    int64_t slot = 0;
     for (int64_t b = g->wave_b0[wv]; b < g->wave_b0[wv + 1]; ++b) {
       const int np = static_cast<int>(bptr[b + 1] - bptr[b]);
       const int nb = static_cast<int>(g->h_bat_fn_ptr[b + 1] - g->h_bat_fn_ptr[b]);
       const int n_jt = (nb + 31) / 32;
-      const int shares = std::max(1, (n_jt + 7) / 8), per = std::max(1, (n_jt + shares - 1) / shares);
-      g->rd_shares = g->rd_shares || shares > 1;
-      for (int j = 0; j < std::max(n_jt, 1); j += per)
+      const int most = std::max(1, (n_jt + 7) / 8), per = std::max(1, (n_jt + most - 1) / most);
+      const int shares = std::max(1, (n_jt + per - 1) / per);
+      for (int k = 0; k < shares; ++k)
         for (int pt = 0; pt * 128 < np; ++pt)
-          rditems.push_back({np, nb, pt, j | std::min(n_jt, j + per) << 16, bptr[b], g->h_scr_off[b], gsl_off[b], 0});
+          rditems.push_back({np, nb, pt, k * per | std::min(n_jt, (k + 1) * per) << 16, bptr[b], g->h_scr_off[b],
+                             gsl_off[b], shares > 1 ? slot + pt * shares + k : -1});
+      for (int pt = 0; shares > 1 && pt * 128 < np; ++pt, slot += shares)
+        rdsums.push_back({bptr[b] + pt * 128, std::min(128, np - pt * 128), static_cast<int>(slot), shares, 0});
     }
+    rd_slots = std::max(rd_slots, slot);
+    g->rd_s0.push_back(static_cast<int64_t>(rdsums.size()));
     auto cost = [](const RdItem& x) { return (x.nb + 15) / 16 * ((x.jts >> 16) - (x.jts & 0xffff)); };
     std::stable_sort(rditems.begin() + first, rditems.end(),
                      [&](const RdItem& x, const RdItem& y) { return cost(x) > cost(y); });
@@ -1124,7 +1135,7 @@ extern "C" q4c_status grid_partition(const q4c_grid_desc* d, const q4c_tables* t
       (st = up(&g->d_kblk_q1, g->h_kblk_q1)) || (st = up(&g->d_kblk_off, g->h_kblk_off)) ||
       (st = up(&g->d_scr_off, g->h_scr_off)) || (st = up(&g->d_tiles, tiles)) || (st = up(&g->d_col_tiles, col_tiles)) || (st = up(&g->d_sched, sched)) ||
       (st = up(&g->d_split_items, sitems)) || (st = up(&g->d_col_items, citems)) ||
-      (st = up(&g->d_rd_items, rditems)) ||
+      (st = up(&g->d_rd_items, rditems)) || (st = up(&g->d_rd_sums, rdsums)) ||
       (st = up(&g->d_bat_idx_ptr, idx_ptr)) ||
       (st = up(&g->d_gsl_off, gsl_off))) {
     q4c_grid_destroy(g);
@@ -1136,6 +1147,7 @@ extern "C" q4c_status grid_partition(const q4c_grid_desc* d, const q4c_tables* t
     if (e == cudaSuccess) e = cudaMalloc(&g->d_counter, sizeof(int) * std::max<size_t>(n_waves, 1));
     if (e == cudaSuccess) e = cudaMalloc(&g->d_colexp, sizeof(int) * 8 * std::max<int64_t>(g->h_bat_fn_ptr[nB], 1));
     if (e == cudaSuccess) e = cudaMalloc(&g->d_rowexp, sizeof(int) * 4 * nP);
+    if (e == cudaSuccess) e = cudaMalloc(&g->d_rd_part, sizeof(double) * 128 * std::max<int64_t>(rd_slots, 1));
     if (e == cudaSuccess) e = cudaMalloc(&g->d_gsl, static_cast<size_t>(std::max<int64_t>(g->gsl_bytes, 16)));
     if (e == cudaSuccess) e = cudaMalloc(&g->d_gdf, sizeof(float2) * 10 * std::max<int64_t>(g->nnz, 1));
     if (e == cudaSuccess) e = cudaMalloc(&g->d_cm, sizeof(float) * 10 * g->cm_total);
@@ -1147,7 +1159,8 @@ extern "C" q4c_status grid_partition(const q4c_grid_desc* d, const q4c_tables* t
     if (e == cudaSuccess) e = cudaMemset(g->d_status, 0, sizeof(unsigned));
     g->split_ws_bytes = static_cast<int64_t>(sizeof(int)) * (8 * g->h_bat_fn_ptr[nB] + 4 * nP) +
                         static_cast<int64_t>(sizeof(float2)) * 5 * g->nnz + g->gsl_bytes +
-                        static_cast<int64_t>(sizeof(float)) * 10 * g->cm_total;
+                        static_cast<int64_t>(sizeof(float)) * 10 * g->cm_total +
+                        static_cast<int64_t>(sizeof(double)) * 128 * rd_slots;
     if (e != cudaSuccess) {
       set_error(std::string("grid_partition: workspace: ") + cudaGetErrorString(e));
       q4c_grid_destroy(g);
@@ -1168,7 +1181,7 @@ extern "C" void q4c_grid_destroy(q4c_grid* g) {
                   g->d_pt_ptr, g->d_bat_atom_ptr, g->d_bat_atoms, g->d_bat_atom_fn0, g->d_bat_fn_ptr,
                   g->d_fn_info, g->d_bat_pair_ptr, g->d_pair_off, g->d_blk_off, g->d_blk_row, g->d_blk_col,
                   g->d_blk_T, g->d_scr_off, g->d_tiles, g->d_col_tiles, g->d_scratch, g->d_sched, g->d_counter, g->d_split_ws,
-                  g->d_split_items, g->d_col_items, g->d_split_mag, g->d_dpad, g->d_tmaps, g->d_colexp, g->d_status, g->d_rd_items, g->d_rowexp, g->d_gsl, g->d_gsl_off,
+                  g->d_split_items, g->d_col_items, g->d_split_mag, g->d_dpad, g->d_tmaps, g->d_colexp, g->d_status, g->d_rd_items, g->d_rd_sums, g->d_rd_part, g->d_rowexp, g->d_gsl, g->d_gsl_off,
                   g->d_bat_idx_ptr, g->d_bat_idx, g->d_pts_df, g->d_atoms_df, g->d_gdf,
                   g->d_c_xyz, g->d_c_sp, g->d_blk_role, g->d_blk_shift, g->d_kblk_q0, g->d_kblk_q1,
                   g->d_kblk_off, g->d_cm_off, g->d_cm, g->d_pair_blk};

@@ -128,7 +128,14 @@ struct DevGrid {
 // it in one read.
 struct __align__(16) RdItem {
   int np, nb, pt, jts;          // points and functions of the batch, point tile, j-tiles [jts & 0xffff, jts >> 16)
-  long long pt0, scr, gsl, pad;  // first point, basis tiles (values), G' blocks (bytes)
+  long long pt0, scr, gsl, part;  // first point, basis tiles (values), G' blocks (bytes), partial sums (-1: none)
+};
+
+// The points [pt0, pt0 + n) of a 128-point tile whose j-tiles are shared out: the
+// shares' partial sums lie at slots slot0 .. slot0 + shares - 1 of 128 values
+struct RdSum {
+  long long pt0;
+  int n, slot0, shares, pad;
 };
 
 // the work-wait limit that q4c_set_wait_limit_ns last set (1 s by default)
@@ -251,7 +258,9 @@ struct q4c_grid {
   int* d_colexp = nullptr;                 // [8 * sum n_b]
   std::vector<int64_t> rd_w0;              // [n_waves+1] ranges into d_rd_items
   q4c::RdItem* d_rd_items = nullptr;       // work of the density/adjoint kernel
-  bool rd_shares = false;                  // some batch's j-tiles are shared out over several items
+  std::vector<int64_t> rd_s0;              // [n_waves+1] ranges into d_rd_sums
+  q4c::RdSum* d_rd_sums = nullptr;         // tiles whose j-tiles are shared out over several items
+  double* d_rd_part = nullptr;             // [slots of the largest wave][128] their partial sums
   int* d_rowexp = nullptr;                 // [n_points][4] per-point exponents
   unsigned char* d_gsl = nullptr;          // G' digit blocks of one wave (density/adjoint)
   int64_t* d_gsl_off = nullptr;            // [n_batches] byte offsets into d_gsl (per wave)

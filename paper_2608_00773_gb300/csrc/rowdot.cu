@@ -283,7 +283,7 @@ __global__ void __launch_bounds__(256, 5) k_gslice(DevGrid G, int64_t b0, const 
 // the price of one exponent for X, Y and Z of a point: on points along an axis,
 // X 2e4 times smaller than Z, the adjoint of SO_z alone then lost 14 bits of F.
 struct Item {
-  int64_t bp0, scr, gsl, plane;
+  int64_t bp0, scr, gsl, part, plane;
   int pt, np, ldp, nb, n_jt, n_ic;
   int jt0, jt1;  // the item's j-tiles
   int seg_len, nq;  // chunks of a K segment, segments in one
@@ -310,6 +310,7 @@ __device__ __forceinline__ Item item_of(const RdItem* __restrict__ it, unsigned 
   I.bp0 = v.x;
   I.scr = v.y;
   I.gsl = w.x;
+  I.part = w.y;
   I.np = u.x;
   I.nb = u.y;
   I.ldp = (I.np + 7) & ~7;
@@ -482,7 +483,7 @@ template <int MODE, int KS>  // MODE 0: density, 1: adjoint; KS: G' blocks per s
 __global__ void __launch_bounds__(kThreads, 1)
     k_split_rowdot(DevGrid G, const RdItem* __restrict__ items, int n_items, const double* __restrict__ scratch,
                    const int* __restrict__ rowexp, const unsigned char* __restrict__ gsl, unsigned present,
-                   int weighted, double* __restrict__ out, unsigned* status) {
+                   int weighted, double* __restrict__ out, double* __restrict__ part, unsigned* status) {
   using L = Layout<KS>;
   constexpr int kStages = L::kStages;
   extern __shared__ __align__(1024) unsigned char smem[];
@@ -839,11 +840,10 @@ __global__ void __launch_bounds__(kThreads, 1)
       if (eg == 0 && live) {
         const double val = sY[r] + sY[kPts + r];
         const int64_t gp = I.bp0 + p;
-        const double res = weighted ? G.w[gp] * val : val;
-        if (I.jt1 - I.jt0 == I.n_jt)
-          out[gp] = res;
+        if (I.part < 0)
+          out[gp] = weighted ? G.w[gp] * val : val;
         else
-          atomicAdd(out + gp, res);  // shares of one batch (zeroed before the first wave)
+          part[I.part * kPts + r] = val;  // a share of the batch's j-tiles: k_rowdot_sum adds them up
       }
       bar_sync(2, kEpiThreads);
     }
@@ -852,6 +852,20 @@ __global__ void __launch_bounds__(kThreads, 1)
   __syncthreads();
   if (warp == kMmaWarp)
     asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(kTmemCols));
+}
+
+// The points of tiles whose j-tiles were shared out: their shares' sums added in
+// order (one CTA per tile; 8 bytes a share and point, 20 MB for the 304-atom slab).
+__global__ void __launch_bounds__(kPts) k_rowdot_sum(const RdSum* __restrict__ sums, const double* __restrict__ part,
+                                                   const double* __restrict__ w, int weighted,
+                                                   double* __restrict__ out) {
+  const RdSum s = sums[blockIdx.x];
+  const int r = threadIdx.x;
+  if (r >= s.n) return;
+  const double* x = part + static_cast<int64_t>(s.slot0) * kPts + r;
+  double y = x[0];
+  for (int k = 1; k < s.shares; ++k) y += x[k * kPts];
+  out[s.pt0 + r] = weighted ? w[s.pt0 + r] * y : y;
 }
 
 // the prepared matrices of one call: FP32-pair copies in slots [slot, slot + 5)
@@ -912,9 +926,16 @@ q4c_status rowdot_kernel(const q4c_grid* g, int wv, unsigned present, bool weigh
     KernelScope ks(name, s);
     k_split_rowdot<MODE, KS><<<grid, kThreads, Layout<KS>::kSmemTotal, s>>>(
         g->view(), g->d_rd_items + i0, n_items, g->d_scratch, g->d_rowexp,
-        reinterpret_cast<const unsigned char*>(g->d_gsl), present, weighted ? 1 : 0, out, g->d_status);
+        reinterpret_cast<const unsigned char*>(g->d_gsl), present, weighted ? 1 : 0, out, g->d_rd_part, g->d_status);
   }
   Q4C_CUDA(cudaGetLastError());
+  const int64_t s0 = g->rd_s0[wv], s1 = g->rd_s0[wv + 1];
+  if (s1 > s0) {
+    KernelScope ks("split_rowdot_sum", s);
+    k_rowdot_sum<<<static_cast<unsigned>(s1 - s0), kPts, 0, s>>>(g->d_rd_sums + s0, g->d_rd_part, g->d_w,
+                                                                 weighted ? 1 : 0, out);
+    Q4C_CUDA(cudaGetLastError());
+  }
   return Q4C_OK;
 }
 
@@ -941,7 +962,6 @@ q4c_status run(const q4c_tables* t, const q4c_grid* g, const double* const mats[
   }
   unsigned present = 0;
   if (q4c_status st = prepare(g, mats, 0, &present, s)) return st;
-  if (g->rd_shares) Q4C_CUDA(cudaMemsetAsync(out, 0, sizeof(double) * g->n_pts, s));
   const int n_waves = static_cast<int>(g->wave_b0.size()) - 1;
   for (int wv = 0; wv < n_waves; ++wv) {
     const int64_t b0 = g->wave_b0[wv], b1 = g->wave_b0[wv + 1];
