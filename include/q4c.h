@@ -420,7 +420,8 @@ Q4C_API q4c_status q4c_scf_pass(const q4c_tables* tables, const q4c_grid* grid, 
  * potential v_dev (each bucket's products launched once untimed and three
  * times between CUDA events on `stream`, into scratch outputs it allocates
  * and frees), keeps the faster one per bucket in the grid, and synchronises
- * the stream.  The choice applies to every later split-path integration
+ * the stream; batches of more than 256 functions are not timed, and a bucket of
+ * nothing else keeps its shape.  The choice applies to every later split-path integration
  * (q4c_integrate, q4c_integrate_columns, q4c_scf_pass) on the grid; results
  * do not depend on it beyond the order of FP64 additions.
  * The density/adjoint kernel (row-dot products over 16-function K-steps)

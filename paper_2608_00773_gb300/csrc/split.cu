@@ -664,9 +664,11 @@ q4c_status integrate_columns_split(const q4c_tables* t, const q4c_grid* g, const
 
 // Tile-shape tuner: on the first wave, with the wave's tables, tiles and
 // rounding constants in place, each batch-size bucket's items run with one
-// and with two K-steps per stage (one untimed launch, then three timed by
+// with two K-steps per stage (one untimed launch, then three timed by
 // CUDA events on the stream) into scratch outputs; the faster shape is kept
-// for the bucket.  The density/adjoint kernel's shape is chosen the same way
+// for the bucket.  Items of the pair kernel, which has one shape, are left out:
+// timed with the others they hid the difference (304-atom slab, last bucket: two
+// timings of 28.0 ms, and noise picked the slower shape).  The density/adjoint kernel's shape is chosen the same way
 // (one per grid) on the same tiles.
 q4c_status autotune_split(const q4c_tables* t, q4c_grid* g, const double* v, cudaStream_t s) {
   if (g->max_np > 341 || g->wave_b0.size() < 2) return Q4C_OK;
@@ -685,9 +687,8 @@ q4c_status autotune_split(const q4c_tables* t, q4c_grid* g, const double* v, cud
   }
   const int64_t* r = g->split_bw0.data();
   const int64_t i0 = r[0], i1 = g->split_pair0[0];
-  if (r[kTileBuckets] <= i0) return Q4C_OK;
-  if (i1 > i0)
-    split::k_item_prep<<<static_cast<unsigned>(i1 - i0), 128, 0, s>>>(g->view(), g->d_split_items + i0, g->d_colexp,
+  if (i1 <= i0) return Q4C_OK;
+  split::k_item_prep<<<static_cast<unsigned>(i1 - i0), 128, 0, s>>>(g->view(), g->d_split_items + i0, g->d_colexp,
                                                                      g->d_split_mag);
   Q4C_CUDA(cudaGetLastError());
   double* scratch = nullptr;
@@ -702,19 +703,19 @@ q4c_status autotune_split(const q4c_tables* t, q4c_grid* g, const double* v, cud
   double* o[5];
   for (int m = 0; m < 5; ++m) o[m] = scratch + m * std::max<int64_t>(g->nnz, 1);
   for (int k = 0; k < kTileBuckets && status == Q4C_OK; ++k) {
-    const int64_t c0 = r[k], c1 = r[k + 1];
-    if (c1 <= c0) continue;
+    const int64_t c0 = r[k], c1 = std::min(r[k + 1], i1);
+    if (c1 <= c0) continue;  // not timed, and its shape stays as it is
     const float* mag = g->d_split_mag + (c0 - i0) * 128;
     for (int ks = 1; ks <= 2 && status == Q4C_OK; ++ks) {
       float ms = 0.f;
-      if (q4c_status st = launch_products_ks(ks, g, g->d_split_items + c0, static_cast<int>(c1 - c0), static_cast<int>(i1 - c0), mag, o[0],
+      if (q4c_status st = launch_products_ks(ks, g, g->d_split_items + c0, static_cast<int>(c1 - c0), static_cast<int>(c1 - c0), mag, o[0],
                                              o[1], o[2], o[3], o[4], "split_tune", s)) {
         fail(st);
         break;
       }
       cudaEventRecord(e0, s);
       for (int rep = 0; rep < 3 && status == Q4C_OK; ++rep)
-        if (q4c_status st = launch_products_ks(ks, g, g->d_split_items + c0, static_cast<int>(c1 - c0), static_cast<int>(i1 - c0), mag, o[0],
+        if (q4c_status st = launch_products_ks(ks, g, g->d_split_items + c0, static_cast<int>(c1 - c0), static_cast<int>(c1 - c0), mag, o[0],
                                                o[1], o[2], o[3], o[4], "split_tune", s))
           fail(st);
       cudaEventRecord(e1, s);
