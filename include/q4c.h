@@ -246,10 +246,11 @@ Q4C_API q4c_status q4c_integrate(const q4c_tables* tables, const q4c_grid* grid,
 /* Density (Eqs. 39-40): n_p = sum_ij P_ij phi_i(p) phi_j(p), P_dev device
  * [nnz] on the block pattern (any P; only its symmetric part contributes),
  * n_dev device [n_points] in batch order, overwritten.  Q4C_SPLIT takes
- * batches of up to 4096 active functions (above 512 the sum over i runs in
- * exact segments of 512 combined in FP64), Q4C_FP64 up to 7264;
- * Q4C_EUNSUPPORTED beyond.  The split limit holds for q4c_density_full and
- * q4c_integrate_backward too; their FP64 path takes up to 5811. */
+ * batches of up to 4096 active functions (the sum over i runs in segments of
+ * at most 112, exact in their leading levels and added up as FP32 pairs), Q4C_FP64
+ * up to 7264; Q4C_EUNSUPPORTED beyond.  The split limit holds for
+ * q4c_density_full and q4c_integrate_backward too; their FP64 path takes up to
+ * 5811.  Equal calls give equal bits. */
 Q4C_API q4c_status q4c_density(const q4c_tables* tables, const q4c_grid* grid, const double* P_dev,
                        q4c_precision prec, double* n_dev, q4c_stream stream);
 

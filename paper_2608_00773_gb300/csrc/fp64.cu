@@ -631,6 +631,8 @@ static q4c_status rowdot_fp64_wave(const q4c_grid* g, int wv, const double* cons
 }
 
 // the density of one wave (its basis tiles in place)
+// (the limits here and below are the calls' own: the kernel's shared memory does
+// not depend on the batch)
 q4c_status density_fp64_wave(const q4c_grid* g, int wv, const double* P, double* n, cudaStream_t s) {
   if (g->max_nb > 7264) {
     set_error("the FP64 density needs at most 7264 active functions per batch");

@@ -16,7 +16,8 @@
 // Each U is computed from six BF16 slices of F (an exponent per point and
 // quantity) and of G' (an exponent per column and matrix) in six FP32
 // accumulators, one per level s + t (see split.cu): levels 0-2 are exact integer
-// sums for K <= 512 terms (here at most 112), levels 3-5 are rounded 2^-24 below.
+// sums for K <= 204 terms (kFine; here at most 112), levels 3-5 are rounded 2^-24
+// below.
 //
 // G' does not depend on the points, so a pre-pass slices every batch's G' once
 // into BF16 digit tiles laid out exactly as the MMA reads them (per matrix,
@@ -50,9 +51,9 @@ constexpr int kThreads = 16 * 32;
 constexpr uint32_t kTmemCols = 512;
 constexpr uint32_t kSetCols = 256;  // two accumulator sets of six levels of up to 32 columns
 constexpr int kMaxNb = 4096;
-// The digits resolve 2^-2 finer than tc::slice6 does against the exponent
-// itself: with |d_0| <= 256 (exact in BF16) and K <= 112 terms the exact levels
-// stay below 112 * (2 * 256 * 128 + 128^2) < 2^24, and the symmetric matrices'
+// The digits resolve 2^-2 finer than tc::slice6x2 does against the exponent
+// itself: with |d_0| <= 256 (exact in BF16) a term of the exact levels is at most
+// 2 * 256 * 128 + 128^2 units, so that they hold 204 terms below 2^24, and the symmetric matrices'
 // doubled coefficients are resolved as finely as their two halves were (error of
 // the 64-atom density against FP64: 1.5e-13 before, 2.7e-13 at the coarser
 // digits, 4.7e-14 with these).

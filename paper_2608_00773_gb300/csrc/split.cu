@@ -7,7 +7,7 @@
 //   x = sum_s d_s 2^(e - 6 - 8s),  s = 0..5,  |d_0| <= 64, |d_1|, |d_2| <= 128,
 //   |d_3| <= 160, |d_4|, |d_5| <= 128,
 // with e a per-column binary exponent (|x| <= 2^e over the batch); the digits
-// come from FP32 round-to-multiple steps (tc::slice6).  Each digit has <= 8
+// come from FP32 round-to-multiple steps (tc::slice6x2).  Each digit has <= 8
 // significant bits, so it is exact in BF16 and every slice product is exact
 // in FP32.  Per output element six FP32 accumulators (one per level s + t)
 // are kept in tensor memory:

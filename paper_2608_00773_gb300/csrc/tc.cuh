@@ -204,11 +204,6 @@ __device__ __forceinline__ bool bar_red_or(int id, int n, bool p) {
   return r != 0;
 }
 
-// the phase of an mbarrier also waits for `bytes` of asynchronous copies
-__device__ __forceinline__ void expect_tx(uint32_t bar, uint32_t bytes) {
-  asm volatile("mbarrier.expect_tx.relaxed.cta.shared::cta.b64 [%0], %1;" ::"r"(bar), "r"(bytes) : "memory");
-}
-
 // bulk global -> shared copy (16-byte aligned addresses, size a multiple of
 // 16) that completes `bytes` of transactions on the mbarrier
 __device__ __forceinline__ void bulk_copy(uint32_t dst, const void* src, uint32_t bytes, uint32_t bar) {
@@ -254,18 +249,6 @@ __device__ __forceinline__ void tc_fence_after() { asm volatile("tcgen05.fence::
 // after tcgen05.wait::ld, so each helper issues its loads and the wait in ONE
 // asm statement; its outputs then exist only after the wait, and no use of
 // them can be scheduled ahead of it.
-__device__ __forceinline__ void tmem_ld16(uint32_t taddr, float* v) {
-  uint32_t r[16];
-  asm volatile(
-      "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, [%16];\n\t"
-      "tcgen05.wait::ld.sync.aligned;"
-      : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]),
-        "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
-      : "r"(taddr)
-      : "memory");
-#pragma unroll
-  for (int i = 0; i < 16; ++i) v[i] = __uint_as_float(r[i]);
-}
 
 // three 8-column loads (one per address) under a single wait
 __device__ __forceinline__ void tmem_ld8x3(uint32_t t0, uint32_t t1, uint32_t t2, float* v0, float* v1, float* v2) {
@@ -341,24 +324,6 @@ __device__ __forceinline__ float magic0(int e) {
   return __int_as_float(((e + 17 + 127) << 23) | 0x400000);
 }
 
-// Six balanced digits of the double-float value h + l (|h + l| <= 2^e) with
-// m0 = magic0(e): digit s is returned already multiplied by its weight
-// 2^(e - 6 - 8s).  Digits 0-2 come from h exactly (|d| <= 64, 128, 128); l
-// joins the residual (|r| <= 2^(e - 23)) before digit 3, rounded at most
-// 2^(e - 48), so |d3| <= 160 and |d4|, |d5| <= 128, all exact in BF16, and
-// the six digits represent h + l within 2^(e - 46).
-__device__ __forceinline__ void slice6(float h, float l, float m0, float d[kSlices]) {
-  float x = h, m = m0;
-#pragma unroll
-  for (int s = 0; s < kSlices; ++s) {
-    if (s == 3) x = __fadd_rn(x, l);
-    const float t = __fsub_rn(__fadd_rn(x, m), m);
-    d[s] = t;
-    x = __fsub_rn(x, t);
-    m = __fmul_rn(m, 0x1p-8f);
-  }
-}
-
 // ------------------------------------------------------------ pairs
 // Two FP32 values operated on by the packed float2 instructions of sm_100
 // and later (CUDA's __fadd2_rn, __fmul2_rn, __ffma2_rn): each half is
@@ -401,8 +366,14 @@ __device__ __forceinline__ void df_mul2(float2 xh, float2 xl, float2 yh, float2 
   rl = sub2(e, sub2(rh, p));
 }
 
-// slice6 on a pair of values (h + l per half) against the same rounding
-// constant m0 for both: d[s] holds digit s of both halves, weighted
+// Six balanced digits of two double-float values h + l (one per half, |h + l| <=
+// 2^e) against the rounding constant m0 = magic0(e): d[s] holds digit s of both,
+// already multiplied by its weight 2^(e - 6 - 8s).  Digits 0-2 come from h exactly
+// (|d| <= 64, 128, 128); l joins the residual (|r| <= 2^(e - 23)) before digit 3,
+// rounded at most 2^(e - 48), so |d3| <= 160 and |d4|, |d5| <= 128, all exact in
+// BF16, and the six digits represent h + l within 2^(e - 46).  Against
+// magic0(e - f), f = 1 or 2, they are f bits finer: |d0| <= 64 2^f, |d3| <= 192 or
+// 256 (still exact), and h + l within 2^(e - 46 - f).
 __device__ __forceinline__ void slice6x2(float2 h, float2 l, float m0, float2 d[kSlices]) {
   float2 x = h;
   float m = m0;
