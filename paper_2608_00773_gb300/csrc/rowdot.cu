@@ -467,7 +467,7 @@ __device__ __forceinline__ void mma_row_levels(uint32_t tmem, uint64_t a, uint64
 //   warps 4-11  read the six levels from tensor memory (lane = point, each group
 //               of four warps half of the columns; R one group ahead), form U = exact levels by
 //               two-sums plus the rounded tail, dot with R in double-float, and
-//               write each point's result at the end of the item.
+//               write each point's result (of a share, its part) at the end of the item.
 // Warps whose points lie past n_p slice and drain nothing.
 // Every wait is bounded; a timeout sets the status bit and an abort flag.
 //
@@ -478,8 +478,8 @@ __device__ __forceinline__ void mma_row_levels(uint32_t tmem, uint64_t a, uint64
 // lanes.  Before, 64-point items re-sliced F for every product and 64-column
 // tile, and their epilogue ran over two half-level sums of all seven products:
 // 89 KB through shared memory a step and 1,360 clocks.
-// Adjoint, before -> now: 64-atom cluster 4.28 -> 2.69 ms, 24 molecules 23.4 ->
-// 12.7 ms, 304-atom slab 64.2 -> 33.2 ms; density of the cluster 0.67 -> 0.45 ms.
+// Adjoint, before -> now: 64-atom cluster 4.28 -> 2.54 ms, 24 molecules 23.4 ->
+// 11.9 ms, 304-atom slab 64.2 -> 32.8 ms; density of the cluster 0.67 -> 0.45 ms.
 template <int MODE, int KS>  // MODE 0: density, 1: adjoint; KS: G' blocks per stage
 __global__ void __launch_bounds__(kThreads, 1)
     k_split_rowdot(DevGrid G, const RdItem* __restrict__ items, int n_items, const double* __restrict__ scratch,
